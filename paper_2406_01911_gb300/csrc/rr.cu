@@ -48,6 +48,8 @@ constexpr int kNStat = 10;             // work counters (stat slots below)
 constexpr int kWQ = 128;               // per-warp queue (members of the warp's set)
 constexpr int kWHashBits = 8;
 constexpr int kWHash = 1 << kWHashBits;  // per-warp open-addressing member set
+// path phase (LT sets): the warp's member set and queue in global memory
+constexpr int kPathMaxBits = 13;         // at most 8,192 member-set slots and 4,096 queue slots
 
 struct RRJobMap {
     int64_t job_base[HYPERIM_NSTRATA + 1];
@@ -97,7 +99,10 @@ struct RRParams {
     int* esc_count;           // jobs the warp phase handed to the block phase
     int32_t* esc_list;        // those jobs
     int block_phase;          // 1: this launch runs the jobs of esc_list (else all jobs)
-    int warp_limit;           // warp phase: the largest RR set a warp builds alone (1..kWQ)
+    int warp_limit;           // warp phase: the largest RR set a warp builds alone (1..kWQ, or the
+                              // path phase's queue length)
+    int32_t* path;            // path phase: per warp a member set and a queue in global memory (else null)
+    int path_bits;            // log2 of the member set's slots; the queue holds half as many ids
     int plain;                // 1: this launch runs jobs [plain_base, plain_base + gridDim.x), one per block
     int64_t plain_base;
     int rewrite;              // 1: a repair launch -- sets go to the arena slots recorded by the first
@@ -346,14 +351,15 @@ struct QueueSink {
 };
 
 struct WarpSink {
-    int32_t* hash;   // kWHash slots, -1 empty
-    int32_t* queue;  // kWQ slots
+    int32_t* hash;   // 2^hash_bits slots, -1 empty
+    int32_t* queue;  // limit slots
     int* tail;       // members so far (may pass limit: the set then leaves the warp phase)
-    int limit;       // the largest set a warp builds alone (<= kWQ)
+    int limit;       // the largest set a warp builds alone
+    int hash_bits;
     __device__ __forceinline__ void push(uint32_t nu) const {
         if (*(volatile int*)tail > limit) return;  // already too large: the set is redone by a block
-        uint32_t h = (nu * 0x9E3779B1u) >> (32 - kWHashBits);
-        for (int probe = 0; probe < kWHash; ++probe) {
+        uint32_t h = (nu * 0x9E3779B1u) >> (32 - hash_bits);
+        for (int probe = 0; probe < (1 << hash_bits); ++probe) {
             const int32_t old = atomicCAS(&hash[h], -1, (int32_t)nu);
             if (old == -1) {
                 const int pos = atomicAdd(tail, 1);
@@ -361,9 +367,9 @@ struct WarpSink {
                 return;
             }
             if (old == (int32_t)nu) return;
-            h = (h + 1) & (kWHash - 1);
+            h = (h + 1) & ((1u << hash_bits) - 1);
         }
-        atomicMax(tail, limit + 1);  // no free slot (cannot happen below kWQ + 32 members)
+        atomicMax(tail, limit + 1);  // no free slot (cannot happen below limit + 32 members)
     }
 };
 
@@ -726,6 +732,21 @@ __device__ void warp_walk(const RRParams& P, SM& S, const Sink& sink, const uint
     __syncwarp();
 }
 
+// Number of entries of the ascending e[0, len) below x, by the whole warp (every lane passes the same
+// arguments): 32 evenly spaced probes a round, so 1,000 entries take two dependent loads.
+__device__ __forceinline__ int warp_lower_bound(const int32_t* __restrict__ e, int len, int32_t x) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0, hi = len;  // the answer lies in [lo, hi]
+    while (hi - lo > 32) {
+        const int step = (hi - lo + 31) >> 5;
+        const int p = lo + (lane + 1) * step - 1;
+        const int below = __popc(__ballot_sync(0xFFFFFFFFu, p < hi && e[p] < x));
+        hi = min(hi, lo + (below + 1) * step - 1);
+        lo += below * step;
+    }
+    return lo + __popc(__ballot_sync(0xFFFFFFFFu, lane < hi - lo && e[lo + lane] < x));
+}
+
 // Returns true when the pop must be handed to the block path.
 template <class SM, class Sink>
 __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j, uint32_t ybase, int32_t mu) {
@@ -833,11 +854,7 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
         // A(mu) = the single hyperedge minus mu, sorted: position x maps to member x or x + 1
         const int2 sp = P.v_span[v_begin];
         const int32_t hb = sp.x, len = sp.y;
-        int pmu = 0;
-        for (int b = 0; b < len; b += 32) {
-            const bool lt = b + lane < len && (uint32_t)P.he_mem[hb + b + lane] < (uint32_t)mu;
-            pmu += __popc(__ballot_sync(0xFFFFFFFFu, lt));
-        }
+        const int pmu = warp_lower_bound(P.he_mem + hb, len, mu);
         const Need nd = need[0];
         if (nd.h >= nd.n) {
             for (int x = lane; x < len - 1; x += 32)
@@ -1403,6 +1420,7 @@ struct WarpShared {
     uint32_t wpoff[kPWarps][kLQ + 1];
     int wcnt[kPWarps][kBLQ];
     int wtail[kPWarps];
+    unsigned long long cyc[3];                   // per-set SM cycles of the path phase: sum, max, count
     int32_t whash[kPWarps][kWHash];
     int32_t wqueue[kPWarps][kWQ];
     union {
@@ -1416,6 +1434,14 @@ struct WarpShared {
 // any other job is listed for the block phase (k_rr with block_phase), which builds it again
 // from its root (the draws are keyed by (RR, vertex, layer), so the set is the same) and the warp's
 // partial counters are dropped. Jobs are taken from the last one down, as in k_rr.
+//
+// Path phase (P.path set): the sets of the LT cascade. Such a set is one path -- every pop adds at
+// most one vertex -- so a block has work for one of its 16 warps, and the launch waits on the
+// latency of one pop after another. Here every warp follows a path of its own, 16 per SM; the
+// member set and the queue sit in global memory (they stay in L2: 48 KB a warp) because paths run
+// to hundreds of members (2M vertices, weighted cascade: mean 377, largest 1,708). A path of more
+// than 4,096 goes to the block phase. Measured on that graph, 10,010 sets: 843 ms with a block per set,
+// 80 ms with a warp per set.
 __global__ void __launch_bounds__(kPThreads, 2) k_rr_warp(RRParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     WarpShared& S = *reinterpret_cast<WarpShared*>(smem_raw);
@@ -1423,12 +1449,20 @@ __global__ void __launch_bounds__(kPThreads, 2) k_rr_warp(RRParams P) {
     const int64_t njobs = P.pool_start[P.npools];
     if (threadIdx.x < kMaxPools * kNStat) (&S.stat[0][0])[threadIdx.x] = 0;
     if (threadIdx.x < kPWarps * kNStat) (&S.wstat[0][0])[threadIdx.x] = 0;
+    if (threadIdx.x < 3) S.cyc[threadIdx.x] = 0;
     for (int i = threadIdx.x; i < kPWarps * kWHash; i += kPThreads) (&S.whash[0][0])[i] = -1;
     __syncthreads();
     int32_t* hash = S.whash[wid];
     int32_t* queue = S.wqueue[wid];
+    int hash_bits = kWHashBits;
+    if (P.path) {  // empty (-1) at the start of the launch and after every set
+        const int64_t slots = 3ll << (P.path_bits - 1);
+        hash = P.path + ((int64_t)blockIdx.x * kPWarps + wid) * slots;
+        queue = hash + (1ll << P.path_bits);
+        hash_bits = P.path_bits;
+    }
     int* tail = &S.wtail[wid];
-    const WarpSink sink{hash, queue, tail, P.warp_limit};
+    const WarpSink sink{hash, queue, tail, P.warp_limit, hash_bits};
     unsigned long long* wst = S.wstat[wid];
     for (;;) {
         int64_t ticket = 0;
@@ -1437,6 +1471,7 @@ __global__ void __launch_bounds__(kPThreads, 2) k_rr_warp(RRParams P) {
         if (ticket >= njobs) break;
         const int64_t job = njobs - 1 - ticket;
         const Job J = decode_job(P, job);
+        const long long cyc0 = clock64();
         if (lane == 0) {
             const int32_t root = draw_root(P, J);
             *tail = 0;
@@ -1451,16 +1486,19 @@ __global__ void __launch_bounds__(kPThreads, 2) k_rr_warp(RRParams P) {
             const int32_t mu = queue[head];
             if (pop_warp(P, S, sink, J.j, J.ybase, mu)) { escalate = true; break; }
             __syncwarp();
-            if (*(volatile int32_t*)&P.st->code != 0) break;  // a failure elsewhere: stop early
+            // a failure elsewhere: stop early (looked for now and then: the read goes to L2)
+            if ((head & 15) == 15 && *(volatile int32_t*)&P.st->code != 0) break;
         }
         __syncwarp();
         const int size = min(*(volatile int*)tail, P.warp_limit);
         if (escalate) {
             if (lane == 0) P.esc_list[atomicAdd(P.esc_count, 1)] = (int32_t)job;
         } else {
-            // output: the members in ascending order
-            uint32_t* buf = S.u.w.wbuf[wid];
-            for (int i = lane; i < size; i += 32) buf[i] = (uint32_t)queue[i];
+            // output: the members in ascending order (a set larger than the sort buffer is sorted in
+            // the queue itself, a power of two long)
+            uint32_t* buf = size <= kWCap ? S.u.w.wbuf[wid] : reinterpret_cast<uint32_t*>(queue);
+            if (size <= kWCap)
+                for (int i = lane; i < size; i += 32) buf[i] = (uint32_t)queue[i];
             __syncwarp();
             group_sort<32>(buf, size);
             unsigned long long pos = 0;
@@ -1476,10 +1514,22 @@ __global__ void __launch_bounds__(kPThreads, 2) k_rr_warp(RRParams P) {
         }
         __syncwarp();
         if (lane < kNStat) wst[lane] = 0;
-        for (int i = lane; i < kWHash; i += 32) hash[i] = -1;
+        for (int i = lane; i < (1 << hash_bits); i += 32) hash[i] = -1;
+        if (P.path && !escalate && lane == 0) {
+            // an SM holds 2 kPWarps paths at once: a set's share of its SM's time
+            const unsigned long long d = (unsigned long long)(clock64() - cyc0);
+            atomicAdd(&S.cyc[0], d / (2 * kPWarps));
+            atomicMax(&S.cyc[1], d);
+            atomicAdd(&S.cyc[2], 1ull);
+        }
         __syncwarp();
     }
     __syncthreads();
+    if (threadIdx.x == 0 && P.path && P.set_cycles && S.cyc[2]) {
+        atomicAdd(P.set_cycles, S.cyc[0]);
+        atomicMax(P.set_cycles + 1, S.cyc[1]);
+        atomicAdd(P.set_cycles + 2, S.cyc[2]);
+    }
     if (threadIdx.x < P.npools) {
         RRCounters* c = P.counters + threadIdx.x;
         const unsigned long long* st = S.stat[threadIdx.x];
@@ -2099,9 +2149,11 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     const uint64_t want = arena_want(g, pools, npools, pool_start, g->n);
     // the warp phase (one RR set per warp) runs first in the persistent schedule, unless the
     // graph's tuning turned it off; its grid
-    const bool warp_phase = g->schedule != HYPERIM_SCHED_PLAIN && g->warp_set_limit > 0;
+    bool warp_phase = g->schedule != HYPERIM_SCHED_PLAIN && g->warp_set_limit > 0;
+    // LT sets are single paths: without a tuned warp phase they take the path phase
+    bool path_phase = g->schedule != HYPERIM_SCHED_PLAIN && !warp_phase && pools[0]->strategy == HYPERIM_STRAT_LT;
     int wblocks = 0;
-    if (warp_phase) {
+    if (warp_phase || path_phase) {
         int wper_sm = 0;
         HYP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&wper_sm, k_rr_warp, kPThreads, sizeof(WarpShared)));
         if (wper_sm < 1) return set_error(HYPERIM_ECUDA, "RR warp-phase kernel does not fit on an SM");
@@ -2124,6 +2176,20 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     if ((st = tmp.alloc(&d_size, sizeof(int32_t) * (size_t)njobs))) return st;
     if ((st = tmp.alloc(&d_esc, sizeof(int32_t) * (size_t)njobs))) return st;
     if ((st = tmp.alloc(&d_ctrl, sizeof(Ctrl)))) return st;
+    int32_t* d_path = nullptr;
+    int path_bits = 0;
+    if (path_phase) {
+        // a member set of up to 2^13 slots and a queue of half as many per warp (never more than a set
+        // of n members can need); without the memory for it the sets go to the block kernel
+        path_bits = std::min(std::max(g->id_bits + 1, 6), kPathMaxBits);
+        const size_t ids = (size_t)wblocks * kPWarps * (3ull << (path_bits - 1));
+        if (tmp.alloc(&d_path, sizeof(int32_t) * ids) == HYPERIM_OK) {
+            HYP_CUDA(cudaMemsetAsync(d_path, 0xFF, sizeof(int32_t) * ids, s));
+            warp_phase = true;
+        } else {
+            path_phase = false;
+        }
+    }
     unsigned long long* d_used = &d_ctrl->arena_used;
     RRParams P;
     std::memset(&P, 0, sizeof(P));
@@ -2151,7 +2217,9 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     P.esc_count = &d_ctrl->esc_count;
     P.esc_list = d_esc;
     P.block_phase = 0;
-    P.warp_limit = std::min(std::max(g->warp_set_limit, 1), kWQ);
+    P.warp_limit = path_phase ? 1 << (path_bits - 1) : std::min(std::max(g->warp_set_limit, 1), kWQ);
+    P.path = d_path;
+    P.path_bits = path_bits;
     P.plain = g->schedule == HYPERIM_SCHED_PLAIN ? 1 : 0;
     P.plain_base = 0;
     P.arena_used = d_used;
