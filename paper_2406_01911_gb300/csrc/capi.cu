@@ -74,6 +74,15 @@ void dev_free(hyperim_graph* g, void* p, size_t bytes) {
     graph_root(g)->device_bytes.fetch_sub(bytes);
 }
 
+void free_memo(hyperim_graph* g) {
+    Scratch& S = g->scratch;
+    dev_free(g, S.memo_slot, sizeof(uint32_t) * (size_t)g->n);
+    dev_free(g, S.memo, sizeof(uint32_t) * S.memo_cap);
+    S.memo_slot = nullptr;
+    S.memo = nullptr;
+    S.memo_cap = 0;
+}
+
 std::mutex& graph_mutex() {
     static std::mutex m;
     return m;
@@ -283,6 +292,7 @@ void free_handle(hyperim_graph* g, bool data) {
     dev_free(g, S.picks, sizeof(uint32_t) * S.pick_cap * S.blocks);
     dev_free(g, S.big, sizeof(uint32_t) * S.big_cap * S.blocks);
     dev_free(g, S.arena, sizeof(int32_t) * S.arena_cap);
+    free_memo(g);
     if (data) {
         void* ptrs[] = {g->he_off, g->he_mem, g->v_off, g->v_he, g->tsum, g->v_span, g->vinfo, g->prof_off,
                         g->prof, g->cdf_tab, g->deg, g->stratum, g->vs_off, g->vs_list, g->idx, g->idx_tab,
@@ -372,6 +382,7 @@ hyperim_status hyperim_graph_share(hyperim_graph_t g, void* cuda_stream, hyperim
     h->max_deg = r->max_deg;
     h->max_tsum = r->max_tsum;
     h->max_layer_n = r->max_layer_n;
+    h->sum_tsum = r->sum_tsum;
     for (int s = 0; s < HYPERIM_NSTRATA; ++s) h->stratum_size[s] = r->stratum_size[s];
     h->theta_lstar = r->theta_lstar;
     h->sm_count = r->sm_count;

@@ -77,7 +77,8 @@ constexpr int kDirMaxBits = 12;
 
 // Profile entry of layer i of A(mu): 32 bytes, two uint4.
 //   [0] = {w_i | (p == 1 ? 1u << 31 : 0), n_i, floor(p 2^32) for 0 <= p < 1, T_0}
-//   [1] = {offset of the layer's CDF table, table length L, Poisson parts c, kind}
+//   [1] = {offset of the layer's CDF table, table length L | kind << 16, Poisson parts c,
+//          members of the layers before it}
 // kind 0: no draw (p = 0 or p = 1); 1: Binomial (n_i <= 20); 2: Poisson with c parts of lambda/c
 // (the paper's strategy for n_i > 20). The table holds the inversion's thresholds T_0..T_{L-1}
 // (capped at 2^32 - 1), computed at load by the same IEEE sequence as the inversion: a draw below
@@ -99,6 +100,10 @@ struct Scratch {
     // output arena
     int32_t* arena = nullptr;
     size_t arena_cap = 0;        // entries
+    // neighbourhoods kept within one growth step (see Memo in rr.cu); optional
+    uint32_t* memo_slot = nullptr;  // n words
+    uint32_t* memo = nullptr;
+    size_t memo_cap = 0;         // entries
 };
 
 }  // namespace hyperim
@@ -139,6 +144,7 @@ struct hyperim_graph {
     int64_t profile_entries = 0;
     int32_t max_layers = 0, max_dh = 0;
     int64_t max_deg = 0, max_tsum = 0, max_layer_n = 0;
+    int64_t sum_tsum = 0;        // sum over all vertices of tsum
     int64_t stratum_size[HYPERIM_NSTRATA] = {};
     double theta_lstar = 0.0;
     // device status + scratch
@@ -213,6 +219,8 @@ hyperim_status cuda_fail(cudaError_t e, const char* what);
 // through the caller's allocator when the graph was loaded with one
 hyperim_status dev_alloc(hyperim_graph* g, void** p, size_t bytes);
 void dev_free(hyperim_graph* g, void* p, size_t bytes);
+// releases the handle's optional scratch (Scratch::memo), stream-ordered
+void free_memo(hyperim_graph* g);
 
 // Device buffers of one call: every allocation made through it is released (stream-ordered)
 // when it goes out of scope, on every return path of the call.

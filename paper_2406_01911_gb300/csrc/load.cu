@@ -445,8 +445,9 @@ k_profile(Incidence I, const int2* __restrict__ v_span, const int32_t* __restric
 
 // ---- layer profile: pass 2 (thresholds, inversion kind, CDF table lengths) ------------------
 // Entry [0] = {w_i | p = 1 flag, n_i, floor(p 2^32), T_0}; entry [1] = {table offset, table
-// length, Poisson parts c, kind}; kind 0: no draw (p = 0 or 1), 1: Binomial (n_i <= 20), 2:
-// Poisson with c parts of lambda / c each (Sec. 3.1.3). The table and T_0 are filled by pass 3.
+// length | kind << 16, Poisson parts c, n_1 + .. + n_{i-1}}; kind 0: no draw (p = 0 or 1), 1:
+// Binomial (n_i <= 20), 2: Poisson with c parts of lambda / c each (Sec. 3.1.3). The table and T_0
+// are filled by pass 3.
 __global__ void k_profile_write(int32_t n, const int32_t* __restrict__ v_off,
                                 const uint2* __restrict__ pairs, const int64_t* __restrict__ poff64,
                                 const uint32_t* __restrict__ deg, int32_t model, uint64_t uthr,
@@ -461,6 +462,7 @@ __global__ void k_profile_write(int32_t n, const int32_t* __restrict__ v_off,
         if (v == n - 1) prof_off[n] = (int32_t)poff64[n];
         stratum[v] = (uint8_t)(l < HYPERIM_NSTRATA - 1 ? l : HYPERIM_NSTRATA - 1);
         const uint32_t dg = deg[v];
+        uint32_t before = 0;
         for (int i = 0; i < l; ++i) {
             const uint2 wn = pairs[v_off[v] + i];
             const uint32_t n_i = wn.y;
@@ -491,8 +493,9 @@ __global__ void k_profile_write(int32_t n, const int32_t* __restrict__ v_off,
                 }
             }
             prof[2 * (pb + i)] = make_uint4(wn.x | flags, n_i, thr >= kPOne ? 0u : (uint32_t)thr, 0u);
-            prof[2 * (pb + i) + 1] = make_uint4(0u, L, c, kind);
+            prof[2 * (pb + i) + 1] = make_uint4(0u, L | (kind << 16), c, before);
             tab_len[pb + i] = L;
+            before += n_i;
         }
     }
 }
@@ -503,7 +506,7 @@ __global__ void k_table_fill(int64_t layers, const int64_t* __restrict__ tab_off
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < layers;
          x += (int64_t)gridDim.x * blockDim.x) {
         uint4 a = prof[2 * x], b = prof[2 * x + 1];
-        const uint32_t n_i = a.y, kind = b.w;
+        const uint32_t n_i = a.y, kind = b.y >> 16;
         const uint32_t off = (uint32_t)tab_off[x];
         b.x = off;
         if (kind == 1) {
@@ -512,7 +515,7 @@ __global__ void k_table_fill(int64_t layers, const int64_t* __restrict__ tab_off
             const double lam = poisson_lambda(n_i, a.z);
             cdf_table(n_i, a.z, true, poisson_part_lambda(lam, b.z), kTableCap, tab + off);
         }
-        a.w = b.y > 0 ? tab[off] : 0u;  // T_0 beside the entry: the common h = 0 needs no table read
+        a.w = kind != 0 ? tab[off] : 0u;  // T_0 beside the entry: the common h = 0 needs no table read
         prof[2 * x] = a;
         prof[2 * x + 1] = b;
     }
@@ -541,13 +544,22 @@ __global__ void k_hist_layers(const int64_t* __restrict__ poff64, int32_t n,
     }
 }
 
-__global__ void k_max_i32(const int32_t* __restrict__ a, int64_t n, unsigned long long* out) {
-    unsigned long long mx = 0;
+// out[0] = max, out[1] = sum (both zeroed by the caller)
+__global__ void k_max_sum_i32(const int32_t* __restrict__ a, int64_t n, unsigned long long* out) {
+    unsigned long long mx = 0, sum = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
+         i += (int64_t)gridDim.x * blockDim.x) {
         mx = max(mx, (unsigned long long)a[i]);
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out, mx);
+        sum += (unsigned long long)a[i];
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(out, mx);
+        atomicAdd(out + 1, sum);
+    }
 }
 
 __global__ void k_vhe_len(const int64_t* __restrict__ v_off64, int32_t n, int32_t* __restrict__ dh) {
@@ -738,13 +750,14 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
     HYP_CUDA(cudaMemsetAsync(d_max, 0, sizeof(unsigned long long) * 8, s));
     int32_t* d_dh = (int32_t*)d_cnt;  // reuse
     { k_vhe_len<<<grid_for(n, 256, sm), 256, 0, s>>>(d_voff64, n, d_dh); count_launch(); }
-    { k_max_i32<<<grid_for(n, 256, sm), 256, 0, s>>>(d_dh, n, d_max + 3); count_launch(); }
-    { k_max_i32<<<grid_for(n, 256, sm), 256, 0, s>>>(g->tsum, n, d_max + 4); count_launch(); }
+    { k_max_sum_i32<<<grid_for(n, 256, sm), 256, 0, s>>>(d_dh, n, d_max + 3); count_launch(); }
+    { k_max_sum_i32<<<grid_for(n, 256, sm), 256, 0, s>>>(g->tsum, n, d_max + 5); count_launch(); }
     unsigned long long hmax[8];
     HYP_CUDA(cudaMemcpyAsync(hmax, d_max, sizeof(hmax), cudaMemcpyDeviceToHost, s));
     HYP_CUDA(cudaStreamSynchronize(s));
     g->max_dh = (int32_t)hmax[3];
-    g->max_tsum = (int64_t)hmax[4];
+    g->max_tsum = (int64_t)hmax[5];
+    g->sum_tsum = (int64_t)hmax[6];
 
     // --- layer profile pass 1
     uint2* d_pairs = nullptr;

@@ -111,10 +111,14 @@ struct RRParams {
     RRCounters* counters;                    // kMaxPools entries
     int spin_limit;                          // rounds of a bounded wait before it gives up
     unsigned long long* set_cycles;          // optional {sum, max, count} of per-set SM cycles
+    uint32_t* memo_slot;      // neighbourhoods kept within this growth step (see Memo), or null
+    uint32_t* memo;
+    uint64_t memo_cap;
+    unsigned long long* memo_used;
 };
 
 struct Need {                    // a layer with h > 0 at the current pop
-    uint32_t w, n, h, ksel, layer;
+    uint32_t w, n, h, ksel, layer, before;  // before: members of the layers before it
 };
 
 // Buffers of phase 1 (warps pop independently) and of phase 2 / output (the whole block works on
@@ -186,7 +190,7 @@ __device__ __forceinline__ bool layer_draw(const uint4 e, const uint4 f, const u
     if (e.x & kPOneFlag) { h = n_i; return false; }
     if (thr == 0) { h = 0; return false; }
     const uint32_t w0 = ws.word(0);
-    const uint32_t kind = f.w, L = f.y, c = f.z;
+    const uint32_t kind = f.y >> 16, L = f.y & 0xFFFFu, c = f.z;
     if (kind == 1) {  // Binomial table: the same draw under both strategies (n_i <= 20)
         ksel = 1;
         if (w0 < e.w) { h = 0; return true; }
@@ -302,7 +306,8 @@ __device__ bool lt_keep(const RRParams& P, int32_t pb, int32_t l, uint32_t j, ui
         const uint64_t t = (e.x & kPOneFlag) ? (1ull << 32) : (uint64_t)e.z;
         const unsigned __int128 m = (unsigned __int128)e.y * t;
         if (y < C + m) {
-            nd = Need{e.x & ~kPOneFlag, e.y, 1u, (uint32_t)((uint64_t)(y - C) / t), (uint32_t)(i + 1)};
+            nd = Need{e.x & ~kPOneFlag, e.y, 1u, (uint32_t)((uint64_t)(y - C) / t), (uint32_t)(i + 1),
+                      P.prof[2 * ((int64_t)pb + i) + 1].w};
             return true;
         }
         C += m;
@@ -747,6 +752,107 @@ __device__ __forceinline__ int warp_lower_bound(const int32_t* __restrict__ e, i
     return lo + __popc(__ballot_sync(0xFFFFFFFFu, lane < hi - lo && e[lo + lane] < x));
 }
 
+// ------------------------------------------------------------------------------------------
+// Memo: neighbourhoods kept within one growth step
+// ------------------------------------------------------------------------------------------
+// A growth step pops the same vertices again and again (100k vertices at p = 0.01: 165 million pops
+// of 36,000 vertices), and the sort of a neighbourhood costs far more than the picks in it. A warp that
+// pops a vertex for the second time in a launch and sorts its neighbourhood leaves the members in
+// a scratch area, layer by layer in id order, so that a later pop reads the member at a picked
+// position with one load. The area holds nothing at the start of a growth step (the slots are
+// cleared), is bounded, and a vertex that finds no room is sorted as ever.
+// It pays where vertices are popped often: the query at p = 0.01 above went from 1,088 to 290 ms. On 2M
+// vertices under weighted cascade (3 pops per vertex and growth step, mostly of hubs that are
+// never sorted whole) it cost 2%, so a growth step uses it from kMemoPops expected pops per vertex on
+// (sets x the mean set size so far), or when no set size is known yet.
+// Slot of a vertex: nothing, popped once, being written (or no room), or kMemoFirst + its offset.
+constexpr uint32_t kMemoNone = 0, kMemoSeen = 1, kMemoFirst = 2, kMemoBusy = 0xFFFFFFFFu;
+constexpr uint64_t kMemoMax = 1ull << 26;      // entries at most (256 MiB)
+constexpr uint64_t kMemoPerSet = 1ull << 14;   // and per new RR set (a short step re-pops little)
+constexpr double kMemoPops = 16.0;
+
+// slots and entries are written by other SMs during the launch: read at the L2, never from an L1 line
+__device__ __forceinline__ uint32_t ld_strong(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// The vertex is popped (slot value `kept`, none or seen): the entry offset for this warp to fill, or
+// ~0. One warp gets it: the one that finds the vertex seen, if its deg(mu) members have room.
+__device__ __forceinline__ unsigned long long memo_touch(const RRParams& P, int32_t mu, int32_t pb, int32_t l,
+                                                         uint32_t kept) {
+    unsigned long long at = ~0ull;
+    if ((threadIdx.x & 31) == 0) {
+        if (kept == kMemoNone) {
+            atomicCAS(P.memo_slot + mu, kMemoNone, kMemoSeen);
+        } else if (atomicCAS(P.memo_slot + mu, kMemoSeen, kMemoBusy) == kMemoSeen) {
+            const int64_t last = 2 * ((int64_t)pb + l - 1);
+            const unsigned long long deg = (unsigned long long)P.prof[last].y + P.prof[last + 1].w;
+            const unsigned long long o = atomicAdd(P.memo_used, deg);
+            if (o + deg <= P.memo_cap) at = o;
+        }
+    }
+    return __shfl_sync(0xFFFFFFFFu, at, 0);
+}
+
+// The runs of the sorted buf[0, got) appended to their layers' places in dst: lane i < l holds the
+// multiplicity `w` of layer i (descending, distinct) and the place of its next member.
+__device__ __forceinline__ void memo_emit(const uint32_t* buf, int got, int l, uint32_t w, uint32_t& next,
+                                          uint32_t* dst) {
+    const int lane = threadIdx.x & 31;
+    for (int base = 0; base < got; base += 32) {
+        const int p = base + lane;
+        bool start = false;
+        uint32_t x = kSentinel;
+        uint32_t mult = 0;
+        if (p < got) {
+            x = buf[p];
+            start = (p == 0) || (buf[p - 1] != x);
+            if (start) {
+                mult = 1;
+                while (p + (int)mult < got && buf[p + mult] == x) ++mult;
+            }
+        }
+        uint32_t todo = __ballot_sync(0xFFFFFFFFu, start);
+        while (todo) {  // one layer a round
+            const uint32_t m = __shfl_sync(0xFFFFFFFFu, mult, __ffs(todo) - 1);
+            const uint32_t bal = __ballot_sync(0xFFFFFFFFu, start && mult == m);
+            const uint32_t own = __ballot_sync(0xFFFFFFFFu, lane < l && w == m);
+            const int q = own ? __ffs(own) - 1 : 0;  // every multiplicity has its layer
+            const uint32_t at = __shfl_sync(0xFFFFFFFFu, next, q);
+            if (own && start && mult == m) dst[at + __popc(bal & lanemask_lt())] = x;
+            if (own && lane == q) next = at + __popc(bal);
+            todo &= ~bal;
+        }
+    }
+}
+
+__device__ __forceinline__ void memo_publish(const RRParams& P, int32_t mu, unsigned long long at) {
+    __threadfence();  // every lane's members before the slot
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) atomicExch(P.memo_slot + mu, kMemoFirst + (uint32_t)at);
+}
+
+// The picks (or all members) of the needed layers, read from the entry at `at`.
+template <class SM, class Sink>
+__device__ __forceinline__ void memo_take(const RRParams& P, SM& S, const Sink& sink, unsigned long long at,
+                                          uint32_t nneed) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t* picks = S.u.w.wpick[wid];
+    for (uint32_t q = 0; q < nneed; ++q) {
+        const Need nd = S.wneed[wid][q];
+        const uint32_t* m = P.memo + at + nd.before;
+        const uint32_t* pk = picks + S.wpoff[wid][q];
+        if (nd.h >= nd.n) {
+            for (uint32_t x = lane; x < nd.n; x += 32) sink.push(ld_strong(m + x));
+        } else {
+            for (uint32_t r = lane; r < nd.h; r += 32) sink.push(ld_strong(m + pk[r]));
+        }
+    }
+    __syncwarp();
+}
+
 // Returns true when the pop must be handed to the block path.
 template <class SM, class Sink>
 __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j, uint32_t ybase, int32_t mu) {
@@ -774,11 +880,11 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
     for (int c0 = 0; c0 < (lt ? 0 : l); c0 += 32) {
         const int i = c0 + lane;
         uint32_t h = 0, ksel = 0;
-        uint4 e = make_uint4(0, 0, 0, 0);
+        uint4 e = make_uint4(0, 0, 0, 0), f = e;
         bool drew = false;
         if (i < l) {
             e = P.prof[2 * (pb + i)];
-            const uint4 f = P.prof[2 * (pb + i) + 1];
+            f = P.prof[2 * (pb + i) + 1];
             WordStream ws;
             ws.init(P.seed, j, ybase, (uint32_t)mu, (uint32_t)(i + 1));
             drew = layer_draw(e, f, P.tab, P.strategy, ws, h, ksel);
@@ -786,7 +892,7 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
         const bool flag = h > 0;
         const uint32_t bal = __ballot_sync(0xFFFFFFFFu, flag);
         const uint32_t pos = nneed + __popc(bal & lanemask_lt());
-        if (flag && pos < kLQ) need[pos] = Need{e.x & ~kPOneFlag, e.y, h, ksel, (uint32_t)(i + 1)};
+        if (flag && pos < kLQ) need[pos] = Need{e.x & ~kPOneFlag, e.y, h, ksel, (uint32_t)(i + 1), f.w};
         hsum += h;
         nneed += __popc(bal);
         ndraw += __popc(__ballot_sync(0xFFFFFFFFu, drew));
@@ -802,6 +908,10 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
     if (nneed == 0) return false;
     hsum = __reduce_add_sync(0xFFFFFFFFu, hsum);
     const int32_t tsum = P.tsum[mu];
+    uint32_t kept = kMemoNone;  // read by one lane: the slot may change while the warp reads it
+    if (P.memo_slot && dh != 1 && lane == 0) kept = ld_strong(P.memo_slot + mu);
+    kept = __shfl_sync(0xFFFFFFFFu, kept, 0);
+    const bool hit = kept >= kMemoFirst && kept < kMemoBusy;
     if (lane == 0) {
         wst[S_SEL] += hsum;
         wst[S_MATS] += 1;
@@ -822,8 +932,17 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
     // a chunk index lets the warp read only the id ranges that hold the picks (and the members
     // of layers taken whole, when there are few of them)
     uint64_t iw = 0;
-    if (dh != 1 && T > kIdxMinT && total_picks + take_all_n <= (uint32_t)kPCap) iw = P.idx[mu];
-    if (dh != 1 && iw == 0 && T > kWCap) return true;
+    const uint32_t wanted = total_picks + take_all_n;
+    if (!hit && dh != 1 && T > kIdxMinT) iw = P.idx[mu];
+    // a neighbourhood to keep: sorted whole anyway, or so many picks that a visit of every chunk
+    // costs no more than two such pops
+    unsigned long long keep_at = ~0ull;
+    if (P.memo_slot && !hit && kept <= kMemoSeen && dh != 1 && l <= 32 &&
+        (iw == 0 ? T <= kWCap : 2ull * wanted >= 1ull << (iw >> kIdxBitsShift)))
+        keep_at = memo_touch(P, mu, pb, l, kept);
+    const bool keep = keep_at != ~0ull;
+    if (!keep && wanted > (uint32_t)kPCap) iw = 0;
+    if (!hit && dh != 1 && iw == 0 && T > kWCap) return true;
     uint32_t* picks = S.u.w.wpick[wid];
     uint32_t* poff = S.wpoff[wid];
     uint32_t acc = 0;
@@ -868,8 +987,37 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
         __syncwarp();
         return false;
     }
+    if (hit) {
+        if (lane == 0) wst[S_GATH] += (unsigned long long)wanted - (unsigned long long)tsum;
+        memo_take(P, S, sink, kept - kMemoFirst, nneed);
+        return false;
+    }
     uint32_t* buf = S.u.w.wbuf[wid];
     int* cnt = S.wcnt[wid];
+    // lane i: layer i's w, and where its next member goes
+    uint32_t keep_w = 0, keep_next = 0;
+    if (keep && lane < l) {
+        keep_w = P.prof[2 * (pb + lane)].x & ~kPOneFlag;
+        keep_next = P.prof[2 * (pb + lane) + 1].w;
+    }
+    if (keep && iw != 0) {
+        const int c = (int)(iw >> kIdxBitsShift), sh = P.id_bits - c;
+        uint32_t probes = 0;
+        for (int k = 0; k < (1 << c); ++k) {
+            const int got = chunk_nbhd(P, S, mu, v_begin, dh, (uint32_t)k << sh, sh, buf, probes);
+            if (got < 0) {
+                if (lane == 0) dev_fail(P.st, kErrBucket, mu);
+                return false;
+            }
+            memo_emit(buf, got, l, keep_w, keep_next, P.memo + keep_at);
+            __syncwarp();  // buf is free again
+        }
+        probes = __reduce_add_sync(0xFFFFFFFFu, probes);
+        if (lane == 0) wst[S_SRCH] += (unsigned long long)probes + 2ull * (unsigned long long)dh * ((1 << c) - 1);
+        memo_publish(P, mu, keep_at);
+        memo_take(P, S, sink, keep_at, nneed);
+        return false;
+    }
     if (iw != 0) {
         // chunk path: lane q follows needed layer q through its row of prefix counts: the next
         // position it needs (its next pick, or for a layer taken whole its next member) and the
@@ -946,6 +1094,10 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
     } else {
         got = sorted_nbhd<32>(P.v_span, P.he_mem, mu, v_begin, dh, T, P.id_bits, buf,
                               S.u.w.wbkt[wid], kWBucketBits, S.wpre[wid], nullptr);
+    }
+    if (keep) {
+        memo_emit(buf, got, l, keep_w, keep_next, P.memo + keep_at);
+        memo_publish(P, mu, keep_at);
     }
     for (uint32_t q = lane; q < nneed; q += 32) cnt[q] = 0;
     __syncwarp();
@@ -1070,7 +1222,7 @@ __device__ __noinline__ void pop_block(const RRParams& P, Shared& S, const Sink&
                 const uint32_t bal = __ballot_sync(0xFFFFFFFFu, flag);
                 const uint32_t pos = nneed + __popc(bal & lanemask_lt());
                 if (flag && pos >= round_lo && pos < round_lo + kBLQ)
-                    S.bneed[pos - round_lo] = Need{e.x & ~kPOneFlag, e.y, h, ksel, (uint32_t)(i + 1)};
+                    S.bneed[pos - round_lo] = Need{e.x & ~kPOneFlag, e.y, h, ksel, (uint32_t)(i + 1), 0u};
                 nneed += __popc(bal);
             }
             __syncwarp();
@@ -1965,7 +2117,7 @@ hyperim_status ensure_scratch(hyperim_graph* g, int blocks, bool vis_smem) {
     if (S.bitmap) dev_free(g, S.bitmap, sizeof(uint32_t) * S.bitmap_words * S.blocks);
     if (S.picks) dev_free(g, S.picks, sizeof(uint32_t) * S.pick_cap * S.blocks);
     if (S.big) dev_free(g, S.big, sizeof(uint32_t) * S.big_cap * S.blocks);
-    S = Scratch{0, 0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, S.arena, S.arena_cap};
+    S = Scratch{0, 0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, S.arena, S.arena_cap, S.memo_slot, S.memo, S.memo_cap};
     hyperim_status st;
     if ((st = dev_alloc(g, (void**)&S.list, sizeof(int32_t) * list_cap * blocks))) return st;
     HYP_CUDA(cudaMemsetAsync(S.list, 0xFF, sizeof(int32_t) * list_cap * blocks, g->stream));  // empty slots
@@ -1981,6 +2133,39 @@ hyperim_status ensure_scratch(hyperim_graph* g, int blocks, bool vis_smem) {
     S.pick_cap = pick_cap;
     S.big_cap = big_cap;
     return HYPERIM_OK;
+}
+
+// Whether a growth step uses the memo: pools' new sets x their mean size so far against n.
+bool memo_pays(const hyperim_graph* g, hyperim_pool* const* pools, int npools, const int64_t* pool_start) {
+    double pops = 0.0;
+    for (int q = 0; q < npools; ++q) {
+        const double hint = pools[q]->mean_size_hint > 0 ? pools[q]->mean_size_hint : g->set_size_hint;
+        if (hint <= 0.0) return true;
+        pops += (double)(pool_start[q + 1] - pool_start[q]) * hint;
+    }
+    return pops >= kMemoPops * (double)g->n;
+}
+
+// Entries of the memo that a growth step of njobs sets may use.
+uint64_t memo_want(int64_t sum_tsum, int64_t njobs) {
+    return std::min<uint64_t>({kMemoMax, (uint64_t)std::max<int64_t>(sum_tsum, 1), (uint64_t)njobs * kMemoPerSet});
+}
+
+// The handle's memo, large enough for a growth step of njobs sets. A graph with a budget gets none
+// (its budget stays for what a growth step cannot do without), nor does one without the memory.
+void ensure_memo(hyperim_graph* g, int64_t njobs) {
+    Scratch& S = g->scratch;
+    const uint64_t want = memo_want(g->sum_tsum, njobs);
+    if (S.memo && S.memo_cap >= want) return;
+    free_memo(g);
+    if (graph_root(g)->budget) return;
+    if (dev_alloc(g, (void**)&S.memo_slot, sizeof(uint32_t) * (size_t)g->n) != HYPERIM_OK) return;
+    if (dev_alloc(g, (void**)&S.memo, sizeof(uint32_t) * want) != HYPERIM_OK) {
+        dev_free(g, S.memo_slot, sizeof(uint32_t) * (size_t)g->n);
+        S.memo_slot = nullptr;
+        return;
+    }
+    S.memo_cap = want;
 }
 
 // Output arena entries for a growth step: 1.25 x the expected members (each pool's mean set size
@@ -2145,6 +2330,8 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     int blocks = g->sm_count * per_sm;
     if ((int64_t)blocks > njobs) blocks = (int)njobs;
     if ((st = ensure_scratch(g, blocks, vis_smem))) return st;
+    const bool use_memo = memo_pays(g, pools, npools, pool_start);
+    if (use_memo) ensure_memo(g, njobs);
 
     const uint64_t want = arena_want(g, pools, npools, pool_start, g->n);
     // the warp phase (one RR set per warp) runs first in the persistent schedule, unless the
@@ -2166,6 +2353,7 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
         int pad;
         unsigned long long arena_used;
         unsigned long long set_cycles[3];  // sum, max, count over the sets the block kernel built
+        unsigned long long memo_used;
     };
     int64_t* d_pos = nullptr;
     int32_t* d_size = nullptr;
@@ -2254,6 +2442,11 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     P.rewrite = 0;
     HYP_CUDA(cudaMemsetAsync(d_ctrl, 0, sizeof(Ctrl), s));
     HYP_CUDA(cudaMemsetAsync(g->d_counters, 0, sizeof(RRCounters) * kMaxPools, s));
+    P.memo_slot = use_memo ? g->scratch.memo_slot : nullptr;
+    P.memo = g->scratch.memo;
+    P.memo_cap = g->scratch.memo_cap;
+    P.memo_used = &d_ctrl->memo_used;
+    if (P.memo_slot) HYP_CUDA(cudaMemsetAsync(P.memo_slot, 0, sizeof(uint32_t) * (size_t)g->n, s));
     HYP_CUDA(cudaEventRecord(ev0, s));
     if (P.plain) {
         // the comparison form: one launch per batch of `blocks` sets, one set per block
@@ -2431,6 +2624,7 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
         int next_job;
         int rerun_count;  // sets listed for an arena repair
         unsigned long long arena_used;
+        unsigned long long memo_used;
     };
     int64_t* d_pos = nullptr;
     int32_t* d_size = nullptr;
@@ -2510,9 +2704,40 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
     double seconds = 0.0;
     if ((st = dev_alloc(g0, (void**)&arena.p, sizeof(int32_t) * want))) return st;
     arena.cap = want;
-    for (RRParams& P : hp) {
+    // the memo of this call, after every allocation the launch needs (and only without a budget): slots
+    // of every group's vertices, entries shared by all groups
+    uint32_t *memo_slot = nullptr, *memo = nullptr;
+    uint64_t memo_cap = 0;
+    auto pays = [&](int q) {
+        return memo_pays(groups[q].g, groups[q].pools, groups[q].npools, &pstart[(size_t)q * (kMaxPools + 1)]);
+    };
+    {
+        size_t slots = 0;
+        int64_t tsum_all = 0;
+        for (int q = 0; q < ngroups; ++q) {
+            if (!pays(q)) continue;
+            slots += (size_t)groups[q].g->n;
+            tsum_all += groups[q].g->sum_tsum;
+        }
+        const uint64_t entries = memo_want(tsum_all, njobs);
+        if (slots && !graph_root(g0)->budget && tmp.alloc(&memo_slot, sizeof(uint32_t) * slots) == HYPERIM_OK &&
+            tmp.alloc(&memo, sizeof(uint32_t) * entries) == HYPERIM_OK) {
+            memo_cap = entries;
+            HYP_CUDA(cudaMemsetAsync(memo_slot, 0, sizeof(uint32_t) * slots, s));
+        }
+    }
+    size_t slot0 = 0;
+    for (int q = 0; q < ngroups; ++q) {
+        RRParams& P = hp[q];
         P.arena = arena.p;
         P.arena_cap = arena.cap;
+        if (memo_cap && pays(q)) {
+            P.memo_slot = memo_slot + slot0;
+            P.memo = memo;
+            P.memo_cap = memo_cap;
+            P.memo_used = &d_ctrl->memo_used;
+            slot0 += (size_t)groups[q].g->n;
+        }
     }
     B.rerun = nullptr;
     B.rerun_count = nullptr;

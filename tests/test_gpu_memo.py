@@ -1,0 +1,58 @@
+"""Neighbourhoods kept within a growth step (the memo) change no RR set: a graph loaded with a budget
+has none, one without a budget has it. Sizes at its edges: 31 to 40 layers (kept up to 32), sorted
+whole (up to 2,048 members) and by chunks, more members than the memo has room for, hyperedges of
+everybody; every strategy; the batched launch."""
+import numpy as np
+import pytest
+
+from tests import gpu_cases as G
+
+pytestmark = pytest.mark.gpu
+
+ROOM = 1 << 36
+
+
+@pytest.fixture(scope="module")
+def H():
+    import paper_2406_01911_gb300 as H
+    H.lib()
+    return H
+
+
+GRAPHS = {
+    "hub": lambda: G.hub_graph(n=6000, hub_edges=40, hub_size=120, mid_edges=8, mid_size=200, m_rest=2500),
+    "layers31": lambda: G.layered_graph(depth=31),
+    "layers32": lambda: G.layered_graph(depth=32),
+    "layers33": lambda: G.layered_graph(depth=33),
+    "layers40": lambda: G.layered_graph(depth=40),
+    "chunks": lambda: G.layered_hub_graph(n=12000, groups=8, size=90, m_rest=3000),
+    "crowded": lambda: (24_000, [list(range(i, 24_000, 2)) + [i + 1] for i in range(2)] + [[0, 1, 2]]),
+    "degenerate": G.degenerate_graph,
+}
+
+
+@pytest.mark.parametrize("name", sorted(GRAPHS))
+@pytest.mark.parametrize("model,p", [("uniform_pair", 0.03), ("uniform_pair", 1.0), ("wc", 0.0), ("paper_layer", 0.0)])
+def test_memo_changes_no_set(H, name, model, p):
+    n, hes = GRAPHS[name]()
+    off, mem = G.csr(hes)
+    theta = 1 if name == "crowded" else 700
+    thr = int(p * G.P32)
+    a = H.Graph(n, off, mem, model, thr, seed=7)
+    b = H.Graph(n, off, mem, model, thr, seed=7, hbm_budget_bytes=ROOM)
+    for strategy in ("paper", "binomial_only", "lt"):
+        if name == "crowded" and strategy == "binomial_only":
+            continue
+        pa = a.pool(tag=0, roots="stratified", strategy=strategy).sample(theta)
+        pb = b.pool(tag=0, roots="stratified", strategy=strategy).sample(theta)
+        sa, sb = G.gpu_sets(pa), G.gpu_sets(pb)
+        assert sa[0] == sb[0] and np.array_equal(sa[1], sb[1]) and np.array_equal(sa[2], sb[2])
+        va, vb = pa.view(), pb.view()
+        for key in ("pops", "layers_seen", "draws", "mats", "mat_he", "mat_members", "selected", "sectors"):
+            assert va[key] == vb[key], key
+    qa = [(a, a.pool(2, "stratified"), a.pool(3, "stratified"), 2, 0.2, 1.0)]
+    qb = [(b, b.pool(2, "stratified"), b.pool(3, "stratified"), 2, 0.2, 1.0)]
+    if name != "crowded":
+        (s1, r1), = H.hyperim_select_seeds_batch(qa)
+        (s2, r2), = H.hyperim_select_seeds_batch(qb)
+        assert s1.tolist() == s2.tolist() and r1["lambda_r1"].tolist() == r2["lambda_r1"].tolist()
