@@ -4,14 +4,15 @@
 // roots), so sums do not depend on the order of the atomic updates. Each round: argmax over the
 // vertices not picked yet (ties to the lowest id), then the RR sets containing the winner that
 // are not covered yet are retired: marked covered, counted in Lambda_s, and their weight is
-// subtracted from the score of every member. The k rounds run back to back on the stream; the
-// winner of a round is read on the device by the next launch.
+// subtracted from the score of every member. The k rounds run inside one launch (k_greedy), whose
+// blocks meet at a barrier between them.
 #include <algorithm>
 #include <cstddef>
 #include <new>
 #include <string>
 #include <vector>
 
+#include "coverage.cuh"
 #include "internal.h"
 
 namespace hyperim {
@@ -112,23 +113,12 @@ __device__ __forceinline__ void scan_unpicked(const unsigned long long* __restri
     }
 }
 
-// argmax of score over unpicked vertices, lowest id on ties; the last block to finish reduces
-// the per-block winners, records the seed and marks it picked.
-// Eq. upper_2 state (see the top-k kernels below)
-struct TopK {
-    unsigned long long prefix;
-    unsigned int kleft, all;  // all: fewer unpicked vertices than k, so all of them count
-    unsigned long long cover;
-    unsigned long long best_lo, best_hi;
-    unsigned int ticket;
-    unsigned int first_pass;  // radix passes before it: every unpicked score's digit is 0 there
-};
-
+// argmax of score over unpicked vertices, lowest id on ties (the stepwise greedy, over a score vector
+// of the caller's); the last block to finish reduces the per-block winners and marks the seed picked.
 __global__ void __launch_bounds__(kArgThreads)
 k_argmax(const unsigned long long* __restrict__ score, uint8_t* __restrict__ picked, int32_t n,
          unsigned long long* __restrict__ bscore, uint32_t* __restrict__ bid,
-         unsigned int* __restrict__ ticket, int32_t* __restrict__ best, int32_t* __restrict__ seeds,
-         int round, TopK* __restrict__ tk) {
+         unsigned int* __restrict__ ticket, int32_t* __restrict__ best) {
     __shared__ unsigned long long ss[kArgThreads / 32];
     __shared__ uint32_t si[kArgThreads / 32];
     __shared__ bool last;
@@ -174,125 +164,9 @@ k_argmax(const unsigned long long* __restrict__ score, uint8_t* __restrict__ pic
         for (int w = 1; w < kArgThreads / 32; ++w)
             if (better(ss[w], si[w], bs, bi)) { bs = ss[w]; bi = si[w]; }
         *best = (int32_t)bi;
-        seeds[round] = (int32_t)bi;
         picked[bi] = 1;
-        // the winner's marginal weight, before its sets are retired; no unpicked score exceeds
-        // it, now or later (scores only decrease), so the radix passes above its leading digit
-        // can be skipped from here on
-        tk->cover += bs;
-        const int lead = bs ? (63 - __clzll((long long)bs)) : 0;
-        tk->first_pass = (unsigned int)((56 - (lead & ~7)) / 8);
         *ticket = 0;
     }
-}
-
-// ---- Eq. upper_2 (p_max = 1): the k largest scores among the vertices not picked yet ---------
-// A radix select over 8-bit digits, most significant first, finds the k-th largest score T
-// (prefix) and how many of its copies belong to the top k (kleft); the top-k sum is then the sum
-// of the scores above T plus kleft T. Every round's bound, cover + top-k sum, enters a running
-// minimum; all of it stays on the device between the greedy's launches. 128-bit sums are kept
-// as (lo, hi) pairs of 64-bit words.
-
-__device__ __forceinline__ void add128(unsigned long long& lo, unsigned long long& hi, unsigned long long a_lo,
-                                       unsigned long long a_hi) {
-    const unsigned long long l = lo + a_lo;
-    hi += a_hi + (l < lo ? 1ull : 0ull);
-    lo = l;
-}
-
-__global__ void k_topk_hist(const unsigned long long* __restrict__ score, const uint8_t* __restrict__ picked,
-                            int32_t n, const TopK* __restrict__ st, int pass, unsigned int* __restrict__ hist) {
-    __shared__ unsigned int h[256];
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) h[i] = 0;
-    __syncthreads();
-    // passes above the top bound's leading digit would find every candidate in digit 0: skipped
-    if (!st->all && pass >= (int)st->first_pass) {
-        const int sh = 56 - 8 * pass;
-        const unsigned long long prefix = st->prefix;
-        const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-        for (int64_t v0 = blockIdx.x * (int64_t)blockDim.x; v0 < n; v0 += stride) {
-            const int64_t v = v0 + threadIdx.x;
-            int d = -1;
-            if (v < n && !picked[v]) {
-                const unsigned long long x = score[v];
-                if (pass == 0 || (x >> (sh + 8)) == prefix) d = (int)((x >> sh) & 255u);
-            }
-            // one shared atomic per distinct digit of the warp
-            const unsigned int same = __match_any_sync(0xFFFFFFFFu, d);
-            if (d >= 0 && (threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&h[d], (unsigned int)__popc(same));
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 256; i += blockDim.x)
-        if (h[i]) atomicAdd(&hist[i], h[i]);
-}
-
-// one thread: the digit of the k-th largest among the candidates; clears the histogram
-__global__ void k_topk_select(TopK* __restrict__ st, unsigned int* __restrict__ hist, int pass) {
-    if (!st->all && pass >= (int)st->first_pass) {
-        unsigned int cum = 0;
-        int d = 255;
-        for (; d >= 0; --d) {
-            if (cum + hist[d] >= st->kleft) break;
-            cum += hist[d];
-        }
-        if (d < 0) {  // fewer candidates than k (only on the first pass): take every unpicked vertex
-            st->all = 1;
-            st->prefix = 0;
-            st->kleft = 0;
-        } else {
-            st->prefix = (st->prefix << 8) | (unsigned long long)d;
-            st->kleft -= cum;
-        }
-    }
-    for (int i = 0; i < 256; ++i) hist[i] = 0;
-}
-
-// sum of the scores above T = prefix over the unpicked vertices (grid reduction, last block
-// finishes): K = sum + kleft T; bound = cover + K; running minimum; state reset for next round
-__global__ void __launch_bounds__(kArgThreads)
-k_topk_sum(const unsigned long long* __restrict__ score, const uint8_t* __restrict__ picked, int32_t n,
-           TopK* __restrict__ st, unsigned long long* __restrict__ part, unsigned int k) {
-    __shared__ unsigned long long slo[kArgThreads / 32], shi[kArgThreads / 32];
-    __shared__ bool last;
-    const unsigned long long T = st->prefix;
-    unsigned long long lo = 0, hi = 0;
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        if (picked[v]) continue;
-        const unsigned long long x = score[v];
-        if (x > T) add128(lo, hi, x, 0ull);
-    }
-    for (int o = 16; o > 0; o >>= 1)
-        add128(lo, hi, __shfl_xor_sync(0xFFFFFFFFu, lo, o), __shfl_xor_sync(0xFFFFFFFFu, hi, o));
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) { slo[wid] = lo; shi[wid] = hi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < kArgThreads / 32; ++w) add128(lo, hi, slo[w], shi[w]);
-        part[2 * blockIdx.x] = lo;
-        part[2 * blockIdx.x + 1] = hi;
-        __threadfence();
-        last = atomicAdd(&st->ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last || threadIdx.x != 0) return;
-    __threadfence();
-    lo = 0;
-    hi = 0;
-    for (unsigned int b = 0; b < gridDim.x; ++b)
-        add128(lo, hi, ((volatile unsigned long long*)part)[2 * b], ((volatile unsigned long long*)part)[2 * b + 1]);
-    const unsigned long long kl = st->kleft;
-    add128(lo, hi, kl * T, __umul64hi(kl, T));
-    add128(lo, hi, st->cover, 0ull);
-    if (hi < st->best_hi || (hi == st->best_hi && lo < st->best_lo)) {
-        st->best_lo = lo;
-        st->best_hi = hi;
-    }
-    st->prefix = 0;
-    st->kleft = k;
-    st->all = 0;
-    st->ticket = 0;
 }
 
 // retire the uncovered RR sets containing the round's winner; one warp per inverted entry
@@ -319,11 +193,435 @@ __global__ void k_retire(const int32_t* __restrict__ best, const int64_t* __rest
     }
 }
 
+// ---- the k rounds in one launch -----------------------------------------------------------------
+// What a round costs is not its arithmetic: with one launch for the argmax and one for the
+// retirement, 2M vertices and 100 to 200 rounds, a round took 19 us for 1 us of score reads. So
+//   - only vertices that some RR set of the view holds take part ("active": a tenth to a third of
+//     2M), numbered 0..na-1, their scores side by side, the RR sets' members renumbered to match:
+//     the argmax reads 8 bytes per active vertex;
+//   - a picked vertex needs no flag, its score is 0 once its sets are retired; when the best score is
+//     0 the rest of the seeds are the lowest ids not picked yet;
+//   - all rounds run in one cooperative launch (its blocks are resident together by the launch's
+//     contract) with two barriers a round; block winners are reduced by every block for itself, so
+//     the winner needs no third one. The barrier's wait is bounded (kErrSpin).
+// A block for every 16K members of the pool, one block (no barrier) for small pools. 200 rounds on the pools
+// of 40,000 sets of that graph: 4.0 ms before, 2.7 ms now (14 us a round: two barriers and a chain of
+// about ten dependent L2 reads); the index build 0.42 -> 0.14 ms with long sets spread over blocks. The
+// Eq. upper_2 bound took 17 launches a round (35 ms of a 100 ms query), now none of its own.
+constexpr int kGThreads = 512;
+constexpr int kGWarps = kGThreads / 32;
+constexpr int64_t kGMembersPerBlock = 1 << 14;
+constexpr int kGSpin = 1 << 24;  // rounds of a barrier wait (seconds) before it gives up
+constexpr int kTopBits = 11;
+constexpr int kTopBins = 1 << kTopBits;
+
+// active vertices: act[c] = v, cidx[v] = c (any order), score[c] = 0; the counts are cleared for
+// the scatter. nact: one word, zeroed by the caller.
+constexpr int kActThreads = 256, kActItems = 8;
+__global__ void __launch_bounds__(kActThreads)
+k_active(uint32_t* __restrict__ cnt, int32_t n, int32_t* __restrict__ act, uint32_t* __restrict__ cidx,
+         unsigned long long* __restrict__ score, unsigned int* __restrict__ nact) {
+    __shared__ int wsum[kActThreads / 32];
+    __shared__ unsigned int base_s;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t v0 = (int64_t)blockIdx.x * (kActThreads * kActItems);
+    uint32_t flags = 0;
+    int mine[kActItems];
+    int run = 0;  // active vertices of this warp so far
+#pragma unroll
+    for (int i = 0; i < kActItems; ++i) {
+        const int64_t v = v0 + (wid * kActItems + i) * 32 + lane;
+        const bool f = v < n && cnt[v] != 0;
+        const uint32_t b = __ballot_sync(0xFFFFFFFFu, f);
+        mine[i] = run + __popc(b & ((1u << lane) - 1u));
+        run += __popc(b);
+        if (f) {
+            flags |= 1u << i;
+            cnt[v] = 0;
+        }
+    }
+    if (lane == 0) wsum[wid] = run;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int w = 0; w < kActThreads / 32; ++w) {
+            const int c = wsum[w];
+            wsum[w] = t;
+            t += c;
+        }
+        base_s = t ? atomicAdd(nact, (unsigned int)t) : 0u;
+    }
+    __syncthreads();
+    const uint32_t base = base_s + (uint32_t)wsum[wid];
+#pragma unroll
+    for (int i = 0; i < kActItems; ++i) {
+        if (!(flags >> i & 1u)) continue;
+        const int32_t v = (int32_t)(v0 + (wid * kActItems + i) * 32 + lane);
+        const uint32_t c = base + (uint32_t)mine[i];
+        act[c] = v;
+        cidx[v] = c;
+        score[c] = 0;
+    }
+}
+
+// RR sets taken by blocks: a batch of kSetsPerWarp sets per warp; a warp does a set of up to kLongSet
+// members alone, longer ones are left to the whole block after its warps are done. (Sets are tiny at the
+// median and 10,000 members at the end of their tail: with one warp per set whatever its size, the longest
+// set's 400 dependent steps were what a launch or a round waited for.)
+// find(i, x0, x1, tag): whether item i takes part, its member range and a tag; body(x, tag).
+constexpr int kLongSet = 256;
+constexpr int kSetsPerWarp = 2;
+struct LongSets {
+    int64_t x0[kGWarps * kSetsPerWarp], x1[kGWarps * kSetsPerWarp];
+    unsigned long long tag[kGWarps * kSetsPerWarp];
+    int count;
+};
+template <typename Find, typename Body>
+__device__ __forceinline__ void block_sets(LongSets& S, int64_t items, Find&& find, Body&& body) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // consecutive items go to different blocks: few long ones still spread over the grid
+    const int64_t batch = (int64_t)gridDim.x * kGWarps * kSetsPerWarp;
+    for (int64_t i0 = blockIdx.x; i0 < items; i0 += batch) {
+        if (threadIdx.x == 0) S.count = 0;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kSetsPerWarp; ++q) {
+            const int64_t i = i0 + (int64_t)(q * kGWarps + wid) * gridDim.x;
+            int64_t x0 = 0, x1 = 0;
+            unsigned long long tag = 0;
+            if (i >= items || !find(i, x0, x1, tag)) continue;
+            if (x1 - x0 <= kLongSet) {
+                for (int64_t x = x0 + lane; x < x1; x += 32) body(x, tag);
+            } else if (lane == 0) {
+                const int at = atomicAdd(&S.count, 1);
+                S.x0[at] = x0;
+                S.x1[at] = x1;
+                S.tag[at] = tag;
+            }
+        }
+        __syncthreads();
+        const int todo = S.count;
+        for (int q = 0; q < todo; ++q) {
+            const int64_t x1 = S.x1[q];
+            const unsigned long long tag = S.tag[q];
+#pragma unroll 4
+            for (int64_t x = S.x0[q] + threadIdx.x; x < x1; x += kGThreads) body(x, tag);
+        }
+        __syncthreads();
+    }
+}
+
+// inverted index (vertex -> RR ids), the members' numbers and the initial scores
+__global__ void __launch_bounds__(kGThreads)
+k_scatter_active(const int64_t* __restrict__ rr_off, const int32_t* __restrict__ mem,
+                 const uint8_t* __restrict__ rr_stratum, const uint32_t* __restrict__ rr_j,
+                 int64_t N, Limits L, const int64_t* __restrict__ inv_off,
+                 uint32_t* __restrict__ cur, uint32_t* __restrict__ inv,
+                 const uint32_t* __restrict__ cidx, uint32_t* __restrict__ memc,
+                 unsigned long long* __restrict__ score, Weights W) {
+    __shared__ LongSets S;
+    block_sets(
+        S, N,
+        [&](int64_t r, int64_t& x0, int64_t& x1, unsigned long long& tag) {
+            if (L.skip(rr_stratum, rr_j, r)) return false;
+            x0 = rr_off[r];
+            x1 = rr_off[r + 1];
+            tag = (unsigned long long)r << 4 | (unsigned long long)rr_stratum[r];
+            return true;
+        },
+        [&](int64_t x, unsigned long long tag) {
+            const int32_t v = mem[x];
+            const uint32_t c = cidx[v];
+            inv[inv_off[v] + atomicAdd(&cur[v], 1u)] = (uint32_t)(tag >> 4);
+            memc[x] = c;
+            atomicAdd(&score[c], W.w[tag & 15]);
+        });
+}
+
+struct GreedyOut {
+    unsigned long long lam[HYPERIM_NSTRATA];
+    unsigned long long best_lo, best_hi;  // Eq. upper_2: the least bound (prefix mode)
+};
+
+struct GreedyParams {
+    const int32_t* act;
+    unsigned long long* score;   // by number
+    const unsigned int* nact;
+    const int64_t* inv_off;      // by vertex
+    const uint32_t* inv;
+    const int64_t* rr_off;
+    const uint32_t* memc;
+    const uint8_t* rr_stratum;
+    uint8_t* covered;            // per RR set
+    uint8_t* picked;             // per vertex
+    int32_t* seeds;
+    GreedyOut* out;
+    Weights W;
+    int32_t n, k;
+    int prefix;                  // 1: also the Eq. upper_2 bound of every prefix of the seeds
+    unsigned long long* pscore;  // per block
+    uint32_t* pid;               // per block: vertex, number
+    unsigned long long* psum;    // per block: 128-bit partial sums
+    unsigned int* hist;          // 3 x kTopBins, zeroed
+    unsigned int* bar;           // zeroed
+    DevStatus* st;
+};
+
+// All blocks of the launch meet; false when the bounded wait gave up here.
+__device__ bool grid_meet(const GreedyParams& P, unsigned int& target) {
+    __shared__ int ok_s;
+    __syncthreads();
+    if (gridDim.x == 1) return true;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        target += gridDim.x;
+        atomicAdd(P.bar, 1u);
+        int it = 0;
+        unsigned int seen;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(P.bar) : "memory");
+        } while ((int)(seen - target) < 0 && ++it < kGSpin);
+        ok_s = (int)(seen - target) >= 0;
+        if (!ok_s && atomicCAS(&P.st->code, 0, (int32_t)kErrSpin) == 0) P.st->detail = -1;
+        __threadfence();
+    }
+    __syncthreads();
+    return ok_s != 0;
+}
+
+__device__ __forceinline__ void add128(unsigned long long& lo, unsigned long long& hi, unsigned long long a_lo,
+                                       unsigned long long a_hi) {
+    const unsigned long long l = lo + a_lo;
+    hi += a_hi + (l < lo ? 1ull : 0ull);
+    lo = l;
+}
+
+// Eq. upper_2 (p_max = 1) for the seeds so far: cover plus the sum of the k largest scores (a picked or
+// inactive vertex counts 0), entered into block 0's running minimum. A radix select over 11-bit digits
+// below the largest score `top`, most significant first, finds the k-th largest score T and how
+// many of its copies belong to the top k; a digit of 0 is never counted (most scores have it), it is
+// what is left when the others hold fewer than k. Three histograms rotate: the next one is cleared
+// between the barriers that separate its last readers from its next writers.
+__device__ bool topk_bound(const GreedyParams& P, unsigned int na, unsigned long long top, unsigned long long cover,
+                           unsigned int* h, int& turn, unsigned int& target, unsigned long long& best_lo,
+                           unsigned long long& best_hi) {
+    __shared__ unsigned long long slo[kGWarps], shi[kGWarps];
+    __shared__ unsigned int digit_s, left_s;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t t0 = blockIdx.x * (int64_t)kGThreads + threadIdx.x, T = (int64_t)gridDim.x * kGThreads;
+    unsigned long long prefix = 0;
+    unsigned int kleft = (unsigned int)P.k;
+    const int bits = top ? 64 - __clzll((long long)top) : 0;
+    for (int sh = ((bits + kTopBits - 1) / kTopBits - 1) * kTopBits; sh >= 0; sh -= kTopBits) {
+        unsigned int* hist = P.hist + turn * kTopBins;
+        const int next = turn == 2 ? 0 : turn + 1;
+        for (int i = threadIdx.x; i < kTopBins; i += kGThreads) {
+            h[i] = 0;
+            if (blockIdx.x == 0) P.hist[next * kTopBins + i] = 0;
+        }
+        __syncthreads();
+        for (int64_t c = t0; c < na; c += T) {
+            const unsigned long long x = __ldcg(P.score + c);
+            const unsigned long long above = sh + kTopBits >= 64 ? 0ull : x >> (sh + kTopBits);
+            const unsigned int d = (unsigned int)(x >> sh) & (kTopBins - 1);
+            if (above == prefix && d) atomicAdd(&h[d], 1u);
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < kTopBins; i += kGThreads)
+            if (h[i]) atomicAdd(&hist[i], h[i]);
+        if (!grid_meet(P, target)) return false;
+        if (wid == 0) {  // lane i: digits [64 i, 64 i + 64), from the highest lane down
+            constexpr int per = kTopBins / 32;
+            unsigned int sum = 0;
+            for (int i = 0; i < per; ++i) sum += __ldcg(hist + lane * per + i);
+            unsigned int suf = sum;  // this lane's digits and all higher ones
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned int t = __shfl_down_sync(0xFFFFFFFFu, suf, o);
+                if (lane + o < 32) suf += t;
+            }
+            const uint32_t reach = __ballot_sync(0xFFFFFFFFu, suf >= kleft);
+            if (reach == 0) {
+                if (lane == 0) {
+                    digit_s = 0;
+                    left_s = kleft - suf;
+                }
+            } else if (lane == 31 - __clz(reach)) {
+                unsigned int cum = suf - sum;
+                int i = per - 1;
+                for (; i > 0; --i) {
+                    const unsigned int v = __ldcg(hist + lane * per + i);
+                    if (cum + v >= kleft) break;
+                    cum += v;
+                }
+                digit_s = (unsigned int)(lane * per + i);
+                left_s = kleft - cum;
+            }
+        }
+        __syncthreads();
+        prefix = (prefix << kTopBits) | digit_s;
+        kleft = left_s;
+        turn = next;
+        __syncthreads();
+    }
+    unsigned long long lo = 0, hi = 0;
+    for (int64_t c = t0; c < na; c += T) {
+        const unsigned long long x = __ldcg(P.score + c);
+        if (x > prefix) add128(lo, hi, x, 0ull);
+    }
+    for (int o = 16; o > 0; o >>= 1)
+        add128(lo, hi, __shfl_xor_sync(0xFFFFFFFFu, lo, o), __shfl_xor_sync(0xFFFFFFFFu, hi, o));
+    if (lane == 0) {
+        slo[wid] = lo;
+        shi[wid] = hi;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kGWarps; ++w) add128(lo, hi, slo[w], shi[w]);
+        P.psum[2 * blockIdx.x] = lo;
+        P.psum[2 * blockIdx.x + 1] = hi;
+    }
+    if (!grid_meet(P, target)) return false;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        lo = hi = 0;
+        for (unsigned int b = 0; b < gridDim.x; ++b) add128(lo, hi, __ldcg(P.psum + 2 * b), __ldcg(P.psum + 2 * b + 1));
+        add128(lo, hi, kleft * prefix, __umul64hi(kleft, prefix));
+        add128(lo, hi, cover, 0ull);
+        if (hi < best_hi || (hi == best_hi && lo < best_lo)) {
+            best_lo = lo;
+            best_hi = hi;
+        }
+    }
+    return true;
+}
+
+__global__ void __launch_bounds__(kGThreads) k_greedy(GreedyParams P) {
+    __shared__ unsigned long long s_lam[HYPERIM_NSTRATA];
+    __shared__ unsigned long long ss[kGWarps];
+    __shared__ uint32_t si[kGWarps], sc[kGWarps];
+    __shared__ unsigned long long win_s;
+    __shared__ uint32_t win_v;
+    __shared__ unsigned int h[kTopBins];
+    __shared__ LongSets sets;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t t0 = blockIdx.x * (int64_t)kGThreads + threadIdx.x, T = (int64_t)gridDim.x * kGThreads;
+    const unsigned int na = *P.nact;
+    unsigned int target = 0;
+    int turn = 0;
+    unsigned long long cover = 0, best_lo = ~0ull, best_hi = ~0ull;
+    if (threadIdx.x < HYPERIM_NSTRATA) s_lam[threadIdx.x] = 0;
+    __syncthreads();
+    int32_t round = 0;
+    for (;; ++round) {
+        if (round == P.k && !P.prefix) break;
+        // the best (score, lowest id): per block, then over the blocks' winners by every block
+        unsigned long long bs = 0;
+        uint32_t bi = 0xFFFFFFFFu;
+        auto take = [&](unsigned long long x, int64_t c) {
+            if (x > bs || (x == bs && x)) {
+                const uint32_t v = (uint32_t)P.act[c];
+                if (better(x, v, bs, bi)) { bs = x; bi = v; }
+            }
+        };
+        const int64_t na4 = na >> 2;
+        for (int64_t q = t0; q < na4; q += T) {
+            const ulonglong2 a = __ldcg(reinterpret_cast<const ulonglong2*>(P.score) + 2 * q);
+            const ulonglong2 b = __ldcg(reinterpret_cast<const ulonglong2*>(P.score) + 2 * q + 1);
+            take(a.x, 4 * q);
+            take(a.y, 4 * q + 1);
+            take(b.x, 4 * q + 2);
+            take(b.y, 4 * q + 3);
+        }
+        for (int64_t c = 4 * na4 + t0; c < na; c += T) take(__ldcg(P.score + c), c);
+        auto reduce = [&]() {  // over the block; the result is thread 0's
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long os = __shfl_xor_sync(0xFFFFFFFFu, bs, o);
+                const uint32_t oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
+                if (better(os, oi, bs, bi)) { bs = os; bi = oi; }
+            }
+            if (lane == 0) { ss[wid] = bs; si[wid] = bi; }
+            __syncthreads();
+            if (wid == 0) {
+                bs = lane < kGWarps ? ss[lane] : 0ull;
+                bi = lane < kGWarps ? si[lane] : 0xFFFFFFFFu;
+                for (int o = 16; o > 0; o >>= 1) {
+                    const unsigned long long os = __shfl_xor_sync(0xFFFFFFFFu, bs, o);
+                    const uint32_t oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
+                    if (better(os, oi, bs, bi)) { bs = os; bi = oi; }
+                }
+            }
+        };
+        reduce();
+        if (gridDim.x > 1) {
+            if (threadIdx.x == 0) {
+                P.pscore[blockIdx.x] = bs;
+                P.pid[blockIdx.x] = bi;
+            }
+            if (!grid_meet(P, target)) return;
+            bs = 0;
+            bi = 0xFFFFFFFFu;
+            for (int b = threadIdx.x; b < (int)gridDim.x; b += kGThreads) {
+                const unsigned long long x = __ldcg(P.pscore + b);
+                const uint32_t v = __ldcg(P.pid + b);
+                if (better(x, v, bs, bi)) { bs = x; bi = v; }
+            }
+            reduce();
+        }
+        if (threadIdx.x == 0) {
+            win_s = bs;
+            win_v = bi;
+        }
+        __syncthreads();
+        const unsigned long long win = win_s;
+        const uint32_t v = win_v;
+        if (P.prefix && !topk_bound(P, na, win, cover, h, turn, target, best_lo, best_hi)) return;
+        if (round == P.k || win == 0) break;
+        cover += win;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            P.seeds[round] = (int32_t)v;
+            P.picked[v] = 1;
+        }
+        // retire the winner's sets that are not covered yet (a set holds it once: one warp finds it)
+        const int64_t b = P.inv_off[v];
+        block_sets(
+            sets, P.inv_off[v + 1] - b,
+            [&](int64_t t, int64_t& x0, int64_t& x1, unsigned long long& tag) {
+                const uint32_t r = P.inv[b + t];
+                x0 = P.rr_off[r];
+                x1 = P.rr_off[r + 1];
+                const int s = P.rr_stratum[r];
+                if (__ldcg(P.covered + r)) return false;
+                __syncwarp();
+                if (lane == 0) {
+                    __stcg(P.covered + r, (uint8_t)1);
+                    atomicAdd(&s_lam[s], 1ull);
+                }
+                tag = 0ull - P.W.w[s];
+                return true;
+            },
+            [&](int64_t x, unsigned long long neg) { atomicAdd(&P.score[P.memc[x]], neg); });
+        if (!grid_meet(P, target)) return;
+    }
+    __syncthreads();
+    if (threadIdx.x < HYPERIM_NSTRATA && s_lam[threadIdx.x]) atomicAdd(&P.out->lam[threadIdx.x], s_lam[threadIdx.x]);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        P.out->best_lo = best_lo;
+        P.out->best_hi = best_hi;
+        // every set is covered: the lowest ids not picked yet
+        for (int32_t v = 0; round < P.k; ++round, ++v) {
+            while (P.picked[v]) ++v;
+            P.seeds[round] = v;
+        }
+    }
+}
+
 // coverage of a seed set: RR sets with at least one member in S, per stratum; one warp per set
 __global__ void k_coverage(const int64_t* __restrict__ rr_off, const int32_t* __restrict__ mem,
                            const uint8_t* __restrict__ rr_stratum, const uint32_t* __restrict__ rr_j,
                            int64_t N, Limits L, const uint8_t* __restrict__ in_s,
                            unsigned long long* __restrict__ lam) {
+    __shared__ unsigned int s_lam[HYPERIM_NSTRATA];  // 16 words for every hit would queue at the L2
+    if (threadIdx.x < HYPERIM_NSTRATA) s_lam[threadIdx.x] = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -335,8 +633,20 @@ __global__ void k_coverage(const int64_t* __restrict__ rr_off, const int32_t* __
             const int64_t x = base + lane;
             if (__any_sync(0xFFFFFFFFu, x < e && in_s[mem[x]] != 0)) { hit = true; break; }
         }
-        if (hit && lane == 0) atomicAdd(&lam[rr_stratum[r]], 1ull);
+        if (hit && lane == 0) atomicAdd(&s_lam[rr_stratum[r]], 1u);
     }
+    __syncthreads();
+    if (threadIdx.x < HYPERIM_NSTRATA && s_lam[threadIdx.x])
+        atomicAdd(&lam[threadIdx.x], (unsigned long long)s_lam[threadIdx.x]);
+}
+
+__global__ void __launch_bounds__(kCoverThreads)
+k_cover_sets(const int64_t* __restrict__ rr_off, const int32_t* __restrict__ mem, const uint8_t* __restrict__ rr_stratum,
+             const uint32_t* __restrict__ rr_j, int64_t N, Limits L, int32_t n, const int32_t* __restrict__ seeds,
+             int32_t k, int per, unsigned long long* __restrict__ lam) {
+    extern __shared__ uint32_t cover_slots[];
+    cover_sets(cover_slots, rr_off, mem, rr_stratum, N, n, seeds, k, per, lam,
+               [&](int64_t r) { return L.skip(rr_stratum, rr_j, r); });
 }
 
 __global__ void k_mark(const int32_t* __restrict__ seeds, int32_t k, uint8_t* __restrict__ in_s) {
@@ -536,89 +846,76 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
     for (int i = 0; i < HYPERIM_NSTRATA; ++i)
         W.w[i] = stratum_weight(g, p->root_mode, view_ns[i], i);
     hyperim_status st;
+    // blocks: by the pool's members, all resident together when more than one
+    int blocks = (int)std::min<int64_t>(std::max<int64_t>(T / kGMembersPerBlock, 1), sm);
+    if (blocks > 1) {
+        int per_sm = 0;
+        HYP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_greedy, kGThreads, 0));
+        blocks = std::max(1, std::min(blocks, per_sm * sm));
+    }
     CallBuffers tmp(g);
-    uint32_t *cnt = nullptr, *inv = nullptr, *covered = nullptr, *bid = nullptr, *ticket = nullptr;
+    uint32_t *cnt = nullptr, *inv = nullptr, *cidx = nullptr, *memc = nullptr, *pid = nullptr;
     int64_t* inv_off = nullptr;
-    unsigned long long *score = nullptr, *lam = nullptr, *bscore = nullptr;
-    uint8_t* picked = nullptr;
-    int32_t *best = nullptr, *seeds_d = nullptr;
-    const int ablocks = grid_cap(n, kArgThreads, sm, 2);
+    unsigned long long *score = nullptr, *pscore = nullptr, *psum = nullptr;
+    int32_t *act = nullptr, *seeds_d = nullptr;
+    // cleared together: the output record, barrier, counters, histograms, picked and covered flags
+    struct Zero {
+        GreedyOut out;
+        unsigned int bar, nact;
+        unsigned int hist[3 * kTopBins];
+    };
+    uint8_t* zero = nullptr;
+    const size_t bytes_zero = sizeof(Zero) + (size_t)n + (size_t)N;
     const size_t bytes_cnt = sizeof(uint32_t) * ((size_t)n + 1);
-    const size_t bytes_inv = sizeof(uint32_t) * (size_t)std::max<int64_t>(T, 1);
-    const size_t bytes_cov = sizeof(uint32_t) * (size_t)std::max<int64_t>(N, 1);
+    const size_t members = (size_t)std::max<int64_t>(T, 1);
     if ((st = tmp.alloc(&cnt, bytes_cnt))) return st;
     if ((st = tmp.alloc(&inv_off, sizeof(int64_t) * ((size_t)n + 1)))) return st;
-    if ((st = tmp.alloc(&inv, bytes_inv))) return st;
+    if ((st = tmp.alloc(&inv, sizeof(uint32_t) * members))) return st;
+    if ((st = tmp.alloc(&memc, sizeof(uint32_t) * members))) return st;
     if ((st = tmp.alloc(&score, sizeof(unsigned long long) * (size_t)n))) return st;
-    if ((st = tmp.alloc(&picked, (size_t)n))) return st;
-    if ((st = tmp.alloc(&covered, bytes_cov))) return st;
-    if ((st = tmp.alloc(&lam, sizeof(unsigned long long) * HYPERIM_NSTRATA))) return st;
-    if ((st = tmp.alloc(&bscore, sizeof(unsigned long long) * ablocks))) return st;
-    if ((st = tmp.alloc(&bid, sizeof(uint32_t) * ablocks))) return st;
-    if ((st = tmp.alloc(&ticket, sizeof(uint32_t) * 2))) return st;
-    if ((st = tmp.alloc(&best, sizeof(int32_t) * 2))) return st;
+    if ((st = tmp.alloc(&act, sizeof(int32_t) * (size_t)n))) return st;
+    if ((st = tmp.alloc(&cidx, sizeof(uint32_t) * (size_t)n))) return st;
+    if ((st = tmp.alloc(&zero, bytes_zero))) return st;
+    if ((st = tmp.alloc(&pscore, sizeof(unsigned long long) * 3 * (size_t)blocks))) return st;
+    if ((st = tmp.alloc(&pid, sizeof(uint32_t) * (size_t)blocks))) return st;
     if ((st = tmp.alloc(&seeds_d, sizeof(int32_t) * (size_t)k))) return st;
-    TopK* tk = nullptr;
-    unsigned int* hist = nullptr;
-    unsigned long long* part = nullptr;
-    const int tblocks = ablocks;
-    if ((st = tmp.alloc(&tk, sizeof(TopK)))) return st;
-    if ((st = tmp.alloc(&hist, sizeof(unsigned int) * 256))) return st;
-    if ((st = tmp.alloc(&part, sizeof(unsigned long long) * 2 * (size_t)tblocks))) return st;
-    {
-        TopK t0{};
-        t0.kleft = (unsigned int)k;
-        t0.best_lo = ~0ull;
-        t0.best_hi = ~0ull;
-        HYP_CUDA(cudaMemcpyAsync(tk, &t0, sizeof(TopK), cudaMemcpyHostToDevice, s));
-        HYP_CUDA(cudaMemsetAsync(hist, 0, sizeof(unsigned int) * 256, s));
-    }
-    auto topk_round = [&]() -> hyperim_status {
-        for (int pass = 0; pass < 8; ++pass) {
-            { k_topk_hist<<<tblocks, kArgThreads, 0, s>>>(score, picked, n, tk, pass, hist); count_launch(); }
-            { k_topk_select<<<1, 1, 0, s>>>(tk, hist, pass); count_launch(); }
-        }
-        { k_topk_sum<<<tblocks, kArgThreads, 0, s>>>(score, picked, n, tk, part, (unsigned int)k); count_launch(); }
-        return HYPERIM_OK;
-    };
+    psum = pscore + blocks;
+    Zero* z = reinterpret_cast<Zero*>(zero);
     HYP_CUDA(cudaMemsetAsync(cnt, 0, bytes_cnt, s));
-    HYP_CUDA(cudaMemsetAsync(score, 0, sizeof(unsigned long long) * (size_t)n, s));
-    HYP_CUDA(cudaMemsetAsync(picked, 0, (size_t)n, s));
-    HYP_CUDA(cudaMemsetAsync(covered, 0, bytes_cov, s));
-    HYP_CUDA(cudaMemsetAsync(lam, 0, sizeof(unsigned long long) * HYPERIM_NSTRATA, s));
-    HYP_CUDA(cudaMemsetAsync(ticket, 0, sizeof(uint32_t) * 2, s));
+    HYP_CUDA(cudaMemsetAsync(zero, 0, bytes_zero, s));
     if (T > 0 && !L.on) { k_count_occ<<<grid_cap(T, 256, sm, 32), 256, 0, s>>>(p->rr_mem, T, cnt); count_launch(); }
     if (T > 0 && L.on)
         { k_count_occ_view<<<grid_cap(N * 32, 256, sm, 32), 256, 0, s>>>(p->rr_off, p->rr_mem, p->rr_stratum,
                                                                         p->rr_j, N, L, cnt); count_launch(); }
     if ((st = exclusive_scan_u32_to_i64(g, cnt, inv_off, n))) return st;
-    HYP_CUDA(cudaMemsetAsync(cnt, 0, bytes_cnt, s));
+    { k_active<<<(unsigned)((n + kActThreads * kActItems - 1) / (kActThreads * kActItems)), kActThreads, 0, s>>>(
+          cnt, n, act, cidx, score, &z->nact); count_launch(); }
     if (N > 0)
-        { k_scatter_inv<<<grid_cap(N * 32, 256, sm, 32), 256, 0, s>>>(p->rr_off, p->rr_mem, p->rr_stratum,
-                                                                    p->rr_j, N, L, inv_off, cnt, inv, score,
-                                                                    W); count_launch(); }
-    const int rblocks = sm * 8;
-    for (int32_t round = 0; round < k; ++round) {
-        if (prefix_upper) topk_round();
-        { k_argmax<<<ablocks, kArgThreads, 0, s>>>(score, picked, n, bscore, bid, ticket, best, seeds_d,
-                                                 round, tk); count_launch(); }
-        { k_retire<<<rblocks, 256, 0, s>>>(best, inv_off, inv, p->rr_off, p->rr_mem, p->rr_stratum,
-                                         covered, score, lam, W); count_launch(); }
-    }
-    if (prefix_upper) topk_round();  // i = k: the whole seed set
+        { k_scatter_active<<<grid_cap(N * 32 / kSetsPerWarp, kGThreads, sm, 32), kGThreads, 0, s>>>(p->rr_off, p->rr_mem, p->rr_stratum, p->rr_j,
+                                                                       N, L, inv_off, cnt, inv, cidx, memc, score,
+                                                                       W); count_launch(); }
     HYP_CUDA(cudaGetLastError());
-    unsigned long long hl[HYPERIM_NSTRATA];
-    TopK th{};
-    HYP_CUDA(cudaMemcpyAsync(seeds_host, seeds_d, sizeof(int32_t) * (size_t)k, cudaMemcpyDeviceToHost, s));
-    HYP_CUDA(cudaMemcpyAsync(hl, lam, sizeof(hl), cudaMemcpyDeviceToHost, s));
-    HYP_CUDA(cudaMemcpyAsync(&th, tk, sizeof(TopK), cudaMemcpyDeviceToHost, s));
-    HYP_CUDA(cudaStreamSynchronize(s));
-    for (int i = 0; i < HYPERIM_NSTRATA; ++i) lambda_s[i] = hl[i];
-    if (prefix_upper) {
-        prefix_upper[0] = th.best_lo;
-        prefix_upper[1] = th.best_hi;
+    GreedyParams G{act, score, &z->nact, inv_off, inv, p->rr_off, memc, p->rr_stratum,
+                   zero + sizeof(Zero) + (size_t)n, zero + sizeof(Zero), seeds_d, &z->out, W, n, k,
+                   prefix_upper ? 1 : 0, pscore, pid, psum, z->hist, &z->bar, g->d_status};
+    if (blocks > 1) {
+        void* args[] = {&G};
+        HYP_CUDA(cudaLaunchCooperativeKernel((const void*)k_greedy, dim3((unsigned)blocks), dim3(kGThreads), args, 0, s));
+    } else {
+        k_greedy<<<1, kGThreads, 0, s>>>(G);
     }
-    return check_device_status(g, "greedy");
+    count_launch();
+    HYP_CUDA(cudaGetLastError());
+    GreedyOut out;
+    HYP_CUDA(cudaMemcpyAsync(seeds_host, seeds_d, sizeof(int32_t) * (size_t)k, cudaMemcpyDeviceToHost, s));
+    HYP_CUDA(cudaMemcpyAsync(&out, &z->out, sizeof(out), cudaMemcpyDeviceToHost, s));
+    if ((st = check_device_status(g, "greedy"))) return st;  // synchronises
+    for (int i = 0; i < HYPERIM_NSTRATA; ++i) lambda_s[i] = out.lam[i];
+    if (prefix_upper) {
+        prefix_upper[0] = out.best_lo;
+        prefix_upper[1] = out.best_hi;
+    }
+    return HYPERIM_OK;
 }
 
 hyperim_status coverage(hyperim_graph* g, hyperim_pool* p, const int32_t* seeds_host, int32_t k,
@@ -633,16 +930,22 @@ hyperim_status coverage(hyperim_graph* g, hyperim_pool* p, const int32_t* seeds_
     unsigned long long* lam = nullptr;
     int32_t* sd = nullptr;
     const size_t kk = (size_t)std::max(k, 1);
-    if ((st = tmp.alloc(&in_s, (size_t)g->n))) return st;
+    const bool on_chip = k <= kCoverSeeds;
+    if (!on_chip && (st = tmp.alloc(&in_s, (size_t)g->n))) return st;
     if ((st = tmp.alloc(&lam, sizeof(unsigned long long) * HYPERIM_NSTRATA))) return st;
     if ((st = tmp.alloc(&sd, sizeof(int32_t) * kk))) return st;
-    HYP_CUDA(cudaMemsetAsync(in_s, 0, (size_t)g->n, s));
     HYP_CUDA(cudaMemsetAsync(lam, 0, sizeof(unsigned long long) * HYPERIM_NSTRATA, s));
-    if (k > 0) {
-        HYP_CUDA(cudaMemcpyAsync(sd, seeds_host, sizeof(int32_t) * (size_t)k, cudaMemcpyHostToDevice, s));
+    if (k > 0) HYP_CUDA(cudaMemcpyAsync(sd, seeds_host, sizeof(int32_t) * (size_t)k, cudaMemcpyHostToDevice, s));
+    if (!on_chip) {
+        HYP_CUDA(cudaMemsetAsync(in_s, 0, (size_t)g->n, s));
         { k_mark<<<grid_cap(k, 256, g->sm_count, 4), 256, 0, s>>>(sd, k, in_s); count_launch(); }
     }
-    if (N > 0)
+    if (N > 0 && on_chip) {
+        const int per = cover_per(N, g->sm_count);
+        { k_cover_sets<<<grid_cap((N + per - 1) / per * 32, kCoverThreads, g->sm_count, 8), kCoverThreads,
+                       cover_smem(k), s>>>(p->rr_off, p->rr_mem, p->rr_stratum, p->rr_j, N, L, g->n, sd, k, per,
+                                           lam); count_launch(); }
+    } else if (N > 0)
         { k_coverage<<<grid_cap(N * 32, 256, g->sm_count, 32), 256, 0, s>>>(p->rr_off, p->rr_mem,
                                                                           p->rr_stratum, p->rr_j, N, L, in_s,
                                                                           lam); count_launch(); }
@@ -674,8 +977,7 @@ struct GreedyState {
     int64_t* inv_off = nullptr;
     unsigned long long *score = nullptr, *lam = nullptr, *bscore = nullptr;
     uint8_t* picked = nullptr;
-    int32_t *best = nullptr, *seed_d = nullptr;
-    TopK* tk = nullptr;
+    int32_t* best = nullptr;
     size_t bytes_cnt = 0, bytes_inv = 0, bytes_cov = 0;
 };
 
@@ -694,8 +996,6 @@ void free_state(GreedyState* s) {
     dev_free(g, s->bid, sizeof(uint32_t) * s->ablocks);
     dev_free(g, s->ticket, sizeof(uint32_t) * 2);
     dev_free(g, s->best, sizeof(int32_t) * 2);
-    dev_free(g, s->seed_d, sizeof(int32_t));
-    dev_free(g, s->tk, sizeof(TopK));
     cudaStreamSynchronize(g->stream);
     delete s;
 }
@@ -734,8 +1034,7 @@ hyperim_status greedy_begin(hyperim_graph* g, hyperim_pool* p, const uint64_t* l
         (st = dev_alloc(g, (void**)&s->lam, sizeof(unsigned long long) * HYPERIM_NSTRATA)) ||
         (st = dev_alloc(g, (void**)&s->bscore, sizeof(unsigned long long) * s->ablocks)) ||
         (st = dev_alloc(g, (void**)&s->bid, sizeof(uint32_t) * s->ablocks)) || (st = dev_alloc(g, (void**)&s->ticket, sizeof(uint32_t) * 2)) ||
-        (st = dev_alloc(g, (void**)&s->best, sizeof(int32_t) * 2)) || (st = dev_alloc(g, (void**)&s->seed_d, sizeof(int32_t))) ||
-        (st = dev_alloc(g, (void**)&s->tk, sizeof(TopK))))
+        (st = dev_alloc(g, (void**)&s->best, sizeof(int32_t) * 2)))
         return fail(st);
     cudaError_t e = cudaMemsetAsync(s->cnt, 0, s->bytes_cnt, st_);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->score, 0, sizeof(unsigned long long) * (size_t)n, st_);
@@ -743,7 +1042,6 @@ hyperim_status greedy_begin(hyperim_graph* g, hyperim_pool* p, const uint64_t* l
     if (e == cudaSuccess) e = cudaMemsetAsync(s->covered, 0, s->bytes_cov, st_);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->lam, 0, sizeof(unsigned long long) * HYPERIM_NSTRATA, st_);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->ticket, 0, sizeof(uint32_t) * 2, st_);
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->tk, 0, sizeof(TopK), st_);
     if (e != cudaSuccess) return fail(cuda_fail(e, "greedy state"));
     if (T > 0 && !L.on) { k_count_occ<<<grid_cap(T, 256, sm, 32), 256, 0, st_>>>(p->rr_mem, T, s->cnt); count_launch(); }
     if (T > 0 && L.on)
@@ -772,7 +1070,7 @@ hyperim_status greedy_pick(GreedyState* s, const unsigned long long* dev_total, 
     hyperim_pool* p = s->p;
     cudaStream_t st_ = g->stream;
     { k_argmax<<<s->ablocks, kArgThreads, 0, st_>>>(dev_total ? dev_total : s->score, s->picked, g->n, s->bscore, s->bid,
-                                                    s->ticket, s->best, s->seed_d, 0, s->tk); count_launch(); }
+                                                    s->ticket, s->best); count_launch(); }
     { k_retire<<<g->sm_count * 8, 256, 0, st_>>>(s->best, s->inv_off, s->inv, p->rr_off, p->rr_mem, p->rr_stratum,
                                                  s->covered, s->score, s->lam, s->W); count_launch(); }
     HYP_CUDA(cudaGetLastError());

@@ -1,15 +1,25 @@
 // hyperim_coverage_noalloc: the coverage step (RR sets of a pool hit by a seed set, per stratum)
-// for callers that must not allocate device memory. Its only scratch is a fixed array of seed
-// flags compiled into the library; every other buffer is the caller's.
+// for callers that must not allocate device memory. Up to kCoverSeeds seeds are held in shared memory
+// (coverage.cuh); beyond that its only scratch is a fixed array of seed flags compiled into the library.
+// Every other buffer is the caller's.
 #include <cuda_runtime.h>
 
 #include <mutex>
 #include <string>
 
+#include "coverage.cuh"
 #include "internal.h"
 
 namespace hyperim {
 namespace {
+
+__global__ void __launch_bounds__(kCoverThreads)
+k_na_cover_sets(const int64_t* __restrict__ rr_off, const int32_t* __restrict__ rr_mem,
+                const uint8_t* __restrict__ rr_stratum, int64_t count, int32_t n, const int32_t* __restrict__ seeds,
+                int32_t k, int per, unsigned long long* __restrict__ lam) {
+    extern __shared__ uint32_t cover_slots[];
+    cover_sets(cover_slots, rr_off, rr_mem, rr_stratum, count, n, seeds, k, per, lam, [](int64_t) { return false; });
+}
 
 // One flag per vertex id. Every GPU that loads the library holds these bytes until the process
 // exits. All calls share them, so calls that overlap on the GPU race (see the header).
@@ -103,6 +113,20 @@ extern "C" hyperim_status hyperim_coverage_noalloc(int32_t n, const int64_t* rr_
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
     if (sm < 1) sm = 1;
+    if (k <= kCoverSeeds) {
+        cudaError_t e = cudaMemsetAsync(lambda_s, 0, sizeof(unsigned long long) * HYPERIM_NSTRATA, s);
+        if (e == cudaSuccess && count > 0) {
+            const int per = cover_per(count, sm);
+            const int64_t warps = (count + per - 1) / per;
+            const int64_t want = (warps * 32 + kCoverThreads - 1) / kCoverThreads;
+            k_na_cover_sets<<<(int)(want < (int64_t)sm * 8 ? want : (int64_t)sm * 8), kCoverThreads, cover_smem(k), s>>>(
+                rr_off, rr_mem, rr_stratum, count, n, seeds, k, per, lambda_s);
+            count_launch();
+            e = cudaGetLastError();
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "coverage kernels");
+        return HYPERIM_OK;
+    }
     const int64_t words = ((int64_t)n + 15) / 16;
     const int gclear = (int)((words + 255) / 256 < sm * 8 ? (words + 255) / 256 : sm * 8);
     { k_na_clear<<<gclear > 0 ? gclear : 1, 256, 0, s>>>(flags, n, lambda_s); count_launch(); }
