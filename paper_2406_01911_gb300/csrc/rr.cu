@@ -386,7 +386,8 @@ struct WarpSink {
 // itself done, so the head and tail read afterwards include them, and a warp leaves only when
 // the queue is quiescent (a warp that left early would idle at the barrier for the rest of the
 // set). The wait is bounded (kErrSpin).
-__device__ int claim_slot(const RRParams& P, Shared& S, int64_t job) {
+template <class SM>
+__device__ int claim_slot(const RRParams& P, SM& S, int64_t job) {
     volatile int* ctrl = S.ctrl;
     for (int it = 0; it < P.spin_limit; ++it) {
         const int d = ctrl[C_DONE];
@@ -1381,6 +1382,8 @@ struct FwdParams {
     uint64_t nsims;
     uint32_t key0, key1;
     uint32_t* counts;
+    const int32_t* deg;   // one threshold per receiver (k_forward_flat): p = 1/deg(v), or, when null,
+    uint64_t thr;         // the same threshold for every pair
 };
 
 __device__ __forceinline__ bool fwd_live(const RRParams& P, uint32_t key0, uint32_t key1, uint32_t r,
@@ -1510,6 +1513,87 @@ __global__ void __launch_bounds__(kThreads, 1) k_forward(FwdParams F) {
             if (lane == 0) u = slot_value(P, list, idx, (int64_t)r);
             u = __shfl_sync(0xFFFFFFFFu, u, 0);
             if (u >= 0) fwd_pop_warp(F, S, vis, list, r, u);
+            __syncwarp();
+            if (lane == 0) {
+                __threadfence_block();  // this pop's pushes before its completion
+                atomicAdd(&S.ctrl[C_DONE], 1);
+            }
+        }
+        __syncthreads();
+        const int size = S.ctrl[C_TAIL];
+        if (threadIdx.x == 0) F.counts[r] = (uint32_t)size;
+        for (int i = threadIdx.x; i < size; i += kThreads) {
+            const int32_t v = __ldcg(list + i);
+            if (v >= 0) vis[v >> 5] = 0;
+            list[i] = -1;
+        }
+        __syncthreads();
+    }
+}
+
+// Forward cascade when the probability of u -> v does not depend on w(u, v) (one p for every pair,
+// or weighted cascade: 1/deg(v)): the coin is keyed by (r, u, v), so a neighbour met in several
+// shared hyperedges flips the same coin each time, and neither the multiplicities nor the sort that
+// finds them are needed. An activated u streams the members of its hyperedges; a member that is
+// active already is passed over before its coin (in a large cascade most are). Without sort buffers
+// several blocks fit on an SM. 256 simulations of 50 seeds on 100k vertices, p = 0.01: 100 ms with the sort and
+// the layer search of k_forward, 15.4 ms so.
+struct FlatShared {
+    int ctrl[16];
+    unsigned long long out_pos;
+    int wpre[kWarps][2 * 32 + 1];
+};
+
+__global__ void __launch_bounds__(kThreads, 2) k_forward_flat(FwdParams F) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const RRParams& P = F.P;
+    FlatShared& S = *reinterpret_cast<FlatShared*>(smem_raw);
+    uint32_t* vis = P.vis_smem ? reinterpret_cast<uint32_t*>(smem_raw + sizeof(FlatShared))
+                               : P.gvis + (int64_t)blockIdx.x * P.vis_words;
+    int32_t* list = P.list + (int64_t)blockIdx.x * P.list_cap;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const QueueSink sink{vis, list, &S.ctrl[C_TAIL]};
+    for (int64_t w = threadIdx.x; w < P.vis_words; w += kThreads) vis[w] = 0;
+    __syncthreads();
+    for (;;) {
+        if (threadIdx.x == 0) {
+            S.out_pos = atomicAdd(reinterpret_cast<unsigned long long*>(P.next_job), 1ull);
+            S.ctrl[C_HEAD] = 0;
+            S.ctrl[C_TAIL] = 0;
+            S.ctrl[C_DONE] = 0;
+            S.ctrl[C_NDEF] = 0;
+        }
+        __syncthreads();
+        if (S.out_pos >= F.nsims) break;
+        const uint32_t r = (uint32_t)S.out_pos;
+        for (int i = threadIdx.x; i < F.k; i += kThreads) sink.push((uint32_t)F.seeds[i]);
+        __syncthreads();
+        for (;;) {
+            int idx = 0;
+            if (lane == 0) idx = claim_slot(P, S, (int64_t)r);
+            idx = __shfl_sync(0xFFFFFFFFu, idx, 0);
+            if (idx < 0) break;
+            int32_t u = 0;
+            if (lane == 0) u = slot_value(P, list, idx, (int64_t)r);
+            u = __shfl_sync(0xFFFFFFFFu, u, 0);
+            if (u >= 0) {
+                const int4 vi = P.vinfo[u];
+                for_each_member<32>(P.v_span, P.he_mem, u, vi.z, vi.w, S.wpre[wid], [&](uint32_t v) {
+                    const uint32_t word = P.vis_smem ? *(volatile uint32_t*)(vis + (v >> 5)) : __ldcg(vis + (v >> 5));
+                    if (word >> (v & 31) & 1u) return;
+                    uint64_t thr = F.thr;
+                    if (F.deg) {
+                        const uint32_t d = (uint32_t)F.deg[v];
+                        const uint32_t q = 0xFFFFFFFFu / max(d, 1u);  // floor(2^32 / d) in 32 bits
+                        thr = d <= 1 ? kPOne : (uint64_t)(q + (0xFFFFFFFFu - q * d == d - 1 ? 1u : 0u));
+                    }
+                    if (thr < kPOne) {
+                        if (thr == 0) return;
+                        if (philox10(make_uint4(r, (uint32_t)u, v, 0xFFFFFFFEu), F.key0, F.key1).x >= thr) return;
+                    }
+                    sink.push(v);
+                });
+            }
             __syncwarp();
             if (lane == 0) {
                 __threadfence_block();  // this pop's pushes before its completion
@@ -2082,6 +2166,9 @@ hyperim_status allow_rr_smem() {
         const int most = (int)std::min<size_t>(sizeof(Shared) + kVisSmemBits / 8, smem_optin());
         err = cudaFuncSetAttribute(k_rr, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (err == cudaSuccess) err = cudaFuncSetAttribute(k_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (err == cudaSuccess)
+            err = cudaFuncSetAttribute(k_forward_flat, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(sizeof(FlatShared) + kVisSmemBits / 8));
         if (err == cudaSuccess)
             err = cudaFuncSetAttribute(k_rr_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WarpShared));
         if (err == cudaSuccess) {
@@ -2871,20 +2958,29 @@ hyperim_status forward_spread(hyperim_graph* g, const int32_t* seeds_host, int32
     cudaStream_t s = g->stream;
     hyperim_status st;
     if ((st = allow_rr_smem())) return st;
+    // one threshold per receiver: no multiplicities, no sort
+    const bool flat = g->model != HYPERIM_P_PAPER_LAYER;
+    const void* kernel = flat ? (const void*)k_forward_flat : (const void*)k_forward;
+    const size_t base_smem = flat ? sizeof(FlatShared) : sizeof(Shared);
     bool vis_smem = (int64_t)g->n <= kVisSmemBits &&
-                    sizeof(Shared) + sizeof(uint32_t) * (((size_t)g->n + 31) / 32) <= smem_optin();
+                    base_smem + sizeof(uint32_t) * (((size_t)g->n + 31) / 32) <= smem_optin();
     size_t smem = 0;
     int per_sm = 0;
     for (;;) {
         const size_t vis_bytes = vis_smem ? sizeof(uint32_t) * (((size_t)g->n + 31) / 32) : 0;
-        smem = sizeof(Shared) + vis_bytes;
-        HYP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forward, kThreads, smem));
+        smem = base_smem + vis_bytes;
+        HYP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem));
         if (per_sm >= 1 || !vis_smem) break;
         vis_smem = false;
     }
     if (per_sm < 1) return set_error(HYPERIM_ECUDA, "forward kernel does not fit on an SM");
     int blocks = g->sm_count * per_sm;
     if ((uint64_t)blocks > nsims) blocks = (int)nsims;
+    // more than one block per SM takes more queues than RR generation keeps: at most 1 GiB of them, and
+    // none under a budget
+    if (blocks > g->sm_count &&
+        (graph_root(g)->budget || (size_t)(blocks - g->sm_count) * (size_t)g->n * sizeof(int32_t) > ((size_t)1 << 30)))
+        blocks = g->sm_count;
     if ((st = ensure_scratch(g, blocks, vis_smem))) return st;
     int32_t* d_seeds = nullptr;
     uint32_t* d_counts = nullptr;
@@ -2923,7 +3019,11 @@ hyperim_status forward_spread(hyperim_graph* g, const int32_t* seeds_host, int32
     F.key0 = (uint32_t)seed;
     F.key1 = (uint32_t)(seed >> 32);
     F.counts = d_counts;
-    { k_forward<<<blocks, kThreads, smem, s>>>(F); count_launch(); }
+    F.deg = g->model == HYPERIM_P_WC ? g->deg : nullptr;
+    F.thr = g->uniform_thr;
+    if (flat) k_forward_flat<<<blocks, kThreads, smem, s>>>(F);
+    else k_forward<<<blocks, kThreads, smem, s>>>(F);
+    count_launch();
     HYP_CUDA(cudaGetLastError());
     if ((st = check_device_status(g, "forward spread"))) {
         cudaMemsetAsync(g->scratch.list, 0xFF, sizeof(int32_t) * g->scratch.list_cap * g->scratch.blocks, s);
