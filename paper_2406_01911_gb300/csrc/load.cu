@@ -38,59 +38,126 @@ __global__ void k_check_offsets(const int32_t* off, int32_t m, DevStatus* st) {
     if (blockIdx.x == 0 && threadIdx.x == 0 && off[0] != 0) dev_fail(st, kErrBadOffsets, 0);
 }
 
-// ---- normalisation: sort each hyperedge's members, drop repeats (a hyperedge is a set) -------
-// One warp per hyperedge. A member is kept at its first occurrence only; its position in the
-// sorted set is the number of distinct values below it.
-__global__ void k_normalise(const int32_t* __restrict__ off, const int32_t* __restrict__ mem,
-                            int32_t m, int32_t n, int32_t* __restrict__ out,
-                            uint8_t* __restrict__ first, uint32_t* __restrict__ newsize,
-                            DevStatus* st) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t e = warp; e < m; e += nwarps) {
-        const int32_t b = off[e], len = off[e + 1] - b;
-        if (len <= 32) {
-            const int32_t x = lane < len ? mem[b + lane] : INT32_MAX;
-            if (lane < len && (x < 0 || x >= n)) dev_fail(st, kErrBadMember, (int32_t)e);
-            bool dup = false;
-            for (int j = 0; j < len; ++j) {
-                const int32_t y = __shfl_sync(0xFFFFFFFFu, x, j);
-                if (y == x && j < lane) dup = true;
-            }
-            int below = 0;
-            for (int j = 0; j < len; ++j) {
-                const int32_t y = __shfl_sync(0xFFFFFFFFu, x, j);
-                const int ydup = __shfl_sync(0xFFFFFFFFu, dup ? 1 : 0, j);
-                if (!ydup && y < x) ++below;
-            }
-            const bool keep = lane < len && !dup;
-            const uint32_t kb = __ballot_sync(0xFFFFFFFFu, keep);
-            if (keep) out[b + below] = x;
-            if (lane == 0) newsize[e] = __popc(kb);
-        } else {
-            // first-occurrence flags, then positions among first occurrences
-            for (int i = lane; i < len; i += 32) {
-                const int32_t x = mem[b + i];
-                if (x < 0 || x >= n) dev_fail(st, kErrBadMember, (int32_t)e);
-                bool dup = false;
-                for (int j = 0; j < i && !dup; ++j) dup = mem[b + j] == x;
-                first[b + i] = dup ? 0 : 1;
-            }
-            __syncwarp();
-            int keep = 0;
-            for (int i = lane; i < len; i += 32) {
-                if (!first[b + i]) continue;
-                const int32_t x = mem[b + i];
-                int below = 0;
-                for (int j = 0; j < len; ++j) below += (first[b + j] && mem[b + j] < x) ? 1 : 0;
-                out[b + below] = x;
-                ++keep;
-            }
-            for (int o = 16; o > 0; o >>= 1) keep += __shfl_xor_sync(0xFFFFFFFFu, keep, o);
-            if (lane == 0) newsize[e] = keep;
-        }
+// ---- short lists sorted on chip -------------------------------------------------------------------
+// Lists (hyperedges, or the hyperedges of a vertex) sorted ascending, one warp per list: up to 32
+// entries across the lanes, up to kListWarp in the warp's part of shared memory, up to kListBlock by
+// the whole block after its warps are done; longer ones by counting smaller entries, n^2 reads. (Every
+// list above 32 took the n^2 way before: 155 us on a graph of 14,142 vertices, 3.3 + 2.7 ms on 2M.)
+constexpr int kListThreads = 256;
+constexpr int kListWarps = kListThreads / 32;
+constexpr int kListWarp = 1024;
+constexpr int kListBlock = kListWarp * kListWarps;
+
+// in[0, len) sorted, repeated values dropped, to out; returns how many. buf: the next power of two.
+template <int G>
+__device__ int sort_unique(const int32_t* __restrict__ in, int len, uint32_t* buf, int32_t* __restrict__ out, int* tmp) {
+    using Gr = Group<G>;
+    for (int i = Gr::rank(); i < len; i += G) buf[i] = (uint32_t)in[i];
+    Gr::sync();
+    group_sort<G>(buf, len);
+    int kept = 0;
+    for (int base = 0; base < len; base += G) {
+        const int p = base + Gr::rank();
+        const bool keep = p < len && (p == 0 || buf[p - 1] != buf[p]);
+        int total;
+        const int at = Gr::excl_count(keep, tmp, &total);
+        if (keep) out[kept + at] = (int32_t)buf[p];
+        kept += total;
     }
+    Gr::sync();
+    return kept;
+}
+
+// the same for a list that fits nowhere on chip (first: one flag byte per entry)
+__device__ int count_unique(const int32_t* __restrict__ in, int64_t len, int32_t* __restrict__ out,
+                            uint8_t* __restrict__ first, int* tmp) {
+    for (int64_t i = threadIdx.x; i < len; i += kListThreads) {
+        const int32_t x = in[i];
+        bool dup = false;
+        for (int64_t j = 0; j < i && !dup; ++j) dup = in[j] == x;
+        first[i] = dup ? 0 : 1;
+    }
+    if (threadIdx.x == 0) tmp[0] = 0;
+    __syncthreads();
+    int mine = 0;
+    for (int64_t i = threadIdx.x; i < len; i += kListThreads) {
+        if (!first[i]) continue;
+        const int32_t x = in[i];
+        int64_t below = 0;
+        for (int64_t j = 0; j < len; ++j) below += (first[j] && in[j] < x) ? 1 : 0;
+        out[below] = x;
+        ++mine;
+    }
+    atomicAdd(&tmp[0], mine);
+    __syncthreads();
+    const int kept = tmp[0];
+    __syncthreads();
+    return kept;
+}
+
+// list i of `lists` is in[off[i], off[i + 1]), its sorted set goes to out at the same place;
+// done(i, kept) is called by one thread, check(i, x) for every entry
+template <typename Off, typename Check, typename Done>
+__device__ __forceinline__ void sort_lists(const Off* __restrict__ off, int32_t lists, const int32_t* __restrict__ in,
+                                           int32_t* __restrict__ out, uint8_t* __restrict__ first, Check&& check,
+                                           Done&& done) {
+    __shared__ uint32_t buf[kListBlock];
+    __shared__ int tmp[kListWarps + 1];
+    __shared__ int nlong;
+    __shared__ int32_t long_s[kListWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int64_t i0 = (int64_t)blockIdx.x * kListWarps; i0 < lists; i0 += (int64_t)gridDim.x * kListWarps) {
+        if (threadIdx.x == 0) nlong = 0;
+        __syncthreads();
+        const int64_t i = i0 + wid;
+        if (i < lists) {
+            const int64_t b = (int64_t)off[i], len = (int64_t)off[i + 1] - b;
+            if (len <= 32) {
+                const int32_t x = lane < len ? in[b + lane] : INT32_MAX;
+                if (lane < len) check(i, x);
+                bool dup = false;
+                int below = 0;
+                for (int j = 0; j < (int)len; ++j) {
+                    const int32_t y = __shfl_sync(0xFFFFFFFFu, x, j);
+                    const bool rep = __ballot_sync(0xFFFFFFFFu, lane < j && x == y) != 0;  // y came before
+                    dup = dup || (rep && lane == j);
+                    below += !rep && y < x ? 1 : 0;
+                }
+                const bool keep = lane < len && !dup;
+                const uint32_t kb = __ballot_sync(0xFFFFFFFFu, keep);
+                if (keep) out[b + below] = x;
+                if (lane == 0) done(i, __popc(kb));
+            } else if (len <= kListWarp) {
+                for (int64_t x = lane; x < len; x += 32) check(i, in[b + x]);
+                const int kept = sort_unique<32>(in + b, (int)len, buf + wid * kListWarp, out + b, nullptr);
+                if (lane == 0) done(i, kept);
+            } else if (lane == 0) {
+                long_s[atomicAdd(&nlong, 1)] = (int32_t)i;
+            }
+        }
+        __syncthreads();
+        const int todo = nlong;
+        for (int q = 0; q < todo; ++q) {
+            const int32_t l = long_s[q];
+            const int64_t b = (int64_t)off[l], len = (int64_t)off[l + 1] - b;
+            for (int64_t x = threadIdx.x; x < len; x += kListThreads) check(l, in[b + x]);
+            const int kept = len <= kListBlock ? sort_unique<kListThreads>(in + b, (int)len, buf, out + b, tmp)
+                                               : count_unique(in + b, len, out + b, first + b, tmp);
+            if (threadIdx.x == 0) done(l, kept);
+        }
+        __syncthreads();
+    }
+}
+
+// ---- normalisation: sort each hyperedge's members, drop repeats (a hyperedge is a set) -------
+__global__ void __launch_bounds__(kListThreads)
+k_normalise(const int32_t* __restrict__ off, const int32_t* __restrict__ mem, int32_t m, int32_t n,
+            int32_t* __restrict__ out, uint8_t* __restrict__ first, uint32_t* __restrict__ newsize, DevStatus* st) {
+    sort_lists(off, m, mem, out, first,
+               [&](int64_t e, int32_t x) {
+                   if (x < 0 || x >= n) dev_fail(st, kErrBadMember, (int32_t)e);
+               },
+               [&](int64_t e, int kept) { newsize[e] = (uint32_t)kept; });
 }
 
 __global__ void k_compact_he(const int32_t* __restrict__ off_in, const int32_t* __restrict__ tmp,
@@ -132,24 +199,16 @@ __global__ void k_scatter_vhe(const int32_t* __restrict__ he_off, const int32_t*
     }
 }
 
-// sort each vertex's hyperedge list (distinct ids): position = number of smaller ids
-__global__ void k_sort_vhe(const int64_t* __restrict__ v_off64, int32_t n,
-                           const int32_t* __restrict__ in, int32_t* __restrict__ out,
-                           int32_t* __restrict__ v_off32) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t v = warp; v < n; v += nwarps) {
-        const int64_t b = v_off64[v], len = v_off64[v + 1] - b;
-        for (int64_t i = lane; i < len; i += 32) {
-            const int32_t x = in[b + i];
-            int below = 0;
-            for (int64_t j = 0; j < len; ++j) below += in[b + j] < x ? 1 : 0;
-            out[b + below] = x;
-        }
-        if (lane == 0) v_off32[v] = (int32_t)b;
-        if (lane == 0 && v == n - 1) v_off32[n] = (int32_t)v_off64[n];
-    }
+// sort each vertex's hyperedge list (distinct ids); first: nnz flag bytes, only for lists longer than
+// kListBlock
+__global__ void __launch_bounds__(kListThreads)
+k_sort_vhe(const int64_t* __restrict__ v_off64, int32_t n, const int32_t* __restrict__ in, int32_t* __restrict__ out,
+           uint8_t* __restrict__ first, int32_t* __restrict__ v_off32) {
+    sort_lists(v_off64, n, in, out, first, [](int64_t, int32_t) {},
+               [&](int64_t v, int) {
+                   v_off32[v] = (int32_t)v_off64[v];
+                   if (v == n - 1) v_off32[n] = (int32_t)v_off64[n];
+               });
 }
 
 // ---- layer profile: pass 1 ----------------------------------------------------------------------
@@ -446,14 +505,13 @@ k_profile(Incidence I, const int2* __restrict__ v_span, const int32_t* __restric
 // ---- layer profile: pass 2 (thresholds, inversion kind, CDF table lengths) ------------------
 // Entry [0] = {w_i | p = 1 flag, n_i, floor(p 2^32), T_0}; entry [1] = {table offset, table
 // length | kind << 16, Poisson parts c, n_1 + .. + n_{i-1}}; kind 0: no draw (p = 0 or 1), 1:
-// Binomial (n_i <= 20), 2: Poisson with c parts of lambda / c each (Sec. 3.1.3). The table and T_0
-// are filled by pass 3.
-__global__ void k_profile_write(int32_t n, const int32_t* __restrict__ v_off,
-                                const uint2* __restrict__ pairs, const int64_t* __restrict__ poff64,
-                                const uint32_t* __restrict__ deg, int32_t model, uint64_t uthr,
-                                const double* __restrict__ ln_l1, uint4* __restrict__ prof,
-                                uint32_t* __restrict__ tab_len, int32_t* __restrict__ prof_off,
-                                uint8_t* __restrict__ stratum) {
+// Binomial (n_i <= 20), 2: Poisson with c parts of lambda / c each (Sec. 3.1.3). One thread per
+// vertex lays the layers down ({w_i, n_i, owner, i}), then one thread per layer does the double
+// arithmetic of its thresholds (a thread per vertex ran its layers one after the other: 155 us on 14,142 vertices, 4.0 ms on 2M);
+// the table and T_0 are filled by pass 3.
+__global__ void k_profile_layers(int32_t n, const int32_t* __restrict__ v_off, const uint2* __restrict__ pairs,
+                                 const int64_t* __restrict__ poff64, uint4* __restrict__ prof,
+                                 int32_t* __restrict__ prof_off, uint8_t* __restrict__ stratum) {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t pb = poff64[v];
@@ -461,42 +519,54 @@ __global__ void k_profile_write(int32_t n, const int32_t* __restrict__ v_off,
         prof_off[v] = (int32_t)pb;
         if (v == n - 1) prof_off[n] = (int32_t)poff64[n];
         stratum[v] = (uint8_t)(l < HYPERIM_NSTRATA - 1 ? l : HYPERIM_NSTRATA - 1);
-        const uint32_t dg = deg[v];
+        const uint2* wn = pairs + v_off[v];
         uint32_t before = 0;
         for (int i = 0; i < l; ++i) {
-            const uint2 wn = pairs[v_off[v] + i];
-            const uint32_t n_i = wn.y;
-            uint64_t thr;
-            if (model == HYPERIM_P_UNIFORM_PAIR) {
-                thr = uthr;
-            } else if (model == HYPERIM_P_WC) {
-                thr = dg <= 1 ? kPOne : (kPOne / (uint64_t)dg);
-            } else {
-                // P(L_i) = 1/(i ln(l+1)) (Sec. 3.1.1); per member P(L_i)/n_i, clamped to 1
-                const double PL = __ddiv_rn(1.0, __dmul_rn((double)(i + 1), ln_l1[l]));
-                const double pd = __ddiv_rn(PL, (double)n_i);
-                thr = pd >= 1.0 ? kPOne : __double2ull_rz(__dmul_rn(pd, 4294967296.0));
-            }
-            uint32_t flags = 0, kind = 0, c = 0, L = 0;
-            if (thr >= kPOne) {
-                flags = kPOneFlag;
-            } else if (thr > 0) {
-                if (n_i <= 20) {
-                    kind = 1;
-                    c = 1;
-                    L = cdf_table(n_i, thr, false, 0.0, kTableCap, nullptr);
-                } else {
-                    kind = 2;
-                    const double lam = poisson_lambda(n_i, thr);
-                    c = poisson_parts(lam);
-                    L = cdf_table(n_i, thr, true, poisson_part_lambda(lam, c), kTableCap, nullptr);
-                }
-            }
-            prof[2 * (pb + i)] = make_uint4(wn.x | flags, n_i, thr >= kPOne ? 0u : (uint32_t)thr, 0u);
-            prof[2 * (pb + i) + 1] = make_uint4(0u, L | (kind << 16), c, before);
-            tab_len[pb + i] = L;
-            before += n_i;
+            const uint2 p = wn[i];
+            prof[2 * (pb + i)] = make_uint4(p.x, p.y, (uint32_t)v, (uint32_t)i);
+            prof[2 * (pb + i) + 1] = make_uint4(0u, (uint32_t)l, 0u, before);
+            before += p.y;
         }
+    }
+}
+
+__global__ void k_profile_write(int64_t layers, const uint32_t* __restrict__ deg, int32_t model, uint64_t uthr,
+                                const double* __restrict__ ln_l1, uint4* __restrict__ prof,
+                                uint32_t* __restrict__ tab_len) {
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < layers;
+         x += (int64_t)gridDim.x * blockDim.x) {
+        const uint4 a = prof[2 * x], b = prof[2 * x + 1];
+        const uint32_t n_i = a.y;
+        uint64_t thr;
+        if (model == HYPERIM_P_UNIFORM_PAIR) {
+            thr = uthr;
+        } else if (model == HYPERIM_P_WC) {
+            const uint32_t dg = deg[a.z];
+            thr = dg <= 1 ? kPOne : (kPOne / (uint64_t)dg);
+        } else {
+            // P(L_i) = 1/(i ln(l+1)) (Sec. 3.1.1); per member P(L_i)/n_i, clamped to 1
+            const double PL = __ddiv_rn(1.0, __dmul_rn((double)(a.w + 1), ln_l1[b.y]));
+            const double pd = __ddiv_rn(PL, (double)n_i);
+            thr = pd >= 1.0 ? kPOne : __double2ull_rz(__dmul_rn(pd, 4294967296.0));
+        }
+        uint32_t flags = 0, kind = 0, c = 0, L = 0;
+        if (thr >= kPOne) {
+            flags = kPOneFlag;
+        } else if (thr > 0) {
+            if (n_i <= 20) {
+                kind = 1;
+                c = 1;
+                L = cdf_table(n_i, thr, false, 0.0, kTableCap, nullptr);
+            } else {
+                kind = 2;
+                const double lam = poisson_lambda(n_i, thr);
+                c = poisson_parts(lam);
+                L = cdf_table(n_i, thr, true, poisson_part_lambda(lam, c), kTableCap, nullptr);
+            }
+        }
+        prof[2 * x] = make_uint4(a.x | flags, n_i, thr >= kPOne ? 0u : (uint32_t)thr, 0u);
+        prof[2 * x + 1] = make_uint4(0u, L | (kind << 16), c, b.w);
+        tab_len[x] = L;
     }
 }
 
@@ -521,27 +591,70 @@ __global__ void k_table_fill(int64_t layers, const int64_t* __restrict__ tab_off
     }
 }
 
-__global__ void k_stratum_flags(const uint8_t* __restrict__ stratum, int32_t n, int s,
-                                uint32_t* __restrict__ flags) {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x)
-        flags[v] = stratum[v] == s ? 1u : 0u;
+// Strata lists, all sixteen at once: a warp owns kStratumRun consecutive vertices, counts them by
+// stratum, and after one scan of the counts (stratum-major, so a run's place in its list is the scanned
+// count itself) writes them to their places in id order. (Stratum by stratum this took 16 x 5 launches.)
+constexpr int kStratumRun = 512;
+
+__global__ void k_stratum_count(const uint8_t* __restrict__ stratum, int32_t n, int64_t runs,
+                                uint32_t* __restrict__ count) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; q < runs;
+         q += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        uint32_t mine = 0;  // lane s counts stratum s
+        for (int i = 0; i < kStratumRun; i += 32) {
+            const int64_t v = q * kStratumRun + i + lane;
+            const int s = v < n ? stratum[v] : -1;
+            const uint32_t same = __match_any_sync(0xFFFFFFFFu, s);
+            for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, s >= 0); todo;) {
+                const int src = __ffs(todo) - 1;
+                const uint32_t grp = __shfl_sync(0xFFFFFFFFu, same, src);
+                if (lane == __shfl_sync(0xFFFFFFFFu, s, src)) mine += __popc(grp);
+                todo &= ~grp;
+            }
+        }
+        if (lane < HYPERIM_NSTRATA) count[lane * runs + q] = mine;
+    }
 }
 
-__global__ void k_stratum_scatter(const uint32_t* __restrict__ flags, const int64_t* __restrict__ pos,
-                                  int32_t n, int32_t base, int32_t* __restrict__ vs_list) {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x)
-        if (flags[v]) vs_list[base + pos[v]] = (int32_t)v;
+__global__ void k_stratum_scatter(const uint8_t* __restrict__ stratum, int32_t n, int64_t runs,
+                                  const int64_t* __restrict__ pos, int32_t* __restrict__ vs_list) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; q < runs;
+         q += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        int32_t at = lane < HYPERIM_NSTRATA ? (int32_t)pos[lane * runs + q] : 0;
+        for (int i = 0; i < kStratumRun; i += 32) {
+            const int64_t v = q * kStratumRun + i + lane;
+            const int s = v < n ? stratum[v] : -1;
+            const uint32_t same = __match_any_sync(0xFFFFFFFFu, s);
+            const int32_t base = __shfl_sync(0xFFFFFFFFu, at, s < 0 ? 0 : s);
+            if (s >= 0) vs_list[base + __popc(same & lanemask_lt())] = (int32_t)v;
+            for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, s >= 0); todo;) {
+                const int src = __ffs(todo) - 1;
+                const uint32_t grp = __shfl_sync(0xFFFFFFFFu, same, src);
+                if (lane == __shfl_sync(0xFFFFFFFFu, s, src)) at += __popc(grp);
+                todo &= ~grp;
+            }
+        }
+    }
 }
 
+// histogram of l: the low bins (nearly every vertex) per block on chip
+constexpr int kLayerBins = 256;
 __global__ void k_hist_layers(const int64_t* __restrict__ poff64, int32_t n,
                               unsigned long long* __restrict__ hist, int hmax) {
+    __shared__ unsigned int h[kLayerBins];
+    for (int i = threadIdx.x; i < kLayerBins; i += blockDim.x) h[i] = 0;
+    __syncthreads();
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t l = poff64[v + 1] - poff64[v];
-        atomicAdd(&hist[l < hmax ? l : hmax], 1ull);
+        const int64_t l = min(poff64[v + 1] - poff64[v], (int64_t)hmax);
+        if (l < kLayerBins) atomicAdd(&h[l], 1u);
+        else atomicAdd(&hist[l], 1ull);
     }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kLayerBins && i <= hmax; i += blockDim.x)
+        if (h[i]) atomicAdd(&hist[i], (unsigned long long)h[i]);
 }
 
 // out[0] = max, out[1] = sum (both zeroed by the caller)
@@ -707,9 +820,8 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
     uint8_t* d_first = nullptr;
     if ((st = tmp.alloc(&d_first, nnz_alloc))) return st;
     if (m > 0)
-        { k_normalise<<<grid_for((int64_t)m * 32, 256, sm), 256, 0, s>>>(d_off_in, d_mem_in, m, n,
-                                                                       d_tmp, d_first, d_newsize,
-                                                                       g->d_status); count_launch(); }
+        { k_normalise<<<grid_for((int64_t)m * 32, kListThreads, sm), kListThreads, 0, s>>>(
+            d_off_in, d_mem_in, m, n, d_tmp, d_first, d_newsize, g->d_status); count_launch(); }
     if ((st = check_device_status(g, "hyperedge members"))) return st;
     if ((st = exclusive_scan_u32_to_i64(g, d_newsize, d_off_new, m))) return st;
     int64_t nnz = 0;
@@ -741,8 +853,8 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
     if (m > 0)
         { k_scatter_vhe<<<grid_for((int64_t)m * 32, 256, sm), 256, 0, s>>>(
             g->he_off, g->he_mem, m, d_voff64, d_cnt, d_tmp, g->tsum); count_launch(); }
-    { k_sort_vhe<<<grid_for((int64_t)n * 32, 256, sm), 256, 0, s>>>(d_voff64, n, d_tmp, g->v_he,
-                                                                   g->v_off); count_launch(); }
+    { k_sort_vhe<<<grid_for((int64_t)n * 32, kListThreads, sm), kListThreads, 0, s>>>(
+        d_voff64, n, d_tmp, g->v_he, d_first, g->v_off); count_launch(); }
 
     // --- maxima of d_H and T
     unsigned long long* d_max = nullptr;
@@ -861,9 +973,11 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
     const size_t Lalloc = (size_t)(L > 0 ? L : 1);
     if ((st = tmp.alloc(&d_tlen, sizeof(uint32_t) * Lalloc))) return st;
     if ((st = tmp.alloc(&d_toff, sizeof(int64_t) * (Lalloc + 1)))) return st;
-    { k_profile_write<<<grid_for(n, 256, sm), 256, 0, s>>>(n, g->v_off, d_pairs, d_poff64, d_deg,
-                                                         g->model, g->uniform_thr, d_ln, g->prof,
-                                                         d_tlen, g->prof_off, g->stratum); count_launch(); }
+    { k_profile_layers<<<grid_for(n, 256, sm), 256, 0, s>>>(n, g->v_off, d_pairs, d_poff64, g->prof, g->prof_off,
+                                                          g->stratum); count_launch(); }
+    if (L > 0)
+        { k_profile_write<<<grid_for(L, 256, sm), 256, 0, s>>>(L, d_deg, g->model, g->uniform_thr, d_ln, g->prof,
+                                                             d_tlen); count_launch(); }
     if ((st = exclusive_scan_u32_to_i64(g, d_tlen, d_toff, L))) return st;
     int64_t tab_total = 0;
     HYP_CUDA(cudaMemcpyAsync(&tab_total, d_toff + L, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
@@ -933,13 +1047,16 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
     hvs[0] = 0;
     for (int s2 = 0; s2 < HYPERIM_NSTRATA; ++s2) hvs[s2 + 1] = hvs[s2] + (int32_t)g->stratum_size[s2];
     HYP_CUDA(cudaMemcpyAsync(g->vs_off, hvs, sizeof(hvs), cudaMemcpyHostToDevice, s));
-    uint32_t* d_flags = d_cnt;
-    for (int s2 = 0; s2 < HYPERIM_NSTRATA; ++s2) {
-        if (g->stratum_size[s2] == 0) continue;
-        { k_stratum_flags<<<grid_for(n, 256, sm), 256, 0, s>>>(g->stratum, n, s2, d_flags); count_launch(); }
-        if ((st = exclusive_scan_u32_to_i64(g, d_flags, d_voff64, n))) return st;
-        { k_stratum_scatter<<<grid_for(n, 256, sm), 256, 0, s>>>(d_flags, d_voff64, n, hvs[s2],
-                                                               g->vs_list); count_launch(); }
+    {
+        const int64_t runs = ((int64_t)n + kStratumRun - 1) / kStratumRun;
+        uint32_t* d_scnt = nullptr;
+        int64_t* d_spos = nullptr;
+        if ((st = tmp.alloc(&d_scnt, sizeof(uint32_t) * HYPERIM_NSTRATA * (size_t)runs))) return st;
+        if ((st = tmp.alloc(&d_spos, sizeof(int64_t) * (HYPERIM_NSTRATA * (size_t)runs + 1)))) return st;
+        const int sgrid = grid_for(runs * 32, 128, sm);
+        { k_stratum_count<<<sgrid, 128, 0, s>>>(g->stratum, n, runs, d_scnt); count_launch(); }
+        if ((st = exclusive_scan_u32_to_i64(g, d_scnt, d_spos, HYPERIM_NSTRATA * runs))) return st;
+        { k_stratum_scatter<<<sgrid, 128, 0, s>>>(g->stratum, n, runs, d_spos, g->vs_list); count_launch(); }
     }
     HYP_CUDA(cudaGetLastError());
     if ((st = check_device_status(g, "profile write"))) return st;
