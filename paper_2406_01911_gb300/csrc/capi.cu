@@ -295,7 +295,7 @@ void free_handle(hyperim_graph* g, bool data) {
     free_memo(g);
     if (data) {
         void* ptrs[] = {g->he_off, g->he_mem, g->v_off, g->v_he, g->tsum, g->v_span, g->vinfo, g->prof_off,
-                        g->prof, g->cdf_tab, g->deg, g->stratum, g->vs_off, g->vs_list, g->idx, g->idx_tab,
+                        g->prof, g->cdf_tab, g->deg, g->stratum, g->vs_off, g->vs_list, g->idx, g->idx_tab, g->idx_sub,
                         g->mat_sect, g->he_dir, g->v_dir};
         for (void* p : ptrs)
             if (p) release(g, p);
@@ -374,6 +374,7 @@ hyperim_status hyperim_graph_share(hyperim_graph_t g, void* cuda_stream, hyperim
     h->vs_list = r->vs_list;
     h->idx = r->idx;
     h->idx_tab = r->idx_tab;
+    h->idx_sub = r->idx_sub;
     h->idx_entries = r->idx_entries;
     h->idx_vertices = r->idx_vertices;
     h->profile_entries = r->profile_entries;

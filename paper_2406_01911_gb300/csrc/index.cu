@@ -164,11 +164,17 @@ __global__ void k_idx_word(const int32_t* __restrict__ list, int32_t nlist, cons
 // bucketed by their top id bits (a bucket is 2^3 whole index chunks, so at most 8 x 1,024
 // members) through a global scratch area and sorted bucket by bucket -- are walked run by run:
 // each distinct neighbour (multiplicity w -> layer by search in the descending w list) adds one
-// to its (layer, chunk) count, kept on chip when the l x 2^c table fits, else in the table
-// itself. Every layer row then becomes an exclusive prefix along the chunks, one warp per row.
+// to its count of (layer, chunk, eighth of the chunk). The counts are 16-bit halves of on-chip
+// words, as many chunks at a time as fit kFillCells of them (all of a small vertex's chunks, one
+// bucket's eight of a large one's): no count ever goes to global memory. They then become the
+// entries of those chunks, lanes side by side along the chunks of a layer, with one running total per
+// layer carried on.
 constexpr int kFillThreads = 512;  // two blocks (32 warps) per SM: the sorts are latency-bound
 constexpr int kFillBuf = 8192;  // members sorted on chip at once (power of two)
-constexpr int kFillCnt = 4096;  // (layer, chunk) counts kept on chip (more: in the table itself)
+constexpr int kFillCnt = 4096;  // words of two counts each
+constexpr int kFillCells = 2 * kFillCnt;
+static_assert(kFillCells >= kIdxMaxL << kIdxSubBits, "one chunk of the most layers must fit");
+static_assert(2 * kFillThreads + 1 >= kIdxMaxL, "the prefix area holds the layers' running totals");
 constexpr int kFillBkt = kBins;
 constexpr int kFillTop = 1 << (kIdxMaxBits - 3);  // top-bit buckets: eight whole chunks each
 // the shared memory above fits three 512-thread blocks per SM
@@ -181,7 +187,7 @@ k_idx_fill(const int32_t* __restrict__ list, int32_t nlist, const uint8_t* __res
            const uint32_t* __restrict__ entries, const int64_t* __restrict__ off,
            const int4* __restrict__ vinfo, const int2* __restrict__ v_span,
            const int32_t* __restrict__ he_mem, const int32_t* __restrict__ tsum,
-           const uint4* __restrict__ prof, int id_bits, uint32_t* __restrict__ tab,
+           const uint4* __restrict__ prof, int id_bits, uint32_t* __restrict__ tab, uint4* __restrict__ sub,
            uint32_t* __restrict__ scratch, int64_t scratch_cap, const int32_t* __restrict__ order,
            int* __restrict__ next, DevStatus* st) {
     extern __shared__ __align__(16) unsigned char fill_smem[];
@@ -209,27 +215,80 @@ k_idx_fill(const int32_t* __restrict__ list, int32_t nlist, const uint8_t* __res
         const int C = 1 << c, shift = id_bits - c;
         const int T = tsum[mu] - vi.w;
         uint32_t* t = tab + off[i];
-        const int64_t cells = (int64_t)l * C;
-        uint32_t* cnt = cells <= kFillCnt ? cnt_s : t;
+        uint4* ts = sub ? sub + off[i] : nullptr;
+        uint32_t* carry = reinterpret_cast<uint32_t*>(pre);  // per layer (pre is free between gathers)
+        const int fb = idx_sub_bits(shift), fshift = shift - fb;
+        int gch = C;  // chunks counted at once
+        while (gch > 1 && ((int64_t)l * gch << kIdxSubBits) > kFillCells) gch >>= 1;
         for (int q = threadIdx.x; q < l; q += kFillThreads) lw[q] = prof[2 * ((int64_t)vi.x + q)].x & ~kPOneFlag;
-        for (int64_t k = threadIdx.x; k < cells; k += kFillThreads) cnt[k] = 0;
         __syncthreads();
-        auto count_run = [&](bool start, uint32_t x, int mult) -> bool {
-            if (start) {
-                int lo = 0, hi = l;  // lw descends: first q with lw[q] <= mult
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (lw[mid] > (uint32_t)mult) lo = mid + 1; else hi = mid;
+        // entries of the chunks [k0, k0 + nk) from the sorted keys[0, got), which hold all members of
+        // these chunks and perhaps others
+        auto count_and_emit = [&](const uint32_t* keys, int got, int k0, int nk) {
+            for (int kb = k0; kb < k0 + nk; kb += gch) {
+                const int g = min(gch, k0 + nk - kb);  // a power of two
+                const int words = (l * g) << (kIdxSubBits - 1);
+                for (int x = threadIdx.x; x < words; x += kFillThreads) cnt_s[x] = 0;
+                __syncthreads();
+                walk_runs<kFillThreads>(keys, got, [&](bool start, uint32_t x, int mult) -> bool {
+                    const int k = start ? (int)(x >> shift) - kb : -1;
+                    if (k >= 0 && k < g) {
+                        int lo = 0, hi = l;  // lw descends: first q with lw[q] <= mult
+                        while (lo < hi) {
+                            const int mid = (lo + hi) >> 1;
+                            if (lw[mid] > (uint32_t)mult) lo = mid + 1; else hi = mid;
+                        }
+                        if (lo < l && lw[lo] == (uint32_t)mult) {
+                            const int cell = ((lo * g + k) << kIdxSubBits) + (int)((x >> fshift) & ((1u << fb) - 1));
+                            atomicAdd(&cnt_s[cell >> 1], 1u << (16 * (cell & 1)));
+                        } else {
+                            dev_fail(st, kErrProfile, mu);
+                        }
+                    }
+                    return false;
+                });
+                __syncthreads();
+                const int gw = min(g, 32), rows = 32 / gw;  // layers side by side in a warp
+                for (int q0 = wid * rows; q0 < l; q0 += kWarps * rows) {
+                    const int q = q0 + lane / gw;
+                    uint32_t run = q < l ? carry[q] : 0u;
+                    for (int kk = lane % gw; kk < g; kk += 32) {  // gw < 32: one step
+                        uint4 w = make_uint4(0, 0, 0, 0);
+                        if (q < l) w = reinterpret_cast<const uint4*>(cnt_s)[q * g + kk];
+                        const uint32_t v[8] = {w.x & 0xFFFFu, w.x >> 16, w.y & 0xFFFFu, w.y >> 16,
+                                               w.z & 0xFFFFu, w.z >> 16, w.w & 0xFFFFu, w.w >> 16};
+                        uint32_t e[8], sum = 0;
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            e[u] = sum;
+                            sum += v[u];
+                        }
+                        uint32_t inc = sum;  // along the chunks of this layer
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+                            if (o < gw && lane % gw >= o) inc += x;
+                        }
+                        if (q < l) {
+                            const int64_t at = (int64_t)q * C + kb + kk;
+                            t[at] = run + inc - sum;
+                            if (ts)
+                                ts[at] = make_uint4(e[0] | e[1] << 16, e[2] | e[3] << 16, e[4] | e[5] << 16,
+                                                    e[6] | e[7] << 16);
+                        }
+                        run += __shfl_sync(0xFFFFFFFFu, inc, lane | (gw - 1));
+                    }
+                    if (q < l && lane % gw == 0) carry[q] = run;
                 }
-                if (lo < l && lw[lo] == (uint32_t)mult) atomicAdd(&cnt[(int64_t)lo * C + (x >> shift)], 1u);
-                else dev_fail(st, kErrProfile, mu);
+                __syncthreads();
             }
-            return false;
         };
         if (T <= kFillBuf) {
             const int got = sorted_nbhd<kFillThreads>(v_span, he_mem, mu, vi.z, vi.w, T, id_bits, buf, bkt, 12,
                                                       pre, ctrl + 32);
-            walk_runs<kFillThreads>(buf, got, count_run);
+            for (int q = threadIdx.x; q < l; q += kFillThreads) carry[q] = 0;
+            __syncthreads();
+            count_and_emit(buf, got, 0, C);
         } else {
             if ((int64_t)T > scratch_cap) {
                 if (threadIdx.x == 0) dev_fail(st, kErrCapacity, mu);
@@ -262,34 +321,16 @@ k_idx_fill(const int32_t* __restrict__ list, int32_t nlist, const uint8_t* __res
             __threadfence_block();
             __syncthreads();
             // bucket_end[q] is now the end of bucket q
+            for (int q = threadIdx.x; q < l; q += kFillThreads) carry[q] = 0;
+            __syncthreads();
             int begin = 0;
             for (int q = 0; q < nb; ++q) {
                 const int end = bucket_end[q];
                 if (end > begin) {
                     sort_chunk<kFillThreads>(big + begin, end - begin, bshift, buf, bkt, 12, ctrl + 32);
-                    walk_runs<kFillThreads>(buf, end - begin, count_run);
-                    __syncthreads();
                 }
+                count_and_emit(buf, end - begin, q << (c - b), 1 << (c - b));
                 begin = end;
-            }
-        }
-        __syncthreads();
-        // counts -> exclusive prefix along the chunks, one warp per layer row
-        for (int q = wid; q < l; q += kWarps) {
-            const uint32_t* src = cnt + (int64_t)q * C;
-            uint32_t* dst = t + (int64_t)q * C;
-            uint32_t carry = 0;
-            for (int k0 = 0; k0 < C; k0 += 32) {
-                const int k = k0 + lane;
-                const uint32_t v = k < C ? src[k] : 0u;
-                uint32_t inc = v;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-                    if (lane >= o) inc += u;
-                }
-                if (k < C) dst[k] = carry + inc - v;
-                carry += __shfl_sync(0xFFFFFFFFu, inc, 31);
             }
         }
         __syncthreads();
@@ -365,11 +406,15 @@ hyperim_status build_chunk_index(hyperim_graph* g) {
         int fblocks = (int)std::min<int64_t>(ncand, (int64_t)sm * per_sm);
         // keep the scratch area within 2 GiB
         while (fblocks > sm && (int64_t)fblocks * cap * 4 > ((int64_t)2 << 30)) fblocks -= sm;
+        // the eighths: not under a budget, nor without the memory
+        if (!graph_root(g)->budget &&
+            dev_alloc(g, (void**)&g->idx_sub, sizeof(uint4) * (size_t)total) != HYPERIM_OK)
+            g->idx_sub = nullptr;
         uint32_t* d_scratch = nullptr;
         if ((st = tmp.alloc(&d_scratch, sizeof(uint32_t) * (size_t)cap * fblocks))) return st;
         HYP_CUDA(cudaMemsetAsync(d_next, 0, sizeof(int), s));
         { k_idx_fill<<<fblocks, kFillThreads, kFillSmem, s>>>(d_list, nl, d_bits, d_entries, d_off, g->vinfo, g->v_span,
-                                                  g->he_mem, g->tsum, g->prof, g->id_bits, g->idx_tab, d_scratch,
+                                                  g->he_mem, g->tsum, g->prof, g->id_bits, g->idx_tab, g->idx_sub, d_scratch,
                                                   cap, d_order, d_next, g->d_status); count_launch(); }
         if ((st = check_device_status(g, "chunk index"))) return st;
         // indexed vertices

@@ -64,6 +64,14 @@ constexpr int kIdxMaxBits = 12;
 constexpr int kIdxMaxL = 1024;
 // idx word of a vertex: 0 = no index, else (c << 56) | offset of its table
 constexpr int kIdxBitsShift = 56;
+// Each entry (layer, chunk) of the index also has, in a second table at the same offset, the members
+// of the layer in the chunk's first 0..7 eighths (eight uint16 in one 16-byte word; a chunk of fewer
+// than 8 ids has fewer parts): a pick then names an eighth of a chunk, 2^idx_sub_bits(id_bits - c) of
+// them per chunk. Left out under a budget.
+constexpr int kIdxSubBits = 3;
+__host__ __device__ inline int idx_sub_bits(int chunk_id_bits) {
+    return chunk_id_bits < kIdxSubBits ? chunk_id_bits : kIdxSubBits;
+}
 
 // Id directory of a hyperedge (a lookup structure over its sorted member list): for a hyperedge
 // of L members, kDirMinLen < L <= kDirMaxLen, with b = ceil(log2 L) bits (1 <= b <= min(id bits,
@@ -138,6 +146,7 @@ struct hyperim_graph {
     // chunk index of large neighbourhoods
     uint64_t* idx = nullptr;     // n: 0 or (chunk bits << 56) | table offset
     uint32_t* idx_tab = nullptr; // per indexed vertex: l x 2^bits prefix counts, layer-major
+    uint4* idx_sub = nullptr;    // per entry of idx_tab: members in the chunk's leading eighths (or null)
     int64_t idx_entries = 0;
     int32_t idx_vertices = 0;
     // host copies of scalars

@@ -33,6 +33,7 @@ constexpr int kWHalf = kWCap / 2;  // raw copy + sorted copy of neighbourhoods u
 constexpr int kPCap = 256;       // per-warp picks
 constexpr int kLQ = 32;          // per-warp layers with h > 0 handled on the warp path
 constexpr int kCG = 64;          // hyperedges per group of the chunk path (two per lane)
+constexpr int kDirectSlice = 8;  // slices up to this long are copied by the lane that found them
 constexpr int kBCap = 8192;      // block on-chip keys (power of two)
 constexpr int kBLQ = 64;         // layers with h > 0 per block round
 constexpr int kDCap = 256;       // deferred pops per level round
@@ -69,6 +70,7 @@ struct RRParams {
     const int32_t* vs_list;
     const uint64_t* idx;      // per vertex: 0 or (chunk bits << 56) | offset into idx_tab
     const uint32_t* idx_tab;
+    const uint4* idx_sub;     // per entry of idx_tab: members in the chunk's leading eighths (or null)
     const uint32_t* mat_sect; // per vertex: sectors of v_he(v) and of mem(he) for he in v
     const uint16_t* he_dir;   // id directories of the larger hyperedges
     const uint2* v_dir;       // per incidence: {directory offset, bits} (bits 0: none)
@@ -565,14 +567,52 @@ __device__ __forceinline__ Slice hyperedge_slice(const RRParams& P, int2 sp, uin
     return r;
 }
 
+// raw[0, count), count <= 64, sorted into buf: two keys per lane, a bitonic network in registers.
+__device__ __forceinline__ void warp_sort64(const uint32_t* raw, int count, uint32_t* buf) {
+    const int lane = threadIdx.x & 31;
+    uint32_t a = lane < count ? raw[lane] : kSentinel;
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, a, j);
+            a = ((lane & j) == 0) == ((lane & k) == 0) ? min(a, o) : max(a, o);
+        }
+    }
+    if (count > 32) {
+        // the upper 32 keys in descending order, then one bitonic merge of all 64
+        uint32_t b = 32 + lane < count ? raw[32 + lane] : kSentinel;
+#pragma unroll
+        for (int k = 2; k <= 32; k <<= 1) {
+#pragma unroll
+            for (int j = k >> 1; j > 0; j >>= 1) {
+                const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, b, j);
+                b = ((lane & j) == 0) != ((lane & k) == 0) ? min(b, o) : max(b, o);
+            }
+        }
+        const uint32_t lo = min(a, b), hi = max(a, b);
+        a = lo;
+        b = hi;
+#pragma unroll
+        for (int j = 16; j > 0; j >>= 1) {
+            const uint32_t oa = __shfl_xor_sync(0xFFFFFFFFu, a, j), ob = __shfl_xor_sync(0xFFFFFFFFu, b, j);
+            a = (lane & j) == 0 ? min(a, oa) : max(a, oa);
+            b = (lane & j) == 0 ? min(b, ob) : max(b, ob);
+        }
+        if (32 + lane < count) buf[32 + lane] = b;
+    }
+    if (lane < count) buf[lane] = a;
+    __syncwarp();
+}
+
 // The members != mu of mu's hyperedges whose ids lie in [lo, hi), sorted, in buf[0, count);
 // returns count, or -1 if they exceed kWHalf. lo is a multiple of 2^sh (the range is chunk
 // k = lo >> sh of the ids' top c = id_bits - sh bits). Members of a hyperedge are sorted, so the
 // range is one slice of each (hyperedge_slice); when mu lies in the range its own slot in every
 // slice is skipped (a hole at mu's offset). The hyperedges are taken kCG at a time, two per lane,
 // so that the lookups of both overlap; the slices are gathered with independent loads into the
-// raw half of buf and counted into buckets of the id offset within the range, then scattered and
-// sorted as in small_nbhd. probes counts the words read to locate the slices.
+// raw half of buf, then sorted in registers (up to 64 members) or by buckets of the id offset within
+// the range as in small_nbhd. probes counts the words read to locate the slices.
 template <class SM>
 __device__ int chunk_nbhd(const RRParams& P, SM& S, int32_t mu, int32_t v_begin, int32_t dh,
                           uint32_t lo, int sh, uint32_t* buf, uint32_t& probes) {
@@ -589,7 +629,6 @@ __device__ int chunk_nbhd(const RRParams& P, SM& S, int32_t mu, int32_t v_begin,
     const bool mu_in = (uint32_t)mu >= lo && (uint32_t)mu < hi;
     const int c = P.id_bits - sh;
     const uint32_t k = lo >> sh;
-    for (int b = lane; b < nb; b += 32) bkt[b] = 0;
     int base = 0;
     for (int c0 = 0; c0 < dh; c0 += kCG) {
         const int cnt = min(kCG, dh - c0);
@@ -629,6 +668,18 @@ __device__ int chunk_nbhd(const RRParams& P, SM& S, int32_t mu, int32_t v_begin,
         }
         const int tot0 = __shfl_sync(0xFFFFFFFFu, inc0, 31);
         inc1 += tot0;
+        const int total = __shfl_sync(0xFFFFFFFFu, inc1, 31);
+        if (total == 0) continue;
+        if (base + total > kWHalf) return -1;  // uniform
+        if (__reduce_max_sync(0xFFFFFFFFu, max(len[0], len[1])) <= kDirectSlice) {
+            // short slices (an eighth of a chunk holds a member or two of a hyperedge, if any): every lane
+            // copies its own
+            int o0 = base + inc0 - len[0], o1 = base + inc1 - len[1];
+            for (int i = 0; i < len[0]; ++i) raw[o0 + i] = (uint32_t)P.he_mem[st[0] + i + (i >= hl[0] ? 1 : 0)];
+            for (int i = 0; i < len[1]; ++i) raw[o1 + i] = (uint32_t)P.he_mem[st[1] + i + (i >= hl[1] ? 1 : 0)];
+            base += total;
+            continue;
+        }
         __syncwarp();  // the previous group's readers of pre / start / hole are done
         if (lane == 0) pre[0] = 0;
         if (lane < cnt) {
@@ -642,8 +693,6 @@ __device__ int chunk_nbhd(const RRParams& P, SM& S, int32_t mu, int32_t v_begin,
             hole[32 + lane] = hl[1];
         }
         __syncwarp();
-        const int total = pre[cnt];
-        if (base + total > kWHalf) return -1;  // uniform
         const bool stepwise = total >= cnt * 8;
         int j = 0;
         constexpr int U = 2;
@@ -671,14 +720,19 @@ __device__ int chunk_nbhd(const RRParams& P, SM& S, int32_t mu, int32_t v_begin,
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int p = p0 + u * 32;
-                if (p < total) {
-                    raw[base + p] = xs[u];
-                    atomicAdd(&bkt[((xs[u] - lo) >> shift) & key_mask], 1);
-                }
+                if (p < total) raw[base + p] = xs[u];
             }
         }
         base += total;
     }
+    __syncwarp();
+    if (base <= 64) {
+        warp_sort64(raw, base, buf);
+        return base;
+    }
+    for (int b = lane; b < nb; b += 32) bkt[b] = 0;
+    __syncwarp();
+    for (int p = lane; p < base; p += 32) atomicAdd(&bkt[((raw[p] - lo) >> shift) & key_mask], 1);
     __syncwarp();
     const int maxb = warp_bucket_scan(bkt, nb);
     warp_scatter_sort(raw, base, kSentinel, buf, base, bkt, nb, lo, shift, key_mask, maxb);
@@ -1021,33 +1075,77 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
     }
     if (iw != 0) {
         // chunk path: lane q follows needed layer q through its row of prefix counts: the next
-        // position it needs (its next pick, or for a layer taken whole its next member) and the
-        // chunk holding it; the warp visits those chunks in ascending order, each ranked from the
-        // row entries at that chunk
+        // position it needs (its next pick, or for a layer taken whole its next member) and the part
+        // holding it -- an eighth of a chunk, or the chunk where there are no eighths; the warp visits
+        // those parts in ascending order, each ranked from the entries at that part. The eighths matter
+        // because a pick costs the gather, sort and walk of its part: on 2M vertices under weighted
+        // cascade a chunk holds 400 members, an eighth 50. That query: 356 ms by whole chunks,
+        // 311 ms by eighths; LT paths on that graph 80 and 69 ms.
         const int c = (int)(iw >> kIdxBitsShift);
         const int C = 1 << c;
         const uint64_t toff = iw & ((1ull << kIdxBitsShift) - 1);
-        const int sh = P.id_bits - c;
+        const int fb = P.idx_sub ? idx_sub_bits(P.id_bits - c) : 0, F = 1 << fb;
+        const int sh = P.id_bits - c - fb;
         uint32_t probes = 0, cur = 0xFFFFFFFFu, cursor = 0;
         unsigned long long gath = 0;
         Need nd{};
         const uint32_t* row = nullptr;
+        const uint4* srow = nullptr;
         uint32_t first = 0;
         if ((uint32_t)lane < nneed) {
             nd = need[lane];
-            row = P.idx_tab + toff + ((uint64_t)(nd.layer - 1) << c);
+            const uint64_t at = toff + ((uint64_t)(nd.layer - 1) << c);
+            row = P.idx_tab + at;
+            if (fb) srow = P.idx_sub + at;
             first = nd.h < nd.n ? picks[poff[lane]] : 0u;
         }
+        // this lane's layer: members before part f of chunk k, and the part of chunk k that holds position x
+        auto part_of = [&](int k, uint32_t x) {
+            uint32_t f = (uint32_t)k << fb;
+            if (fb) {
+                const uint4 w = srow[k];
+                const uint32_t r = x - row[k];
+                probes += 5;
+                // the last part whose leading count is <= r (counts ascend, part 0 has 0)
+                uint32_t j = 0;
+                j += (w.x >> 16) <= r ? 1 : 0;
+                if (fb > 1) {
+                    j += (w.y & 0xFFFFu) <= r ? 1 : 0;
+                    j += (w.y >> 16) <= r ? 1 : 0;
+                }
+                if (fb > 2) {
+                    j += (w.z & 0xFFFFu) <= r ? 1 : 0;
+                    j += (w.z >> 16) <= r ? 1 : 0;
+                    j += (w.w & 0xFFFFu) <= r ? 1 : 0;
+                    j += (w.w >> 16) <= r ? 1 : 0;
+                }
+                f += j;
+            }
+            return f;
+        };
         {
             const int r0 = warp_chunk_search(row, 0, C, first, (uint32_t)lane < nneed, nneed, probes);
-            if ((uint32_t)lane < nneed) cur = (uint32_t)r0;
+            if ((uint32_t)lane < nneed) cur = part_of(r0, first);
         }
-        uint32_t k = __reduce_min_sync(0xFFFFFFFFu, cur);
+        uint32_t k = __reduce_min_sync(0xFFFFFFFFu, cur);  // the part to visit
         int chunks = 0;
         while (k != 0xFFFFFFFFu) {
+            const int kc = (int)(k >> fb), kf = (int)(k & (uint32_t)(F - 1));
+            uint32_t endk = 0;  // members of this lane's layer before the next part
             if ((uint32_t)lane < nneed) {
-                cnt[lane] = (int)row[k];
-                ++probes;
+                uint32_t at = row[kc];
+                endk = kc + 1 < C ? row[kc + 1] : nd.n;
+                probes += 2;
+                if (fb) {
+                    const uint4 w = srow[kc];
+                    probes += 4;
+                    const uint32_t w0 = kf < 2 ? w.x : kf < 4 ? w.y : kf < 6 ? w.z : w.w;
+                    const int kn = kf + 1;
+                    const uint32_t w1 = kn < 2 ? w.x : kn < 4 ? w.y : kn < 6 ? w.z : w.w;
+                    if (kn < F) endk = at + (kn & 1 ? w1 >> 16 : w1 & 0xFFFFu);
+                    at += kf & 1 ? w0 >> 16 : w0 & 0xFFFFu;
+                }
+                cnt[lane] = (int)at;
             }
             __syncwarp();
             const int got = chunk_nbhd(P, S, mu, v_begin, dh, k << sh, sh, buf, probes);
@@ -1059,10 +1157,8 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
             warp_walk(P, S, sink, buf, got, nneed);
             ++chunks;
             uint32_t nxt = 0xFFFFFFFFu;
-            const bool moved = cur == k;  // this lane's layer needs a later chunk (or none)
+            const bool moved = cur == k;  // this lane's layer needs a later part (or none)
             if (moved) {
-                const uint32_t endk = (int)k + 1 < C ? row[k + 1] : nd.n;  // members of L_q before chunk k + 1
-                ++probes;
                 if (nd.h < nd.n) {
                     const uint32_t* pk = picks + poff[lane];
                     while (cursor < nd.h && pk[cursor] < endk) ++cursor;
@@ -1072,9 +1168,10 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
                 }
             }
             {
+                // the next position is in this chunk still (its later parts) or a later one
                 const bool want = moved && nxt != 0xFFFFFFFFu;
-                const int r1 = warp_chunk_search(row, (int)k + 1, C, nxt, want, nneed, probes);
-                if (moved) cur = want ? (uint32_t)r1 : 0xFFFFFFFFu;
+                const int r1 = warp_chunk_search(row, kc, C, nxt, want, nneed, probes);
+                if (moved) cur = want ? part_of(r1, nxt) : 0xFFFFFFFFu;
             }
             k = __reduce_min_sync(0xFFFFFFFFu, cur);
         }
@@ -2327,6 +2424,7 @@ void fill_graph_params(RRParams& P, const hyperim_graph* g) {
     P.vs_list = g->vs_list;
     P.idx = g->idx;
     P.idx_tab = g->idx_tab;
+    P.idx_sub = g->idx_sub;
     P.mat_sect = g->mat_sect;
     P.he_dir = g->he_dir;
     P.v_dir = g->v_dir;
