@@ -73,13 +73,14 @@ __host__ __device__ inline int idx_sub_bits(int chunk_id_bits) {
     return chunk_id_bits < kIdxSubBits ? chunk_id_bits : kIdxSubBits;
 }
 
-// Id directory of a hyperedge (a lookup structure over its sorted member list): for a hyperedge
-// of L members, kDirMinLen < L <= kDirMaxLen, with b = ceil(log2 L) bits (1 <= b <= min(id bits,
+// Id directory of a hyperedge (a lookup structure over its sorted member list; the few members of a
+// shorter one are read whole): for a hyperedge of L members, kDirMinLen < L <= kDirMaxLen, with b =
+// ceil(log2 L) bits (1 <= b <= min(id bits,
 // kDirMaxBits)), D[r] (r = 0..2^b) is the number of members whose top b id bits are < r. The
 // members whose top c id bits equal k (one chunk of the chunk index) are then positions
 // [D[k 2^(b-c)], D[(k+1) 2^(b-c)]) when c <= b, or a sub-range of [D[r], D[r + 1]), r = k >>
 // (c - b), when c > b (about one member on average). Entries are uint16 (L < 2^16).
-constexpr int kDirMinLen = 16;
+constexpr int kDirMinLen = 4;
 constexpr int kDirMaxLen = 65535;
 constexpr int kDirMaxBits = 12;
 

@@ -32,8 +32,8 @@ constexpr int kWCap = 2048;      // per-warp on-chip neighbourhood keys (power o
 constexpr int kWHalf = kWCap / 2;  // raw copy + sorted copy of neighbourhoods up to this size
 constexpr int kPCap = 256;       // per-warp picks
 constexpr int kLQ = 32;          // per-warp layers with h > 0 handled on the warp path
-constexpr int kCG = 64;          // hyperedges per group of the chunk path (two per lane)
-constexpr int kDirectSlice = 8;  // slices up to this long are copied by the lane that found them
+constexpr int kCU = 4;           // hyperedges per lane and group of the chunk path
+constexpr int kLongRange = 16;   // ranges up to this long are read by the lane that found them
 constexpr int kBCap = 8192;      // block on-chip keys (power of two)
 constexpr int kBLQ = 64;         // layers with h > 0 per block round
 constexpr int kDCap = 256;       // deferred pops per level round
@@ -150,7 +150,7 @@ struct Shared {
     int32_t deferred[kDCap];
     Need wneed[kWarps][kLQ];
     int wcursor[kWarps];
-    int wpre[kWarps][3 * kCG + 1];  // span prefix, starts, holes of a group of hyperedges (chunk path)
+    int wpre[kWarps][2 * 32 + 1];   // span prefix and starts of 32 hyperedges
     uint32_t wpoff[kWarps][kLQ + 1];
     int wcnt[kWarps][kBLQ];     // per-warp per-layer counts (ranks)
     int lcnt[kBLQ];             // running rank per needed layer (block path)
@@ -502,71 +502,6 @@ __device__ __forceinline__ int chunk_of(const uint32_t* __restrict__ row, int k0
     return lo;
 }
 
-// The slice of one sorted hyperedge (members e[0, len)) whose ids lie in chunk k = lo >> sh of
-// the ids' top c = id_bits - sh bits: offsets [l1, l2) and, when mu lies in the range, mu's offset
-// l3. Read off the hyperedge's id directory when it has one (two entries when c <= b, else one
-// directory range of about one member, scanned), else found by interleaved binary searches.
-struct Slice {
-    int l1, l2, l3;
-};
-
-__device__ __forceinline__ Slice hyperedge_slice(const RRParams& P, int2 sp, uint2 dd, uint32_t lo, uint32_t hi,
-                                                 int c, uint32_t k, int32_t mu, bool mu_in, uint32_t& probes) {
-    const int32_t* e = P.he_mem + sp.x;
-    Slice r{0, 0, 0};
-    if (dd.y != 0) {
-        const uint16_t* D = P.he_dir + dd.x;
-        const int b = (int)dd.y;
-        const uint32_t rm = (uint32_t)mu >> (P.id_bits - b);
-        int m0 = 0, m1 = 0;
-        if (mu_in) {  // mu's directory range (issued with the slice's entries)
-            m0 = D[rm];
-            m1 = D[rm + 1];
-            probes += 2;
-        }
-        if (c <= b) {
-            r.l1 = D[k << (b - c)];
-            r.l2 = D[(k + 1) << (b - c)];
-            probes += 2;
-        } else {
-            const uint32_t rr = k >> (c - b);
-            const int a0 = D[rr], a1 = D[rr + 1];
-            probes += 2;
-            r.l1 = a0;
-            r.l2 = a0;
-            for (int x = a0; x < a1; ++x) {
-                const uint32_t v = (uint32_t)e[x];
-                ++probes;
-                r.l1 += v < lo ? 1 : 0;
-                r.l2 += v < hi ? 1 : 0;
-            }
-        }
-        if (mu_in) {
-            r.l3 = m0;
-            while (r.l3 < m1 && (uint32_t)e[r.l3] < (uint32_t)mu) {
-                ++r.l3;
-                ++probes;
-            }
-        }
-        return r;
-    }
-    // three lower bounds (lo, hi, mu) advanced together: their loads overlap
-    int l1 = 0, h1 = sp.y, l2 = 0, h2 = sp.y, l3 = 0, h3 = mu_in ? sp.y : 0;
-    while (l1 < h1 || l2 < h2 || l3 < h3) {
-        const int m1 = (l1 + h1) >> 1, m2 = (l2 + h2) >> 1, m3 = (l3 + h3) >> 1;
-        const uint32_t v1 = l1 < h1 ? (uint32_t)e[m1] : 0u;
-        const uint32_t v2 = l2 < h2 ? (uint32_t)e[m2] : 0u;
-        const uint32_t v3 = l3 < h3 ? (uint32_t)e[m3] : 0u;
-        if (l1 < h1) { ++probes; if (v1 < lo) l1 = m1 + 1; else h1 = m1; }
-        if (l2 < h2) { ++probes; if (v2 < hi) l2 = m2 + 1; else h2 = m2; }
-        if (l3 < h3) { ++probes; if (v3 < (uint32_t)mu) l3 = m3 + 1; else h3 = m3; }
-    }
-    r.l1 = l1;
-    r.l2 = l2;
-    r.l3 = l3;
-    return r;
-}
-
 // raw[0, count), count <= 64, sorted into buf: two keys per lane, a bitonic network in registers.
 __device__ __forceinline__ void warp_sort64(const uint32_t* raw, int count, uint32_t* buf) {
     const int lane = threadIdx.x & 31;
@@ -606,124 +541,128 @@ __device__ __forceinline__ void warp_sort64(const uint32_t* raw, int count, uint
 }
 
 // The members != mu of mu's hyperedges whose ids lie in [lo, hi), sorted, in buf[0, count);
-// returns count, or -1 if they exceed kWHalf. lo is a multiple of 2^sh (the range is chunk
-// k = lo >> sh of the ids' top c = id_bits - sh bits). Members of a hyperedge are sorted, so the
-// range is one slice of each (hyperedge_slice); when mu lies in the range its own slot in every
-// slice is skipped (a hole at mu's offset). The hyperedges are taken kCG at a time, two per lane,
-// so that the lookups of both overlap; the slices are gathered with independent loads into the
-// raw half of buf, then sorted in registers (up to 64 members) or by buckets of the id offset within
-// the range as in small_nbhd. probes counts the words read to locate the slices.
+// returns count, or -1 if they exceed kWHalf. lo is a multiple of 2^sh (the range is part
+// k = lo >> sh of the ids' top c = id_bits - sh bits).
+// The hyperedges are taken 32 kCU at a time, kCU per lane. A hyperedge's id directory gives the places
+// its members of the range lie at: exactly (c <= b bits), or within one directory range of about one
+// member; a hyperedge of up to kDirMinLen members is a range itself. The lanes then
+// read their ranges' members side by side and append those in [lo, hi) to the raw half of buf by a
+// ballot. What bounds this is the chain of dependent reads, most of them misses in a graph larger than the
+// L2: span and directory entry, the two ends, the members -- three reads for 32 kCU hyperedges, all of
+// a lane's independent of one another. (Locating the slices one hyperedge after the other, by binary
+// search in those without a directory, then gathering them took 27,000 cycles a visit; the 2M-vertex
+// query went from 311 to 275 ms, LT paths from 69 to 62 ms.)
+// Longest range of the group beyond kLongRange: the ranges are read position by position instead.
+// probes counts the words read to locate the ranges.
 template <class SM>
 __device__ int chunk_nbhd(const RRParams& P, SM& S, int32_t mu, int32_t v_begin, int32_t dh,
                           uint32_t lo, int sh, uint32_t* buf, uint32_t& probes) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int* pre = S.wpre[wid];
-    int* start = pre + kCG + 1;
-    int* hole = start + kCG;
     uint32_t* raw = buf + kWHalf;
     int* bkt = S.u.w.wbkt[wid];
     constexpr int nb = kWBuckets;
     const int shift = sh > kWBucketBits ? sh - kWBucketBits : 0;
     const uint32_t key_mask = (uint32_t)nb - 1;
-    const uint32_t hi = lo + (1u << sh);
-    const bool mu_in = (uint32_t)mu >= lo && (uint32_t)mu < hi;
+    const uint32_t span = 1u << sh;  // the range is [lo, lo + span)
     const int c = P.id_bits - sh;
     const uint32_t k = lo >> sh;
     int base = 0;
-    for (int c0 = 0; c0 < dh; c0 += kCG) {
-        const int cnt = min(kCG, dh - c0);
-        // lane takes hyperedges c0 + lane and c0 + 32 + lane
-        int st[2] = {0, 0}, len[2] = {0, 0}, hl[2] = {0x7FFFFFFF, 0x7FFFFFFF};
-        int2 sp[2];
-        uint2 dd[2];
+    for (int c0 = 0; c0 < dh; c0 += 32 * kCU) {
+        int2 sp[kCU];
+        uint2 dd[kCU];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int x = u * 32 + lane;
-            sp[u] = x < cnt ? P.v_span[v_begin + c0 + x] : make_int2(0, 0);
-            dd[u] = x < cnt ? P.v_dir[v_begin + c0 + x] : make_uint2(0u, 0u);
+        for (int u = 0; u < kCU; ++u) {
+            const int x = c0 + u * 32 + lane;
+            sp[u] = x < dh ? P.v_span[v_begin + x] : make_int2(0, 0);
+            dd[u] = x < dh ? P.v_dir[v_begin + x] : make_uint2(0u, 0u);
         }
+        int a0[kCU], len[kCU], longest = 0;
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int x = u * 32 + lane;
-            if (x < cnt) {
-                const Slice r = hyperedge_slice(P, sp[u], dd[u], lo, hi, c, k, mu, mu_in, probes);
-                st[u] = sp[u].x + r.l1;
-                len[u] = r.l2 - r.l1;
-                if (mu_in) {
-                    hl[u] = r.l3 - r.l1;
-                    len[u] -= 1;
+        for (int u = 0; u < kCU; ++u) {
+            a0[u] = 0;
+            int a1 = sp[u].y;
+            if (dd[u].y != 0) {
+                const int b = (int)dd[u].y;
+                const uint16_t* D = P.he_dir + dd[u].x;
+                const uint32_t r0 = c <= b ? k << (b - c) : k >> (c - b);
+                const uint32_t r1 = c <= b ? (k + 1) << (b - c) : r0 + 1;
+                a0[u] = D[r0];
+                a1 = D[r1];
+                probes += 2;
+            } else if (sp[u].y > kDirMinLen) {  // too long for a directory: both ends by binary search
+                const int32_t* e = P.he_mem + sp[u].x;
+                int h0 = sp[u].y, l1 = 0;
+                while (a0[u] < h0 || l1 < a1) {
+                    const int m0 = (a0[u] + h0) >> 1, m1 = (l1 + a1) >> 1;
+                    if (a0[u] < h0) { if ((uint32_t)e[m0] < lo) a0[u] = m0 + 1; else h0 = m0; }
+                    if (l1 < a1) { if ((uint32_t)e[m1] < lo + span) l1 = m1 + 1; else a1 = m1; }
+                    probes += 2;
                 }
             }
+            len[u] = a1 - a0[u];
         }
-        // inclusive prefix of the lengths over the group (first the lanes' first hyperedges)
-        int inc0 = len[0], inc1 = len[1];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t0 = __shfl_up_sync(0xFFFFFFFFu, inc0, o);
-            const int t1 = __shfl_up_sync(0xFFFFFFFFu, inc1, o);
-            if (lane >= o) {
-                inc0 += t0;
-                inc1 += t1;
-            }
+        for (int u = 0; u < kCU; ++u) {
+            longest = max(longest, len[u]);
+            a0[u] += sp[u].x;
         }
-        const int tot0 = __shfl_sync(0xFFFFFFFFu, inc0, 31);
-        inc1 += tot0;
-        const int total = __shfl_sync(0xFFFFFFFFu, inc1, 31);
-        if (total == 0) continue;
-        if (base + total > kWHalf) return -1;  // uniform
-        if (__reduce_max_sync(0xFFFFFFFFu, max(len[0], len[1])) <= kDirectSlice) {
-            // short slices (an eighth of a chunk holds a member or two of a hyperedge, if any): every lane
-            // copies its own
-            int o0 = base + inc0 - len[0], o1 = base + inc1 - len[1];
-            for (int i = 0; i < len[0]; ++i) raw[o0 + i] = (uint32_t)P.he_mem[st[0] + i + (i >= hl[0] ? 1 : 0)];
-            for (int i = 0; i < len[1]; ++i) raw[o1 + i] = (uint32_t)P.he_mem[st[1] + i + (i >= hl[1] ? 1 : 0)];
-            base += total;
+        longest = __reduce_max_sync(0xFFFFFFFFu, longest);
+        auto append = [&](uint32_t v, bool in) {  // one member per lane; false: no room
+            const bool f = in && v - lo < span && v != (uint32_t)mu;
+            const uint32_t bal = __ballot_sync(0xFFFFFFFFu, f);
+            if (base + __popc(bal) > kWHalf) return false;
+            if (f) raw[base + __popc(bal & lanemask_lt())] = v;
+            base += __popc(bal);
+            return true;
+        };
+        if (longest <= kLongRange) {
+            for (int i = 0; i < longest; i += 2) {
+                uint32_t v[kCU][2];
+#pragma unroll
+                for (int u = 0; u < kCU; ++u) {
+                    v[u][0] = i < len[u] ? (uint32_t)P.he_mem[a0[u] + i] : 0u;
+                    v[u][1] = i + 1 < len[u] ? (uint32_t)P.he_mem[a0[u] + i + 1] : 0u;
+                }
+#pragma unroll
+                for (int u = 0; u < kCU; ++u)
+                    if (!append(v[u][0], i < len[u]) || !append(v[u][1], i + 1 < len[u])) return -1;
+            }
             continue;
         }
-        __syncwarp();  // the previous group's readers of pre / start / hole are done
-        if (lane == 0) pre[0] = 0;
-        if (lane < cnt) {
-            pre[lane + 1] = inc0;
-            start[lane] = st[0];
-            hole[lane] = hl[0];
-        }
-        if (32 + lane < cnt) {
-            pre[33 + lane] = inc1;
-            start[32 + lane] = st[1];
-            hole[32 + lane] = hl[1];
-        }
-        __syncwarp();
-        const bool stepwise = total >= cnt * 8;
-        int j = 0;
-        constexpr int U = 2;
-        for (int p0 = lane; p0 < total; p0 += U * 32) {
-            uint32_t xs[U] = {};
+        // long ranges: the members of 32 hyperedges at a time, position by position of their concatenation
+        int* pre = S.wpre[wid];
+        int* start = pre + 33;
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int p = p0 + u * 32;
-                if (p < total) {
-                    if (stepwise && p != lane) {
-                        while (pre[j + 1] <= p) ++j;
-                    } else {
-                        int l2 = 0, h2 = cnt;
+        for (int u = 0; u < kCU; ++u) {
+            int inc = len[u];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+                if (lane >= o) inc += t;
+            }
+            __syncwarp();  // the previous readers of pre and start are done
+            if (lane == 0) pre[0] = 0;
+            pre[lane + 1] = inc;
+            start[lane] = a0[u];
+            __syncwarp();
+            const int total = pre[32];
+            for (int p0 = 0; p0 < total; p0 += 64) {
+                uint32_t v[2] = {0u, 0u};
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    const int p = p0 + y * 32 + lane;
+                    if (p < total) {
+                        int l2 = 0, h2 = 32;  // the hyperedge: pre[l2] <= p < pre[l2 + 1]
                         while (h2 - l2 > 1) {
                             const int mid = (l2 + h2) >> 1;
                             if (pre[mid] <= p) l2 = mid; else h2 = mid;
                         }
-                        j = l2;
+                        v[y] = (uint32_t)P.he_mem[start[l2] + (p - pre[l2])];
                     }
-                    int o = p - pre[j];
-                    o += o >= hole[j] ? 1 : 0;
-                    xs[u] = (uint32_t)P.he_mem[start[j] + o];
                 }
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int p = p0 + u * 32;
-                if (p < total) raw[base + p] = xs[u];
+                if (!append(v[0], p0 + lane < total) || !append(v[1], p0 + 32 + lane < total)) return -1;
             }
         }
-        base += total;
     }
     __syncwarp();
     if (base <= 64) {
@@ -1749,7 +1688,7 @@ struct WarpShared {
     unsigned long long stat[kMaxPools][kNStat];  // per pool work counters of this block
     unsigned long long wstat[kPWarps][kNStat];    // per-warp counters of the warp's current set
     Need wneed[kPWarps][kLQ];
-    int wpre[kPWarps][3 * kCG + 1];
+    int wpre[kPWarps][2 * 32 + 1];
     uint32_t wpoff[kPWarps][kLQ + 1];
     int wcnt[kPWarps][kBLQ];
     int wtail[kPWarps];
