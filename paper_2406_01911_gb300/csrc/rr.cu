@@ -36,7 +36,7 @@ constexpr int kCU = 4;           // hyperedges per lane and group of the chunk p
 constexpr int kLongRange = 16;   // ranges up to this long are read by the lane that found them
 constexpr int kBCap = 8192;      // block on-chip keys (power of two)
 constexpr int kBLQ = 64;         // layers with h > 0 per block round
-constexpr int kDCap = 256;       // deferred pops per level round
+constexpr int kDCap = 1024;      // deferred pops per level round (every warp may hold 32 claimed ones)
 constexpr int kBucketBits = 12;
 constexpr int kBuckets = 1 << kBucketBits;    // block-path buckets
 constexpr int kWBucketBits = 8;
@@ -45,6 +45,11 @@ constexpr int kChunks = 1024;        // first-level id chunks of the largest nei
 constexpr int kVisSmemBits = 1 << 19;  // visited bitmap on chip when n <= this
 constexpr int kMaxPools = 2;           // pools grown by one launch (R1 and R2 of a BRR round)
 constexpr int kNStat = 10;             // work counters (stat slots below)
+// pops by lane (see pop_lanes)
+constexpr int kLaneLayers = 8;
+constexpr uint32_t kLanePicks = 7, kLaneAll = 16;
+constexpr int kLaneMin = 4;
+constexpr int kLaneMaxDh = 1 << 20, kLaneMaxT = 1 << 26;  // keep the warp's 32-bit sums of counters exact
 // warp phase: a warp builds a whole RR set alone while it stays within kWQ members
 constexpr int kWQ = 128;               // per-warp queue (members of the warp's set)
 constexpr int kWHashBits = 8;
@@ -388,15 +393,21 @@ struct WarpSink {
 // itself done, so the head and tail read afterwards include them, and a warp leaves only when
 // the queue is quiescent (a warp that left early would idle at the barrier for the rest of the
 // set). The wait is bounded (kErrSpin).
+// take (in): the most slots to claim, (out): the slots claimed (consecutive); see Pops by lane.
 template <class SM>
-__device__ int claim_slot(const RRParams& P, SM& S, int64_t job) {
+__device__ int claim_slot(const RRParams& P, SM& S, int64_t job, int& take) {
     volatile int* ctrl = S.ctrl;
     for (int it = 0; it < P.spin_limit; ++it) {
         const int d = ctrl[C_DONE];
         __threadfence_block();
         const int h = ctrl[C_HEAD], t = ctrl[C_TAIL], nd = ctrl[C_NDEF];
-        if (h < t && nd <= kDCap - kWarps) {
-            if (atomicCAS(&S.ctrl[C_HEAD], h, h + 1) == h) return h;
+        if (h < t && nd <= kDCap - 32 * kWarps) {
+            const int share = (t - h) / (2 * kWarps);
+            const int want = share < kLaneMin ? 1 : min(share, take);
+            if (atomicCAS(&S.ctrl[C_HEAD], h, h + want) == h) {
+                take = want;
+                return h;
+            }
             continue;
         }
         if (h - nd == d) return -1;
@@ -731,21 +742,6 @@ __device__ void warp_walk(const RRParams& P, SM& S, const Sink& sink, const uint
     __syncwarp();
 }
 
-// Number of entries of the ascending e[0, len) below x, by the whole warp (every lane passes the same
-// arguments): 32 evenly spaced probes a round, so 1,000 entries take two dependent loads.
-__device__ __forceinline__ int warp_lower_bound(const int32_t* __restrict__ e, int len, int32_t x) {
-    const int lane = threadIdx.x & 31;
-    int lo = 0, hi = len;  // the answer lies in [lo, hi]
-    while (hi - lo > 32) {
-        const int step = (hi - lo + 31) >> 5;
-        const int p = lo + (lane + 1) * step - 1;
-        const int below = __popc(__ballot_sync(0xFFFFFFFFu, p < hi && e[p] < x));
-        hi = min(hi, lo + (below + 1) * step - 1);
-        lo += below * step;
-    }
-    return lo + __popc(__ballot_sync(0xFFFFFFFFu, lane < hi - lo && e[lo + lane] < x));
-}
-
 // ------------------------------------------------------------------------------------------
 // Memo: neighbourhoods kept within one growth step
 // ------------------------------------------------------------------------------------------
@@ -845,6 +841,115 @@ __device__ __forceinline__ void memo_take(const RRParams& P, SM& S, const Sink& 
         }
     }
     __syncwarp();
+}
+
+// A(mu) of a vertex in one hyperedge (members from place hb on, sorted) is that hyperedge minus mu:
+// position x is its member x, or x + 1 from mu's own place on.
+__device__ __forceinline__ uint32_t single_member(const RRParams& P, int32_t hb, int x, int32_t mu) {
+    const int32_t v = P.he_mem[hb + x];
+    return (uint32_t)(v >= mu ? P.he_mem[hb + x + 1] : v);
+}
+
+// ------------------------------------------------------------------------------------------
+// Pops by lane
+// ------------------------------------------------------------------------------------------
+// Once neighbourhoods are kept (the memo), a pop is a chain of dependent reads and one Philox block for
+// one or two layers, 31 of a warp's lanes idle: 3,200 cycles of draws and 2,400 of picks at p = 0.01 on
+// 100k vertices. While a set's queue is long its warps therefore claim up to 32 pops at once and every
+// lane does one alone: the draws of at most kLaneLayers layers, and, where A(mu) is a kept
+// neighbourhood or one hyperedge, up to kLanePicks picks a layer, pushed as they are drawn. A pop that
+// turns out to be more than that goes to the whole warp and starts over (the draws are keyed, so it
+// finds the same; what was pushed already is in R either way).
+// The query there went from 295 to 108 ms, the 2M-vertex one from 275 to 263 ms.
+// A warp takes its 32nd of the waiting pops, so that claims stay spread, and batches from kLaneMin on:
+// short queues (most sets on 2M vertices) are popped one by one as before.
+// Lane pops mu (-1: nothing); returns the lanes whose pop must be done by the warp.
+template <class SM, class Sink>
+__device__ uint32_t pop_lanes(const RRParams& P, SM& S, const Sink& sink, uint32_t j, uint32_t ybase, int32_t mu) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const bool act = mu >= 0;
+    int4 vi = make_int4(0, 0, 0, 0);
+    uint32_t kept = kMemoNone;
+    int32_t tsum = 0;
+    if (act) {
+        vi = P.vinfo[mu];
+        tsum = P.tsum[mu];
+        if (P.memo_slot) kept = ld_strong(P.memo_slot + mu);
+    }
+    const int l = vi.y, dh = vi.w;
+    bool slow = act && (l > kLaneLayers || dh >= kLaneMaxDh || tsum >= kLaneMaxT);
+    const uint32_t* members = nullptr;  // A(mu) layer by layer, when kept
+    if (kept >= kMemoFirst && kept < kMemoBusy) members = P.memo + (kept - kMemoFirst);
+    int32_t hb = 0;
+    if (act && !slow && dh == 1) hb = P.v_span[vi.z].x;
+    const bool direct = dh == 1 || members != nullptr;
+    uint32_t draws = 0, sel = 0, read = 0;
+    const int lmax = __reduce_max_sync(0xFFFFFFFFu, slow ? 0 : l);
+    for (int i = 0; i < lmax; ++i) {
+        if (slow || i >= l) continue;
+        const uint4 e = P.prof[2 * ((int64_t)vi.x + i)], f = P.prof[2 * ((int64_t)vi.x + i) + 1];
+        WordStream ws;
+        ws.init(P.seed, j, ybase, (uint32_t)mu, (uint32_t)(i + 1));
+        uint32_t h = 0, ksel = 0;
+        draws += layer_draw(e, f, P.tab, P.strategy, ws, h, ksel) ? 1u : 0u;
+        if (h == 0) continue;
+        const uint32_t n = e.y;
+        if (!direct || (h < n ? h > kLanePicks || ksel > 64 : n > kLaneAll)) {
+            slow = true;
+            continue;
+        }
+        sel += h;
+        read += h < n ? h : n;
+        auto push_at = [&](uint32_t x) {
+            sink.push(dh == 1 ? single_member(P, hb, (int)x, mu) : ld_strong(members + f.w + x));
+        };
+        if (h >= n) {
+            for (uint32_t x = 0; x < n; ++x) push_at(x);
+            continue;
+        }
+        // the picks so far in ascending order: the a-th position not picked yet moves past each that is
+        // not above it
+        uint32_t s[kLanePicks];
+#pragma unroll
+        for (uint32_t t = 0; t < kLanePicks; ++t) s[t] = 0xFFFFFFFFu;
+        for (uint32_t r = 0; r < h; ++r) {
+            uint32_t x = (uint32_t)(((uint64_t)ws.word(ksel + r) * (uint64_t)(n - r)) >> 32);
+#pragma unroll
+            for (uint32_t t = 0; t < kLanePicks; ++t) x += s[t] <= x ? 1u : 0u;
+            push_at(x);
+#pragma unroll
+            for (uint32_t t = kLanePicks - 1; t > 0; --t) s[t] = max(s[t - 1], min(s[t], x));
+            s[0] = min(s[0], x);
+        }
+    }
+    // work counters of the pops that are finished
+    const bool done = act && !slow;
+    const bool mat = done && sel > 0;
+    const uint32_t sect = done ? (uint32_t)sectors_of(12ull * (uint64_t)vi.x, 12ull * (uint64_t)l) + (mat ? P.mat_sect[mu] : 0u)
+                               : 0u;
+    const uint32_t sums[9] = {
+        __reduce_add_sync(0xFFFFFFFFu, done ? 1u : 0u),
+        __reduce_add_sync(0xFFFFFFFFu, done ? (uint32_t)l : 0u),
+        __reduce_add_sync(0xFFFFFFFFu, done ? draws : 0u),
+        __reduce_add_sync(0xFFFFFFFFu, mat ? 1u : 0u),
+        __reduce_add_sync(0xFFFFFFFFu, mat ? (uint32_t)dh : 0u),
+        __reduce_add_sync(0xFFFFFFFFu, mat ? (uint32_t)tsum : 0u),
+        __reduce_add_sync(0xFFFFFFFFu, mat ? sel : 0u),
+        __reduce_add_sync(0xFFFFFFFFu, mat ? (dh == 1 ? (uint32_t)tsum : read) : 0u),
+        __reduce_add_sync(0xFFFFFFFFu, sect)};
+    if (lane == 0) {
+        unsigned long long* wst = S.wstat[wid];
+        wst[S_POPS] += sums[0];
+        wst[S_LAYERS] += sums[1];
+        wst[S_DRAWS] += sums[2];
+        wst[S_MATS] += sums[3];
+        wst[S_MAT_HE] += sums[4];
+        wst[S_MAT_MEM] += sums[5];
+        wst[S_SEL] += sums[6];
+        wst[S_GATH] += sums[7];
+        wst[S_SECT] += sums[8];
+    }
+    return __ballot_sync(0xFFFFFFFFu, slow);
 }
 
 // Returns true when the pop must be handed to the block path.
@@ -964,19 +1069,12 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
     if (lane == 0) poff[nneed] = acc;
     __syncwarp();
     if (dh == 1) {
-        // A(mu) = the single hyperedge minus mu, sorted: position x maps to member x or x + 1
         const int2 sp = P.v_span[v_begin];
-        const int32_t hb = sp.x, len = sp.y;
-        const int pmu = warp_lower_bound(P.he_mem + hb, len, mu);
         const Need nd = need[0];
         if (nd.h >= nd.n) {
-            for (int x = lane; x < len - 1; x += 32)
-                sink.push((uint32_t)P.he_mem[hb + x + (x >= pmu ? 1 : 0)]);
+            for (int x = lane; x < sp.y - 1; x += 32) sink.push(single_member(P, sp.x, x, mu));
         } else {
-            for (uint32_t r = lane; r < nd.h; r += 32) {
-                const uint32_t x = picks[r];
-                sink.push((uint32_t)P.he_mem[hb + x + ((int)x >= pmu ? 1 : 0)]);
-            }
+            for (uint32_t r = lane; r < nd.h; r += 32) sink.push(single_member(P, sp.x, (int)picks[r], mu));
         }
         __syncwarp();
         return false;
@@ -1542,7 +1640,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_forward(FwdParams F) {
         __syncthreads();
         for (;;) {
             int idx = 0;
-            if (lane == 0) idx = claim_slot(P, S, (int64_t)r);
+            int take = 1;
+            if (lane == 0) idx = claim_slot(P, S, (int64_t)r, take);
             idx = __shfl_sync(0xFFFFFFFFu, idx, 0);
             if (idx < 0) break;
             int32_t u = 0;
@@ -1606,7 +1705,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_forward_flat(FwdParams F) {
         __syncthreads();
         for (;;) {
             int idx = 0;
-            if (lane == 0) idx = claim_slot(P, S, (int64_t)r);
+            int take = 1;
+            if (lane == 0) idx = claim_slot(P, S, (int64_t)r, take);
             idx = __shfl_sync(0xFFFFFFFFu, idx, 0);
             if (idx < 0) break;
             int32_t u = 0;
@@ -1916,21 +2016,35 @@ __device__ __forceinline__ void run_job(const RRParams& P, Shared& S, uint32_t* 
     // the block only meets when every pending pop needs the block path
     for (;;) {
         for (;;) {
-            int idx = 0;
-            if (lane == 0) idx = claim_slot(P, S, job);
+            int idx = 0, take = P.strategy == HYPERIM_STRAT_LT ? 1 : 32;
+            if (lane == 0) idx = claim_slot(P, S, job, take);
             idx = __shfl_sync(0xFFFFFFFFu, idx, 0);
             if (idx < 0) break;
-            int32_t mu = 0;
-            if (lane == 0) mu = slot_value(P, list, idx, job);
-            mu = __shfl_sync(0xFFFFFFFFu, mu, 0);
-            const bool defer = mu >= 0 && pop_warp(P, S, QueueSink{vis, list, &S.ctrl[C_TAIL]}, j, ybase, mu);
+            take = __shfl_sync(0xFFFFFFFFu, take, 0);
+            int32_t mine = -1;
+            if (lane < take) mine = slot_value(P, list, idx + lane, job);
             __syncwarp();
-            if (lane == 0) {
-                if (defer) {
-                    S.deferred[atomicAdd(&S.ctrl[C_NDEF], 1)] = mu;
-                } else {
-                    __threadfence_block();  // this pop's pushes before its completion
-                    atomicAdd(&S.ctrl[C_DONE], 1);
+            const QueueSink sink{vis, list, &S.ctrl[C_TAIL]};
+            uint32_t todo = 1u;  // lanes whose pop is the warp's
+            if (take > 1) {
+                todo = pop_lanes(P, S, sink, j, ybase, mine);
+                __syncwarp();
+                if (lane == 0) {
+                    __threadfence_block();  // the pops' pushes before their completion
+                    atomicAdd(&S.ctrl[C_DONE], take - __popc(todo));
+                }
+            }
+            for (; todo; todo &= todo - 1) {
+                const int32_t mu = __shfl_sync(0xFFFFFFFFu, mine, __ffs(todo) - 1);
+                const bool defer = mu >= 0 && pop_warp(P, S, sink, j, ybase, mu);
+                __syncwarp();
+                if (lane == 0) {
+                    if (defer) {
+                        S.deferred[atomicAdd(&S.ctrl[C_NDEF], 1)] = mu;
+                    } else {
+                        __threadfence_block();  // this pop's pushes before its completion
+                        atomicAdd(&S.ctrl[C_DONE], 1);
+                    }
                 }
             }
         }

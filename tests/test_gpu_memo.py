@@ -59,3 +59,39 @@ def test_memo_changes_no_set(H, name, model, p):
         (s1, r1), = H.hyperim_select_seeds_batch(qa)
         (s2, r2), = H.hyperim_select_seeds_batch(qb)
         assert s1.tolist() == s2.tolist() and r1["lambda_r1"].tolist() == r2["lambda_r1"].tolist()
+
+
+def layered_crowd(layers, copies):
+    """`copies` hubs with `layers` layers each (one vertex a layer) in one connected graph."""
+    hes = []
+    for c in range(copies):
+        b = c * (layers + 1)
+        hes += [[b, *range(b + j, b + layers + 1)] for j in range(1, layers + 1)]
+    n = copies * (layers + 1)
+    return n, hes + [[v, (v * 7 + 3) % n] for v in range(n)]
+
+
+LANES = {
+    "random": lambda: G.random_graph(4, 4000, 3000, 9),
+    "layers8": lambda: layered_crowd(8, 300),
+    "layers9": lambda: layered_crowd(9, 300),
+    "large": lambda: (3000, [list(range(3000)), [0, 1, 2]]),
+}
+
+
+@pytest.mark.parametrize("name", sorted(LANES))
+@pytest.mark.parametrize("p", [0.02, 0.3, 0.9])
+@pytest.mark.parametrize("roots", ["plain", "stratified"])
+def test_lane_pops_equal_oracle(H, oracle, name, p, roots):
+    """Sets with long queues, popped lane by lane: one and several layers around the 8 a lane draws, layers
+    taken whole and picks around the 7 a lane makes, kept neighbourhoods and single hyperedges."""
+    n, hes = LANES[name]()
+    off, mem = G.csr(hes)
+    p = p / 100 if name == "large" else p
+    g = H.Graph(n, off, mem, "uniform_pair", int(p * G.P32), seed=9)
+    og = oracle.Graph(n, off, mem, "uniform_pair", int(p * G.P32))
+    pool = g.pool(tag=0, roots=roots).sample(40)
+    op = oracle.Pool(og, seed=9, tag=0, roots=roots)
+    op.grow_theta(40)
+    G.assert_same_pool(pool, op)
+    G.assert_same_counters(pool, op)
