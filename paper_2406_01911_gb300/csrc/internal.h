@@ -110,6 +110,7 @@ struct Scratch {
     int32_t* arena = nullptr;
     size_t arena_cap = 0;        // entries
     // neighbourhoods kept within one growth step (see Memo in rr.cu); optional
+    double* bin_p0 = nullptr;    // per profile entry: P(h = 0) of the Binomial strategy (see binomial_h)
     uint32_t* memo_slot = nullptr;  // n words
     uint32_t* memo = nullptr;
     size_t memo_cap = 0;         // entries

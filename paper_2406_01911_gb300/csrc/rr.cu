@@ -118,6 +118,7 @@ struct RRParams {
     RRCounters* counters;                    // kMaxPools entries
     int spin_limit;                          // rounds of a bounded wait before it gives up
     unsigned long long* set_cycles;          // optional {sum, max, count} of per-set SM cycles
+    double* bin_p0;           // per profile entry: P(h = 0) of the Binomial strategy, or null
     uint32_t* memo_slot;      // neighbourhoods kept within this growth step (see Memo), or null
     uint32_t* memo;
     uint64_t memo_cap;
@@ -189,9 +190,10 @@ __device__ __forceinline__ void dev_fail(DevStatus* st, int32_t code, int32_t de
 // h for one layer (lane-level) from its two profile words and its CDF table. Returns whether a
 // draw was made (0 < p < 1). The draw is decided by integer compares against the layer's table
 // (T_0 first, which sits in the entry); only words beyond the table's last threshold run the
-// double-precision inversion.
+// double-precision inversion. So does every draw of the Binomial strategy on a layer that the paper
+// draws by Poisson: its P(0), in p0 (or null), is kept for the handle's later draws.
 __device__ __forceinline__ bool layer_draw(const uint4 e, const uint4 f, const uint32_t* __restrict__ tab,
-                                          int strategy, WordStream& ws, uint32_t& h, uint32_t& ksel) {
+                                          int strategy, WordStream& ws, uint32_t& h, uint32_t& ksel, double* p0) {
     const uint32_t n_i = e.y, thr = e.z;
     ksel = 0;
     if (e.x & kPOneFlag) { h = n_i; return false; }
@@ -218,7 +220,7 @@ __device__ __forceinline__ bool layer_draw(const uint4 e, const uint4 f, const u
         h = sum > n_i ? n_i : (uint32_t)sum;
         return true;
     }
-    h = binomial_h(n_i, thr, w0);  // Binomial strategy on a layer the paper draws by Poisson
+    h = binomial_h(n_i, thr, w0, p0);  // Binomial strategy on a layer the paper draws by Poisson
     ksel = 1;
     return true;
 }
@@ -891,7 +893,7 @@ __device__ uint32_t pop_lanes(const RRParams& P, SM& S, const Sink& sink, uint32
         WordStream ws;
         ws.init(P.seed, j, ybase, (uint32_t)mu, (uint32_t)(i + 1));
         uint32_t h = 0, ksel = 0;
-        draws += layer_draw(e, f, P.tab, P.strategy, ws, h, ksel) ? 1u : 0u;
+        draws += layer_draw(e, f, P.tab, P.strategy, ws, h, ksel, P.bin_p0 ? P.bin_p0 + vi.x + i : nullptr) ? 1u : 0u;
         if (h == 0) continue;
         const uint32_t n = e.y;
         if (!direct || (h < n ? h > kLanePicks || ksel > 64 : n > kLaneAll)) {
@@ -986,7 +988,7 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
             f = P.prof[2 * (pb + i) + 1];
             WordStream ws;
             ws.init(P.seed, j, ybase, (uint32_t)mu, (uint32_t)(i + 1));
-            drew = layer_draw(e, f, P.tab, P.strategy, ws, h, ksel);
+            drew = layer_draw(e, f, P.tab, P.strategy, ws, h, ksel, P.bin_p0 ? P.bin_p0 + pb + i : nullptr);
         }
         const bool flag = h > 0;
         const uint32_t bal = __ballot_sync(0xFFFFFFFFu, flag);
@@ -1351,7 +1353,7 @@ __device__ __noinline__ void pop_block(const RRParams& P, Shared& S, const Sink&
                     const uint4 f = P.prof[2 * (pb + i) + 1];
                     WordStream ws;
                     ws.init(P.seed, j, ybase, (uint32_t)mu, (uint32_t)(i + 1));
-                    layer_draw(e, f, P.tab, P.strategy, ws, h, ksel);
+                    layer_draw(e, f, P.tab, P.strategy, ws, h, ksel, P.bin_p0 ? P.bin_p0 + pb + i : nullptr);
                 }
                 const bool flag = h > 0;
                 const uint32_t bal = __ballot_sync(0xFFFFFFFFu, flag);
@@ -2354,7 +2356,8 @@ hyperim_status ensure_scratch(hyperim_graph* g, int blocks, bool vis_smem) {
     if (S.bitmap) dev_free(g, S.bitmap, sizeof(uint32_t) * S.bitmap_words * S.blocks);
     if (S.picks) dev_free(g, S.picks, sizeof(uint32_t) * S.pick_cap * S.blocks);
     if (S.big) dev_free(g, S.big, sizeof(uint32_t) * S.big_cap * S.blocks);
-    S = Scratch{0, 0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, S.arena, S.arena_cap, S.memo_slot, S.memo, S.memo_cap};
+    S = Scratch{0, 0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, S.arena, S.arena_cap, S.bin_p0,
+                S.memo_slot, S.memo, S.memo_cap};
     hyperim_status st;
     if ((st = dev_alloc(g, (void**)&S.list, sizeof(int32_t) * list_cap * blocks))) return st;
     HYP_CUDA(cudaMemsetAsync(S.list, 0xFF, sizeof(int32_t) * list_cap * blocks, g->stream));  // empty slots
@@ -2369,6 +2372,18 @@ hyperim_status ensure_scratch(hyperim_graph* g, int blocks, bool vis_smem) {
     S.bitmap_words = vis_words;
     S.pick_cap = pick_cap;
     S.big_cap = big_cap;
+    return HYPERIM_OK;
+}
+
+// The handle's kept P(0) values (Binomial strategy), all unknown at first. Not under a budget, and not
+// without the memory: the draws then find P(0) each time.
+hyperim_status ensure_bin_p0(hyperim_graph* g, int32_t strategy) {
+    Scratch& S = g->scratch;
+    if (strategy != HYPERIM_STRAT_BINOMIAL_ONLY || S.bin_p0 || graph_root(g)->budget || g->profile_entries == 0)
+        return HYPERIM_OK;
+    const size_t bytes = sizeof(double) * (size_t)g->profile_entries;
+    if (dev_alloc(g, (void**)&S.bin_p0, bytes) != HYPERIM_OK) return HYPERIM_OK;
+    HYP_CUDA(cudaMemsetAsync(S.bin_p0, 0xFF, bytes, g->stream));
     return HYPERIM_OK;
 }
 
@@ -2570,6 +2585,7 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     if ((st = ensure_scratch(g, blocks, vis_smem))) return st;
     const bool use_memo = memo_pays(g, pools, npools, pool_start);
     if (use_memo) ensure_memo(g, njobs);
+    if ((st = ensure_bin_p0(g, pools[0]->strategy))) return st;
 
     const uint64_t want = arena_want(g, pools, npools, pool_start, g->n);
     // the warp phase (one RR set per warp) runs first in the persistent schedule, unless the
@@ -2680,6 +2696,7 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     P.rewrite = 0;
     HYP_CUDA(cudaMemsetAsync(d_ctrl, 0, sizeof(Ctrl), s));
     HYP_CUDA(cudaMemsetAsync(g->d_counters, 0, sizeof(RRCounters) * kMaxPools, s));
+    P.bin_p0 = P.strategy == HYPERIM_STRAT_BINOMIAL_ONLY ? g->scratch.bin_p0 : nullptr;
     P.memo_slot = use_memo ? g->scratch.memo_slot : nullptr;
     P.memo = g->scratch.memo;
     P.memo_cap = g->scratch.memo_cap;
@@ -2801,6 +2818,7 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
         deg_max = std::max<int64_t>(deg_max, G.g->max_deg);
         tsum_max = std::max<int64_t>(tsum_max, G.g->max_tsum);
         if (std::find(streams.begin(), streams.end(), G.g->stream) == streams.end()) streams.push_back(G.g->stream);
+        if ((st = ensure_bin_p0(G.g, G.pools[0]->strategy))) return st;
     }
     const int64_t njobs = gstart[ngroups];
     if (njobs == 0) return HYPERIM_OK;
@@ -2900,6 +2918,7 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
         P.root_mode = G.pools[0]->root_mode;
         P.strategy = G.pools[0]->strategy;
         P.npools = G.npools;
+        P.bin_p0 = P.strategy == HYPERIM_STRAT_BINOMIAL_ONLY ? G.g->scratch.bin_p0 : nullptr;
         for (int i = 0; i <= G.npools; ++i) P.pool_start[i] = pstart[(size_t)q * (kMaxPools + 1) + i];
         for (int i = 0; i < G.npools; ++i) {
             P.tags[i] = G.pools[i]->tag;
