@@ -52,6 +52,11 @@ constexpr int kLaneMin = 4;
 constexpr int kLaneMaxDh = 1 << 20, kLaneMaxT = 1 << 26;  // keep the warp's 32-bit sums of counters exact
 // warp phase: a warp builds a whole RR set alone while it stays within kWQ members
 constexpr int kWQ = 128;               // per-warp queue (members of the warp's set)
+// without a tuned limit, sets of this mean size or less so far start in the warp phase: a block per set
+// leaves most of its warps idle on a set of a few members, and its barriers and output cost more than such a
+// set. Mean 1.7 members: the tiny query 0.85 -> 0.46 ms; mean 37: 27.9 -> 25.8 ms; mean 90 (2M vertices,
+// largest 12,000): 251 -> 243 ms. At a mean of 13,000 half of the sets would be begun twice.
+constexpr double kSmallMean = 200.0;
 constexpr int kWHashBits = 8;
 constexpr int kWHash = 1 << kWHashBits;  // per-warp open-addressing member set
 // path phase (LT sets): the warp's member set and queue in global memory
@@ -1889,8 +1894,8 @@ __global__ void __launch_bounds__(kPThreads, 2) k_rr_warp(RRParams P) {
         __syncwarp();
         if (lane < kNStat) wst[lane] = 0;
         for (int i = lane; i < (1 << hash_bits); i += 32) hash[i] = -1;
-        if (P.path && !escalate && lane == 0) {
-            // an SM holds 2 kPWarps paths at once: a set's share of its SM's time
+        if (!escalate && lane == 0) {
+            // an SM holds 2 kPWarps such sets at once: a set's share of its SM's time
             const unsigned long long d = (unsigned long long)(clock64() - cyc0);
             atomicAdd(&S.cyc[0], d / (2 * kPWarps));
             atomicMax(&S.cyc[1], d);
@@ -1899,7 +1904,7 @@ __global__ void __launch_bounds__(kPThreads, 2) k_rr_warp(RRParams P) {
         __syncwarp();
     }
     __syncthreads();
-    if (threadIdx.x == 0 && P.path && P.set_cycles && S.cyc[2]) {
+    if (threadIdx.x == 0 && P.set_cycles && S.cyc[2]) {
         atomicAdd(P.set_cycles, S.cyc[0]);
         atomicMax(P.set_cycles + 1, S.cyc[1]);
         atomicAdd(P.set_cycles + 2, S.cyc[2]);
@@ -2590,7 +2595,15 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     const uint64_t want = arena_want(g, pools, npools, pool_start, g->n);
     // the warp phase (one RR set per warp) runs first in the persistent schedule, unless the
     // graph's tuning turned it off; its grid
-    bool warp_phase = g->schedule != HYPERIM_SCHED_PLAIN && g->warp_set_limit > 0;
+    // the sets' mean size so far, when every pool's is known
+    double mean = 0.0;
+    for (int q = 0; q < npools; ++q) {
+        const double hint = pools[q]->mean_size_hint > 0 ? pools[q]->mean_size_hint : g->set_size_hint;
+        mean = hint > 0 && mean >= 0 ? std::max(mean, hint) : -1.0;
+    }
+    int32_t warp_limit = g->warp_set_limit;
+    if (warp_limit == 0 && mean > 0.0 && mean <= kSmallMean && pools[0]->strategy != HYPERIM_STRAT_LT) warp_limit = kWQ;
+    bool warp_phase = g->schedule != HYPERIM_SCHED_PLAIN && warp_limit > 0;
     // LT sets are single paths: without a tuned warp phase they take the path phase
     bool path_phase = g->schedule != HYPERIM_SCHED_PLAIN && !warp_phase && pools[0]->strategy == HYPERIM_STRAT_LT;
     int wblocks = 0;
@@ -2659,7 +2672,7 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     P.esc_count = &d_ctrl->esc_count;
     P.esc_list = d_esc;
     P.block_phase = 0;
-    P.warp_limit = path_phase ? 1 << (path_bits - 1) : std::min(std::max(g->warp_set_limit, 1), kWQ);
+    P.warp_limit = path_phase ? 1 << (path_bits - 1) : std::min(std::max(warp_limit, 1), kWQ);
     P.path = d_path;
     P.path_bits = path_bits;
     P.plain = g->schedule == HYPERIM_SCHED_PLAIN ? 1 : 0;
