@@ -201,17 +201,33 @@ __global__ void k_retire(const int32_t* __restrict__ best, const int64_t* __rest
 //     the argmax reads 8 bytes per active vertex;
 //   - a picked vertex needs no flag, its score is 0 once its sets are retired; when the best score is
 //     0 the rest of the seeds are the lowest ids not picked yet;
-//   - all rounds run in one cooperative launch (its blocks are resident together by the launch's
-//     contract) with two barriers a round; block winners are reduced by every block for itself, so
-//     the winner needs no third one. The barrier's wait is bounded (kErrSpin).
-// A block for every 16K members of the pool, one block (no barrier) for small pools. 200 rounds on the pools
-// of 40,000 sets of that graph: 4.0 ms before, 2.7 ms now (14 us a round: two barriers and a chain of
-// about ten dependent L2 reads); the index build 0.42 -> 0.14 ms with long sets spread over blocks. The
-// Eq. upper_2 bound took 17 launches a round (35 ms of a 100 ms query), now none of its own.
+//   - all rounds run in one launch with two barriers a round; block winners are reduced by every block
+//     for itself, so the winner needs no third one. Up to kGClusterMembers members in the pool the launch
+//     is one cluster of kGCluster blocks: its barrier is the hardware's and the block winners go straight
+//     into the other blocks' shared memory. Larger pools (a round may retire tens of millions of
+//     members) take a block for every 16K members, resident together by the contract of a cooperative
+//     launch, with a barrier in global memory whose wait is bounded (kErrSpin); the smallest pools one block
+//     and no barrier at all;
+//   - in a cluster the argmax looks at candidates only: the vertices whose score is at least that of the
+//     kCand-th largest, found once by the radix select below, one per thread, which keeps its vertex and
+//     its index range in registers: what is left of an argmax is one read of a score. Scores only
+//     decrease, so while the best candidate still reaches that threshold it is the best of all (every
+//     vertex at the threshold is a candidate, so ties are settled among them); when it does not, one
+//     round looks at every active vertex and the candidates are chosen anew. (A grid of 152 blocks loses
+//     more in the select's histograms than it gains: 106 -> 112 ms on the 100k query.)
+// 200 seeds chosen on the pools of 40,000 sets of that graph, with the estimate: 4.9 ms with two launches a
+// round, 4.0 ms with a cooperative launch over 152 blocks and no candidates, 3.3 ms so (k_greedy itself 2.7
+// and 2.2 ms: a round is still a chain of six or seven dependent L2 reads); the index build 0.42 -> 0.14 ms
+// with long sets spread over blocks. The Eq. upper_2 bound took 17 launches a round (35 ms of a 100 ms
+// query), now none of its own. Above 4M members a cluster's 16 SMs lose: a pool of 8M (608 sets of a third
+// of 100k vertices) retires nearly all of them in its first round.
 constexpr int kGThreads = 512;
 constexpr int kGWarps = kGThreads / 32;
 constexpr int64_t kGMembersPerBlock = 1 << 14;
 constexpr int kGSpin = 1 << 24;  // rounds of a barrier wait (seconds) before it gives up
+constexpr int kGCluster = 16;
+constexpr int64_t kGClusterMembers = 1 << 22;
+constexpr unsigned int kCand = 4096, kCandCap = kGCluster * kGThreads;  // at most one per thread
 constexpr int kTopBits = 11;
 constexpr int kTopBins = 1 << kTopBits;
 
@@ -359,6 +375,8 @@ struct GreedyParams {
     Weights W;
     int32_t n, k;
     int prefix;                  // 1: also the Eq. upper_2 bound of every prefix of the seeds
+    uint32_t* cand;              // kCandCap numbers
+    unsigned int* ncand;
     unsigned long long* pscore;  // per block
     uint32_t* pid;               // per block: vertex, number
     unsigned long long* psum;    // per block: 128-bit partial sums
@@ -368,8 +386,14 @@ struct GreedyParams {
 };
 
 // All blocks of the launch meet; false when the bounded wait gave up here.
+template <bool kCluster>
 __device__ bool grid_meet(const GreedyParams& P, unsigned int& target) {
     __shared__ int ok_s;
+    if (kCluster) {  // the cluster's barrier: what a block wrote before is seen by the others after
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        return true;
+    }
     __syncthreads();
     if (gridDim.x == 1) return true;
     if (threadIdx.x == 0) {
@@ -389,6 +413,24 @@ __device__ bool grid_meet(const GreedyParams& P, unsigned int& target) {
     return ok_s != 0;
 }
 
+// a block's winner: score, vertex, its range of the index (end = 0: not known)
+struct Winner {
+    unsigned long long score;
+    int64_t begin, end;
+    uint32_t v, pad;
+};
+
+// w into block `rank`'s copy of the shared array `to`, at this block's place (one cluster)
+__device__ __forceinline__ void send_winner(Winner* to, unsigned int rank, const Winner& w) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(to + blockIdx.x);
+    uint32_t ra;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(ra), "l"(w.score) : "memory");
+    asm volatile("st.shared::cluster.u64 [%0 + 8], %1;" ::"r"(ra), "l"(w.begin) : "memory");
+    asm volatile("st.shared::cluster.u64 [%0 + 16], %1;" ::"r"(ra), "l"(w.end) : "memory");
+    asm volatile("st.shared::cluster.u32 [%0 + 24], %1;" ::"r"(ra), "r"(w.v) : "memory");
+}
+
 __device__ __forceinline__ void add128(unsigned long long& lo, unsigned long long& hi, unsigned long long a_lo,
                                        unsigned long long a_hi) {
     const unsigned long long l = lo + a_lo;
@@ -396,21 +438,20 @@ __device__ __forceinline__ void add128(unsigned long long& lo, unsigned long lon
     lo = l;
 }
 
-// Eq. upper_2 (p_max = 1) for the seeds so far: cover plus the sum of the k largest scores (a picked or
-// inactive vertex counts 0), entered into block 0's running minimum. A radix select over 11-bit digits
-// below the largest score `top`, most significant first, finds the k-th largest score T and how
-// many of its copies belong to the top k; a digit of 0 is never counted (most scores have it), it is
-// what is left when the others hold fewer than k. Three histograms rotate: the next one is cleared
-// between the barriers that separate its last readers from its next writers.
-__device__ bool topk_bound(const GreedyParams& P, unsigned int na, unsigned long long top, unsigned long long cover,
-                           unsigned int* h, int& turn, unsigned int& target, unsigned long long& best_lo,
-                           unsigned long long& best_hi) {
-    __shared__ unsigned long long slo[kGWarps], shi[kGWarps];
+// The want-th largest score `kth` and how many of its copies are among the want largest (kleft; fewer
+// scores than want: kth = 0). A radix select over 11-bit digits below the largest score `top`, most
+// significant first; a digit of 0 is never counted (most scores have it), it is what is left when the
+// others hold too few. Three histograms rotate: the next one is cleared between the barriers that
+// separate its last readers from its next writers.
+template <bool kCluster>
+__device__ bool kth_score(const GreedyParams& P, unsigned int na, unsigned long long top, unsigned int want,
+                          unsigned int* h, int& turn, unsigned int& target, unsigned long long& kth,
+                          unsigned int& kleft) {
     __shared__ unsigned int digit_s, left_s;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t t0 = blockIdx.x * (int64_t)kGThreads + threadIdx.x, T = (int64_t)gridDim.x * kGThreads;
     unsigned long long prefix = 0;
-    unsigned int kleft = (unsigned int)P.k;
+    kleft = want;
     const int bits = top ? 64 - __clzll((long long)top) : 0;
     for (int sh = ((bits + kTopBits - 1) / kTopBits - 1) * kTopBits; sh >= 0; sh -= kTopBits) {
         unsigned int* hist = P.hist + turn * kTopBins;
@@ -429,7 +470,7 @@ __device__ bool topk_bound(const GreedyParams& P, unsigned int na, unsigned long
         __syncthreads();
         for (int i = threadIdx.x; i < kTopBins; i += kGThreads)
             if (h[i]) atomicAdd(&hist[i], h[i]);
-        if (!grid_meet(P, target)) return false;
+        if (!grid_meet<kCluster>(P, target)) return false;
         if (wid == 0) {  // lane i: digits [64 i, 64 i + 64), from the highest lane down
             constexpr int per = kTopBins / 32;
             unsigned int sum = 0;
@@ -463,6 +504,22 @@ __device__ bool topk_bound(const GreedyParams& P, unsigned int na, unsigned long
         turn = next;
         __syncthreads();
     }
+    kth = prefix;
+    return true;
+}
+
+// Eq. upper_2 (p_max = 1) for the seeds so far: cover plus the sum of the k largest scores (a picked or
+// inactive vertex counts 0), entered into block 0's running minimum.
+template <bool kCluster>
+__device__ bool topk_bound(const GreedyParams& P, unsigned int na, unsigned long long top, unsigned long long cover,
+                           unsigned int* h, int& turn, unsigned int& target, unsigned long long& best_lo,
+                           unsigned long long& best_hi) {
+    __shared__ unsigned long long slo[kGWarps], shi[kGWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t t0 = blockIdx.x * (int64_t)kGThreads + threadIdx.x, T = (int64_t)gridDim.x * kGThreads;
+    unsigned long long prefix = 0;
+    unsigned int kleft = 0;
+    if (!kth_score<kCluster>(P, na, top, (unsigned int)P.k, h, turn, target, prefix, kleft)) return false;
     unsigned long long lo = 0, hi = 0;
     for (int64_t c = t0; c < na; c += T) {
         const unsigned long long x = __ldcg(P.score + c);
@@ -480,7 +537,7 @@ __device__ bool topk_bound(const GreedyParams& P, unsigned int na, unsigned long
         P.psum[2 * blockIdx.x] = lo;
         P.psum[2 * blockIdx.x + 1] = hi;
     }
-    if (!grid_meet(P, target)) return false;
+    if (!grid_meet<kCluster>(P, target)) return false;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         lo = hi = 0;
         for (unsigned int b = 0; b < gridDim.x; ++b) add128(lo, hi, __ldcg(P.psum + 2 * b), __ldcg(P.psum + 2 * b + 1));
@@ -494,10 +551,14 @@ __device__ bool topk_bound(const GreedyParams& P, unsigned int na, unsigned long
     return true;
 }
 
-__global__ void __launch_bounds__(kGThreads) k_greedy(GreedyParams P) {
+template <bool kCluster>
+__global__ void __launch_bounds__(kGThreads, 1) k_greedy(GreedyParams P) {
+    __shared__ Winner winners[kGCluster];  // the blocks' winners (one cluster)
+    __shared__ Winner mine_s;              // this block's
+    __shared__ int64_t win_b, win_e;
     __shared__ unsigned long long s_lam[HYPERIM_NSTRATA];
     __shared__ unsigned long long ss[kGWarps];
-    __shared__ uint32_t si[kGWarps], sc[kGWarps];
+    __shared__ uint32_t si[kGWarps];
     __shared__ unsigned long long win_s;
     __shared__ uint32_t win_v;
     __shared__ unsigned int h[kTopBins];
@@ -511,6 +572,10 @@ __global__ void __launch_bounds__(kGThreads) k_greedy(GreedyParams P) {
     if (threadIdx.x < HYPERIM_NSTRATA) s_lam[threadIdx.x] = 0;
     __syncthreads();
     int32_t round = 0;
+    unsigned int nc = 0;            // candidates (0: none, every active vertex is looked at)
+    unsigned long long floor = 0;   // every other vertex scores less than this
+    uint32_t own_c = 0, own_v = 0xFFFFFFFFu;  // this thread's candidate: number, vertex, index range
+    int64_t own_b = 0, own_e = 0;
     for (;; ++round) {
         if (round == P.k && !P.prefix) break;
         // the best (score, lowest id): per block, then over the blocks' winners by every block
@@ -522,17 +587,7 @@ __global__ void __launch_bounds__(kGThreads) k_greedy(GreedyParams P) {
                 if (better(x, v, bs, bi)) { bs = x; bi = v; }
             }
         };
-        const int64_t na4 = na >> 2;
-        for (int64_t q = t0; q < na4; q += T) {
-            const ulonglong2 a = __ldcg(reinterpret_cast<const ulonglong2*>(P.score) + 2 * q);
-            const ulonglong2 b = __ldcg(reinterpret_cast<const ulonglong2*>(P.score) + 2 * q + 1);
-            take(a.x, 4 * q);
-            take(a.y, 4 * q + 1);
-            take(b.x, 4 * q + 2);
-            take(b.y, 4 * q + 3);
-        }
-        for (int64_t c = 4 * na4 + t0; c < na; c += T) take(__ldcg(P.score + c), c);
-        auto reduce = [&]() {  // over the block; the result is thread 0's
+        auto reduce = [&]() {  // over the block; the result is warp 0's
             for (int o = 16; o > 0; o >>= 1) {
                 const unsigned long long os = __shfl_xor_sync(0xFFFFFFFFu, bs, o);
                 const uint32_t oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
@@ -550,30 +605,107 @@ __global__ void __launch_bounds__(kGThreads) k_greedy(GreedyParams P) {
                 }
             }
         };
-        reduce();
-        if (gridDim.x > 1) {
-            if (threadIdx.x == 0) {
-                P.pscore[blockIdx.x] = bs;
-                P.pid[blockIdx.x] = bi;
+        auto share = [&]() {  // over the blocks; the result is every thread's, in win_s and win_v
+            reduce();
+            if (kCluster) {
+                if (threadIdx.x == 0) mine_s = Winner{bs, 0, 0, bi, 0u};
+                __syncthreads();
+                if (own_e && own_v == mine_s.v) {
+                    mine_s.begin = own_b;
+                    mine_s.end = own_e;
+                }
+                __syncthreads();
+                if (wid == 0 && lane < (int)gridDim.x) send_winner(winners, (unsigned int)lane, mine_s);
+                if (!grid_meet<kCluster>(P, target)) return false;
+                if (wid == 0) {
+                    bs = lane < (int)gridDim.x ? winners[lane].score : 0ull;
+                    bi = lane < (int)gridDim.x ? winners[lane].v : 0xFFFFFFFFu;
+                    const uint32_t sent = bi;
+                    for (int o = 16; o > 0; o >>= 1) {
+                        const unsigned long long os = __shfl_xor_sync(0xFFFFFFFFu, bs, o);
+                        const uint32_t oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
+                        if (better(os, oi, bs, bi)) { bs = os; bi = oi; }
+                    }
+                    if (lane < (int)gridDim.x && sent == bi && bs) {  // the one block that sent the winner
+                        win_b = winners[lane].begin;
+                        win_e = winners[lane].end;
+                    }
+                }
+            } else if (gridDim.x > 1) {
+                if (threadIdx.x == 0) {
+                    P.pscore[blockIdx.x] = bs;
+                    P.pid[blockIdx.x] = bi;
+                }
+                if (!grid_meet<kCluster>(P, target)) return false;
+                bs = 0;
+                bi = 0xFFFFFFFFu;
+                for (int b = threadIdx.x; b < (int)gridDim.x; b += kGThreads) {
+                    const unsigned long long x = __ldcg(P.pscore + b);
+                    const uint32_t v = __ldcg(P.pid + b);
+                    if (better(x, v, bs, bi)) { bs = x; bi = v; }
+                }
+                reduce();
             }
-            if (!grid_meet(P, target)) return;
+            if (threadIdx.x == 0) {
+                win_s = bs;
+                win_v = bi;
+            }
+            __syncthreads();
+            return true;
+        };
+        bool full = nc == 0;
+        if (kCluster && !full) {
+            if (own_e) {
+                bs = __ldcg(P.score + own_c);
+                if (bs) bi = own_v;
+            }
+            if (!share()) return;
+            full = win_s < floor;
             bs = 0;
             bi = 0xFFFFFFFFu;
-            for (int b = threadIdx.x; b < (int)gridDim.x; b += kGThreads) {
-                const unsigned long long x = __ldcg(P.pscore + b);
-                const uint32_t v = __ldcg(P.pid + b);
-                if (better(x, v, bs, bi)) { bs = x; bi = v; }
+        }
+        if (full) {
+            // the blocks have read the winners above before any of them is written again
+            if (nc && !grid_meet<kCluster>(P, target)) return;
+            own_e = 0;
+            own_v = 0xFFFFFFFFu;
+            const int64_t na4 = na >> 2;
+            for (int64_t q = t0; q < na4; q += T) {
+                const ulonglong2 a = __ldcg(reinterpret_cast<const ulonglong2*>(P.score) + 2 * q);
+                const ulonglong2 b = __ldcg(reinterpret_cast<const ulonglong2*>(P.score) + 2 * q + 1);
+                take(a.x, 4 * q);
+                take(a.y, 4 * q + 1);
+                take(b.x, 4 * q + 2);
+                take(b.y, 4 * q + 3);
             }
-            reduce();
+            for (int64_t c = 4 * na4 + t0; c < na; c += T) take(__ldcg(P.score + c), c);
+            if (!share()) return;
+            nc = 0;
+            if (kCluster && !P.prefix && na > 4 * kCand && P.k - round > 8 && win_s) {
+                unsigned int kleft;
+                if (blockIdx.x == 0 && threadIdx.x == 0) *P.ncand = 0;
+                if (!kth_score<kCluster>(P, na, win_s, kCand, h, turn, target, floor, kleft)) return;
+                if (floor) {
+                    for (int64_t c = t0; c < na; c += T)
+                        if (__ldcg(P.score + c) >= floor) {
+                            const unsigned int at = atomicAdd(P.ncand, 1u);
+                            if (at < kCandCap) P.cand[at] = (uint32_t)c;
+                        }
+                    if (!grid_meet<kCluster>(P, target)) return;
+                    nc = __ldcg(P.ncand);
+                    if (nc > kCandCap) nc = 0;  // too many at the threshold: no candidates
+                    if (t0 < nc) {
+                        own_c = __ldcg(P.cand + t0);
+                        own_v = (uint32_t)P.act[own_c];
+                        own_b = P.inv_off[own_v];
+                        own_e = P.inv_off[own_v + 1];
+                    }
+                }
+            }
         }
-        if (threadIdx.x == 0) {
-            win_s = bs;
-            win_v = bi;
-        }
-        __syncthreads();
         const unsigned long long win = win_s;
         const uint32_t v = win_v;
-        if (P.prefix && !topk_bound(P, na, win, cover, h, turn, target, best_lo, best_hi)) return;
+        if (P.prefix && !topk_bound<kCluster>(P, na, win, cover, h, turn, target, best_lo, best_hi)) return;
         if (round == P.k || win == 0) break;
         cover += win;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -581,9 +713,16 @@ __global__ void __launch_bounds__(kGThreads) k_greedy(GreedyParams P) {
             P.picked[v] = 1;
         }
         // retire the winner's sets that are not covered yet (a set holds it once: one warp finds it)
-        const int64_t b = P.inv_off[v];
+        int64_t b, e;
+        if (kCluster && win_e) {
+            b = win_b;
+            e = win_e;
+        } else {
+            b = P.inv_off[v];
+            e = P.inv_off[v + 1];
+        }
         block_sets(
-            sets, P.inv_off[v + 1] - b,
+            sets, e - b,
             [&](int64_t t, int64_t& x0, int64_t& x1, unsigned long long& tag) {
                 const uint32_t r = P.inv[b + t];
                 x0 = P.rr_off[r];
@@ -599,7 +738,7 @@ __global__ void __launch_bounds__(kGThreads) k_greedy(GreedyParams P) {
                 return true;
             },
             [&](int64_t x, unsigned long long neg) { atomicAdd(&P.score[P.memc[x]], neg); });
-        if (!grid_meet(P, target)) return;
+        if (!grid_meet<kCluster>(P, target)) return;
     }
     __syncthreads();
     if (threadIdx.x < HYPERIM_NSTRATA && s_lam[threadIdx.x]) atomicAdd(&P.out->lam[threadIdx.x], s_lam[threadIdx.x]);
@@ -833,6 +972,35 @@ Limits make_limits(const hyperim_pool* p, const uint64_t* lim, uint64_t view_ns[
 }
 }  // namespace
 
+namespace {
+// one launch of kGCluster blocks as one cluster
+void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, cudaStream_t s) {
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kGCluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(kGCluster);
+    cfg.blockDim = dim3(kGThreads);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+}
+
+// whether the device takes such a cluster (16 blocks is more than the portable 8): asked once
+bool cluster_fits() {
+    static const bool fits = [] {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        cluster_config(cfg, at, nullptr);
+        int clusters = 0;
+        bool ok = cudaFuncSetAttribute(k_greedy<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                  cudaOccupancyMaxActiveClusters(&clusters, k_greedy<true>, &cfg) == cudaSuccess && clusters > 0;
+        if (!ok) cudaGetLastError();
+        return ok;
+    }();
+    return fits;
+}
+}  // namespace
+
 hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* seeds_host,
                       uint64_t lambda_s[HYPERIM_NSTRATA], uint64_t* prefix_upper, const uint64_t* lim) {
     cudaStream_t s = g->stream;
@@ -848,20 +1016,23 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
     hyperim_status st;
     // blocks: by the pool's members, all resident together when more than one
     int blocks = (int)std::min<int64_t>(std::max<int64_t>(T / kGMembersPerBlock, 1), sm);
-    if (blocks > 1) {
+    const bool cluster = blocks > 1 && T <= kGClusterMembers && cluster_fits();
+    if (cluster) {
+        blocks = kGCluster;
+    } else if (blocks > 1) {
         int per_sm = 0;
-        HYP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_greedy, kGThreads, 0));
+        HYP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_greedy<false>, kGThreads, 0));
         blocks = std::max(1, std::min(blocks, per_sm * sm));
     }
     CallBuffers tmp(g);
-    uint32_t *cnt = nullptr, *inv = nullptr, *cidx = nullptr, *memc = nullptr, *pid = nullptr;
+    uint32_t *cnt = nullptr, *inv = nullptr, *cidx = nullptr, *memc = nullptr, *pid = nullptr, *cand = nullptr;
     int64_t* inv_off = nullptr;
     unsigned long long *score = nullptr, *pscore = nullptr, *psum = nullptr;
     int32_t *act = nullptr, *seeds_d = nullptr;
     // cleared together: the output record, barrier, counters, histograms, picked and covered flags
     struct Zero {
         GreedyOut out;
-        unsigned int bar, nact;
+        unsigned int bar, nact, ncand, pad;
         unsigned int hist[3 * kTopBins];
     };
     uint8_t* zero = nullptr;
@@ -878,6 +1049,7 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
     if ((st = tmp.alloc(&zero, bytes_zero))) return st;
     if ((st = tmp.alloc(&pscore, sizeof(unsigned long long) * 3 * (size_t)blocks))) return st;
     if ((st = tmp.alloc(&pid, sizeof(uint32_t) * (size_t)blocks))) return st;
+    if ((st = tmp.alloc(&cand, sizeof(uint32_t) * kCandCap))) return st;
     if ((st = tmp.alloc(&seeds_d, sizeof(int32_t) * (size_t)k))) return st;
     psum = pscore + blocks;
     Zero* z = reinterpret_cast<Zero*>(zero);
@@ -897,12 +1069,18 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
     HYP_CUDA(cudaGetLastError());
     GreedyParams G{act, score, &z->nact, inv_off, inv, p->rr_off, memc, p->rr_stratum,
                    zero + sizeof(Zero) + (size_t)n, zero + sizeof(Zero), seeds_d, &z->out, W, n, k,
-                   prefix_upper ? 1 : 0, pscore, pid, psum, z->hist, &z->bar, g->d_status};
-    if (blocks > 1) {
+                   prefix_upper ? 1 : 0, cand, &z->ncand, pscore, pid, psum, z->hist, &z->bar, g->d_status};
+    if (cluster) {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        cluster_config(cfg, at, s);
+        HYP_CUDA(cudaLaunchKernelEx(&cfg, k_greedy<true>, G));
+    } else if (blocks > 1) {
         void* args[] = {&G};
-        HYP_CUDA(cudaLaunchCooperativeKernel((const void*)k_greedy, dim3((unsigned)blocks), dim3(kGThreads), args, 0, s));
+        HYP_CUDA(cudaLaunchCooperativeKernel((const void*)k_greedy<false>, dim3((unsigned)blocks), dim3(kGThreads), args,
+                                             0, s));
     } else {
-        k_greedy<<<1, kGThreads, 0, s>>>(G);
+        k_greedy<false><<<1, kGThreads, 0, s>>>(G);
     }
     count_launch();
     HYP_CUDA(cudaGetLastError());

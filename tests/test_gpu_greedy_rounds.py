@@ -89,3 +89,19 @@ def test_coverage_on_chip_and_with_flags(H, k, theta):
                                             v["count"], C.c_void_p(sd.data_ptr() if k else None), k,
                                             C.c_void_p(lam.data_ptr()), C.c_void_p(H.current_stream())) == 0
     assert lam.tolist() == want.tolist()
+
+
+@pytest.mark.parametrize("p,theta", [(0.02, 60000), (0.3, 30000), (0.9, 60), (0.9, 400)])
+@pytest.mark.parametrize("roots", ["plain", "stratified"])
+def test_candidates_give_the_stepwise_picks(H, p, theta, roots):
+    """Enough vertices for candidates: scores that fall slowly, and (one giant component, p = 0.9) to
+    nothing after the first picks, so that the candidates have to be chosen anew; pools of one cluster and
+    of a grid. The stepwise greedy looks at every vertex in every round."""
+    n, hes = G.random_graph(11, 60_000, 60_000, 5)
+    g = H.Graph(n, *G.csr(hes), "uniform_pair", int(p * G.P32), seed=6)
+    pool = g.pool(tag=0, roots=roots).sample(theta)
+    k = 120
+    seeds, res = g.select_seeds(pool, None, k, mode="fixed")
+    rounds = H.GreedyRounds(g, pool)
+    assert seeds.tolist() == [rounds.pick() for _ in range(k)]
+    assert res["lambda_r1"].tolist() == rounds.end().tolist()
