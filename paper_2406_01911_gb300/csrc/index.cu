@@ -11,9 +11,9 @@
 // Build (after the layer profile):
 //   k_idx_candidates  vertices with d_H >= 2, more than kIdxMinT members besides mu, l <= kIdxMaxL
 //   k_idx_plan        per candidate: the expected picks per pop decide the chunk target (or
-//                     no index); histogram of the members over 2^hb id bins (hb = min(12, id
-//                     bits)); c = the fewest bits for which no chunk holds more than the target
-//                     (0 bits: not indexed); entries = l 2^c
+//                     no index); c = the fewest bits for which no chunk holds more than the target
+//                     (0 bits: not indexed), found by the layer profile on its sorted members (a pass
+//                     over the members of its own took 8.7 ms of a 2M-vertex load); entries = l 2^c
 //   scan              table offsets
 //   k_idx_fill        per indexed vertex: members sorted by id on chip (bucketed through a global
 //                     scratch area when large), runs (multiplicity w -> layer) counted per
@@ -28,7 +28,6 @@
 namespace hyperim {
 namespace {
 
-constexpr int kThreads = 256;
 constexpr int kBins = 1 << kIdxMaxBits;
 
 __device__ __forceinline__ void dev_fail(DevStatus* st, int32_t code, int32_t detail) {
@@ -71,83 +70,27 @@ __device__ void warp0_exclusive_scan(int* a, int count) {
     }
 }
 
-__global__ void __launch_bounds__(kThreads)
-k_idx_plan(const int32_t* __restrict__ list, int32_t nlist, const int32_t* __restrict__ order,
-           int* __restrict__ next, const int4* __restrict__ vinfo,
-           const int2* __restrict__ v_span, const int32_t* __restrict__ he_mem,
-           const int32_t* __restrict__ tsum, const uint4* __restrict__ prof, int id_bits,
-           uint8_t* __restrict__ bits_out, uint32_t* __restrict__ entries) {
-    __shared__ int hist_a[kBins];
-    __shared__ int hist_b[kBins / 2];
-    __shared__ int pre[2 * kThreads + 1];
-    __shared__ int wmax[kThreads / 32];
-    __shared__ int target_s, ticket_s;
-    const int hb = id_bits < kIdxMaxBits ? id_bits : kIdxMaxBits;
-    const int shift = id_bits - hb;
-    for (;;) {
-        // candidates largest first, from a counter
-        if (threadIdx.x == 0) ticket_s = atomicAdd(next, 1);
-        __syncthreads();
-        const int ticket = ticket_s;
-        __syncthreads();
-        if (ticket >= nlist) break;
-        const int i = order[ticket];
+__global__ void k_idx_plan(const int32_t* __restrict__ list, int32_t nlist, const int4* __restrict__ vinfo,
+                           const int32_t* __restrict__ tsum, const uint4* __restrict__ prof,
+                           const uint8_t* __restrict__ chunk_bits, uint8_t* __restrict__ bits_out,
+                           uint32_t* __restrict__ entries) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nlist; i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t mu = list[i];
         const int4 vi = vinfo[mu];
-        if (threadIdx.x == 0) {
-            // expected picks per pop, sum_i n_i p_i, against kIdxFewPicks on the integers
-            // n_i floor(p_i 2^32) (p = 1 counts 2^32), stopping once the bound is reached
-            const unsigned long long cap = kIdxFewPicks << 32;
-            unsigned long long acc = 0;
-            for (int q = 0; q < vi.y && acc < cap; ++q) {
-                const uint4 e = prof[2 * ((int64_t)vi.x + q)];
-                const unsigned long long t = (e.x & kPOneFlag) ? (1ull << 32) : (unsigned long long)e.z;
-                acc += (unsigned long long)e.y * t;
-            }
-            const bool few = acc < cap;
-            const int T = tsum[mu] - vi.w;
-            target_s = few ? kIdxTargetFew : (T > kIdxMinTMany ? kIdxTargetMany : 0);
+        // expected picks per pop, sum_i n_i p_i, against kIdxFewPicks on the integers
+        // n_i floor(p_i 2^32) (p = 1 counts 2^32), stopping once the bound is reached
+        const unsigned long long cap = kIdxFewPicks << 32;
+        unsigned long long acc = 0;
+        for (int q = 0; q < vi.y && acc < cap; ++q) {
+            const uint4 e = prof[2 * ((int64_t)vi.x + q)];
+            const unsigned long long t = (e.x & kPOneFlag) ? (1ull << 32) : (unsigned long long)e.z;
+            acc += (unsigned long long)e.y * t;
         }
-        __syncthreads();
-        const int target = target_s;
-        __syncthreads();
-        if (target == 0) {  // many picks on a neighbourhood one warp sorts whole: no index
-            if (threadIdx.x == 0) {
-                bits_out[i] = 0;
-                entries[i] = 0;
-            }
-            continue;
-        }
-        for (int b = threadIdx.x; b < (1 << hb); b += kThreads) hist_a[b] = 0;
-        __syncthreads();
-        for_each_member<kThreads>(v_span, he_mem, mu, vi.z, vi.w, pre,
-                                  [&](uint32_t x) { atomicAdd(&hist_a[x >> shift], 1); });
-        __syncthreads();
-        int* hist = hist_a;
-        int* half = hist_b;
-        // level c = hb down to 1: the largest chunk at c bits; pairs are merged for c - 1
-        int best = 0;
-        for (int c = hb; c >= 1; --c) {
-            const int nb = 1 << c;
-            int mx = 0;
-            for (int b = threadIdx.x; b < nb; b += kThreads) mx = max(mx, hist[b]);
-            mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-            if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = mx;
-            __syncthreads();
-            int all = 0;
-            for (int w = 0; w < kThreads / 32; ++w) all = max(all, wmax[w]);
-            if (all <= target) best = c;  // uniform: every thread saw the same maxima
-            for (int b = threadIdx.x; b < nb / 2; b += kThreads) half[b] = hist[2 * b] + hist[2 * b + 1];
-            __syncthreads();
-            int* tmp = hist;
-            hist = half;
-            half = tmp;
-        }
-        if (threadIdx.x == 0) {
-            bits_out[i] = (uint8_t)best;
-            entries[i] = best ? (uint32_t)vi.y << best : 0u;
-        }
-        __syncthreads();
+        const int both = chunk_bits[mu];
+        // many picks on a neighbourhood one warp sorts whole: no index
+        const int best = acc < cap ? both & 15 : tsum[mu] - vi.w > kIdxMinTMany ? both >> 4 : 0;
+        bits_out[i] = (uint8_t)best;
+        entries[i] = best ? (uint32_t)vi.y << best : 0u;
     }
 }
 
@@ -346,7 +289,7 @@ int grid_for(int64_t items, int threads, int sm) {
 
 }  // namespace
 
-hyperim_status build_chunk_index(hyperim_graph* g) {
+hyperim_status build_chunk_index(hyperim_graph* g, const uint8_t* chunk_bits) {
     cudaStream_t s = g->stream;
     const int32_t n = g->n;
     const int sm = g->sm_count;
@@ -378,16 +321,14 @@ hyperim_status build_chunk_index(hyperim_graph* g) {
     if ((st = tmp.alloc(&d_off, sizeof(int64_t) * ((size_t)ncand + 1)))) return st;
     { k_idx_list<<<grid_for(n, 256, sm), 256, 0, s>>>(n, d_flag, d_pos, d_list); count_launch(); }
     const int nl = (int)ncand;
-    // the candidates' indices, largest neighbourhood first (both passes take them in this order)
+    // the candidates' indices, largest neighbourhood first (the fill takes them in this order)
     int32_t* d_order = nullptr;
     int* d_next = nullptr;
     if ((st = tmp.alloc(&d_order, sizeof(int32_t) * (size_t)ncand))) return st;
     if ((st = tmp.alloc(&d_next, sizeof(int)))) return st;
     if ((st = size_order(g, d_list, ncand, true, d_order))) return st;
-    HYP_CUDA(cudaMemsetAsync(d_next, 0, sizeof(int), s));
-    const int pblocks = (int)std::min<int64_t>(ncand, (int64_t)sm * 8);  // 8 x 256 threads per SM
-    { k_idx_plan<<<pblocks, kThreads, 0, s>>>(d_list, nl, d_order, d_next, g->vinfo, g->v_span, g->he_mem, g->tsum,
-                                              g->prof, g->id_bits, d_bits, d_entries); count_launch(); }
+    { k_idx_plan<<<grid_for(ncand, 256, sm), 256, 0, s>>>(d_list, nl, g->vinfo, g->tsum, g->prof, chunk_bits, d_bits,
+                                                        d_entries); count_launch(); }
     if ((st = exclusive_scan_u32_to_i64(g, d_entries, d_off, ncand))) return st;
     int64_t total = 0;
     HYP_CUDA(cudaMemcpyAsync(&total, d_off + ncand, sizeof(int64_t), cudaMemcpyDeviceToHost, s));

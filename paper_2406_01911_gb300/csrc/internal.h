@@ -265,7 +265,9 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off, const int32_
 hyperim_status size_order(hyperim_graph* g, const int32_t* list, int64_t count, bool emit_index, int32_t* out);
 
 // index.cu: chunk index of the vertices with large neighbourhoods (after the layer profile)
-hyperim_status build_chunk_index(hyperim_graph* g);
+// chunk_bits: per vertex, the fewest chunk bits for kIdxTargetFew (low half) and kIdxTargetMany (high half),
+// 0: none; only those of vertices with more than kIdxMinT members are read
+hyperim_status build_chunk_index(hyperim_graph* g, const uint8_t* chunk_bits);
 
 // scan.cu: exclusive scan of n uint32/int32 counts into int64 (out has n + 1 entries)
 hyperim_status exclusive_scan_u32_to_i64(hyperim_graph* g, const uint32_t* in, int64_t* out,

@@ -251,6 +251,30 @@ __device__ void emit_layers(const uint32_t* hist, int dh, int32_t mu, int32_t e0
     }
 }
 
+// Chunk bits of a neighbourhood (see the chunk index) from its sorted members: a chunk of the ids' top c
+// bits holds more than t of them iff some members t places apart agree in their top c bits, so the
+// fewest bits for a target are the most that any such pair needs to differ. Bits needed by one pair:
+__device__ __forceinline__ int bits_apart(uint32_t x, uint32_t y, int id_bits) {
+    return x == y ? 32 : id_bits - 31 + __clz((int)(x ^ y));
+}
+
+// the two targets' bits (index.cu picks one once the probabilities are known) in one byte, 0: no index
+__device__ __forceinline__ uint8_t pack_chunk_bits(int few, int many, int id_bits) {
+    const int most = min(id_bits, kIdxMaxBits);
+    few = max(few, 1);
+    many = max(many, 1);
+    return (uint8_t)((few <= most ? few : 0) | (many <= most ? many : 0) << 4);
+}
+
+// the same from buf[0, count) sorted, by the lanes or threads r, r + G, ..: this thread's share
+__device__ __forceinline__ void pair_bits(const uint32_t* buf, int count, int r, int G, int id_bits, int& few,
+                                          int& many) {
+    for (int p = r; p + kIdxTargetFew < count; p += G) {
+        few = max(few, bits_apart(buf[p], buf[p + kIdxTargetFew], id_bits));
+        if (p + kIdxTargetMany < count) many = max(many, bits_apart(buf[p], buf[p + kIdxTargetMany], id_bits));
+    }
+}
+
 // Layer profile, small vertices: one warp per vertex whose hyperedges hold at most Cap
 // positions (mu's own included), and every vertex with d_H <= 1 (list == nullptr: all vertices;
 // else the listed ones, all with d_H >= 2 and more than the smaller cap's positions). The
@@ -263,7 +287,7 @@ k_profile_warp(int32_t n, const int32_t* __restrict__ list, const int32_t* __res
                const int2* __restrict__ v_span, const int32_t* __restrict__ he_mem,
                const int32_t* __restrict__ tsum, int id_bits, uint2* __restrict__ pairs,
                uint32_t* __restrict__ nlayers, uint32_t* __restrict__ deg,
-               unsigned long long* __restrict__ maxima) {
+               unsigned long long* __restrict__ maxima, uint8_t* __restrict__ chunk_bits) {
     __shared__ uint32_t raw_s[W][Cap + 4];
     __shared__ uint32_t buf_s[W][Cap];
     __shared__ int bkt_s[W][256];
@@ -309,6 +333,13 @@ k_profile_warp(int32_t n, const int32_t* __restrict__ list, const int32_t* __res
         });
         const int maxb = warp_bucket_scan(bkt, nb);
         warp_scatter_sort(raw, ts, (uint32_t)mu, buf, T, bkt, nb, 0u, shift, key_mask, maxb);
+        if (Cap > kIdxMinT) {  // some of these vertices get a chunk index
+            int few = 0, many = 0;
+            pair_bits(buf, T, lane, 32, id_bits, few, many);
+            few = __reduce_max_sync(0xFFFFFFFFu, few);
+            many = __reduce_max_sync(0xFFFFFFFFu, many);
+            if (lane == 0) chunk_bits[mu] = pack_chunk_bits(few, many, id_bits);
+        }
         // multiplicity histogram over w in [1, dh] (the raw copy is free again)
         uint32_t* hist = raw;
         for (int w = lane; w <= dh; w += 32) hist[w] = 0;
@@ -390,7 +421,8 @@ k_profile(Incidence I, const int2* __restrict__ v_span, const int32_t* __restric
           int id_bits, const int32_t* __restrict__ tsum,
           uint2* __restrict__ pairs, uint32_t* __restrict__ nlayers, uint32_t* __restrict__ deg,
           int* __restrict__ next_vertex, ProfScratch S, DevStatus* st,
-          unsigned long long* __restrict__ maxima /* [max_l, max_deg, max_layer_n] */) {
+          unsigned long long* __restrict__ maxima /* [max_l, max_deg, max_layer_n] */,
+          uint8_t* __restrict__ chunk_bits) {
     extern __shared__ uint32_t smem[];
     uint32_t* buf = smem;                                  // kProfBuf
     uint32_t* hist_s = buf + kProfBuf;                     // kProfHist
@@ -424,10 +456,12 @@ k_profile(Incidence I, const int2* __restrict__ v_span, const int32_t* __restric
             return false;
         };
         const int T = tsum[mu] - dh;  // members other than mu
+        int few = 0, many = 0;        // chunk bits, this thread's share
         if (T <= kProfBuf) {
             const int got = sorted_nbhd<kProfThreads>(v_span, I.he_mem, mu, e0, dh, T, id_bits, buf, bkt, 12,
                                                       pre, ctrl + 32);
             walk_runs<kProfThreads>(buf, got, count_runs);
+            pair_bits(buf, got, threadIdx.x, kProfThreads, id_bits, few, many);
         } else {
             // bucket the members by their top id bits so each bucket fits on chip
             if ((int64_t)T > S.big_cap) {
@@ -491,10 +525,35 @@ k_profile(Incidence I, const int2* __restrict__ v_span, const int32_t* __restric
                 if (cnt > 0) {
                     sort_chunk<kProfThreads>(big + begin, cnt, shift, buf, bkt, 12, ctrl + 32);
                     walk_runs<kProfThreads>(buf, cnt, count_runs);
+                    pair_bits(buf, cnt, threadIdx.x, kProfThreads, id_bits, few, many);
                     __syncthreads();
                 }
                 begin = end;
             }
+            // pairs in different buckets share fewer than b bits: whether whole runs of buckets, the
+            // chunks of fewer bits, hold too many (bucket_cnt[q] is the end of bucket q)
+            for (int c = 1; c <= b; ++c) {
+                const int run = 1 << (b - c);
+                for (int k = threadIdx.x; k < (1 << c); k += kProfThreads) {
+                    const int cnt = bucket_cnt[(k + 1) * run - 1] - (k ? bucket_cnt[k * run - 1] : 0);
+                    if (cnt > kIdxTargetFew) few = max(few, c + 1);
+                    if (cnt > kIdxTargetMany) many = max(many, c + 1);
+                }
+            }
+        }
+        few = __reduce_max_sync(0xFFFFFFFFu, few);
+        many = __reduce_max_sync(0xFFFFFFFFu, many);
+        if ((threadIdx.x & 31) == 0) {
+            ctrl[8 + (threadIdx.x >> 5)] = few;
+            ctrl[32 + (threadIdx.x >> 5)] = many;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 0; w < kProfThreads / 32; ++w) {
+                few = max(few, ctrl[8 + w]);
+                many = max(many, ctrl[32 + w]);
+            }
+            chunk_bits[mu] = pack_chunk_bits(few, many, id_bits);
         }
         __syncthreads();
         if (threadIdx.x < 32) emit_layers(hist, dh, mu, e0, pairs, nlayers, deg, maxima);
@@ -881,12 +940,15 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
     d_deg = (uint32_t*)g->deg;
     if ((st = tmp.alloc(&d_next, sizeof(int)))) return st;
     HYP_CUDA(cudaMemsetAsync(d_next, 0, sizeof(int), s));
+    // chunk bits of the larger neighbourhoods (both targets), from the profile's sorts
+    uint8_t* d_cbits = nullptr;
+    if ((st = tmp.alloc(&d_cbits, (size_t)n))) return st;
     // per-incidence spans first: both profile kernels gather through them
     if ((st = dev_alloc(g, (void**)&g->v_span, sizeof(int2) * nnz_a))) return st;
     if (nnz > 0)
         { k_build_spans<<<grid_for(nnz, 256, sm), 256, 0, s>>>(g->v_he, nnz, g->he_off, g->v_span); count_launch(); }
     { k_profile_warp<kProfWarpT, kPWWarps><<<grid_for((int64_t)n * 32, kPWThreads, sm), kPWThreads, 0, s>>>(
-        n, nullptr, g->v_off, g->v_span, g->he_mem, g->tsum, g->id_bits, d_pairs, d_nl, d_deg, d_max); count_launch(); }
+        n, nullptr, g->v_off, g->v_span, g->he_mem, g->tsum, g->id_bits, d_pairs, d_nl, d_deg, d_max, d_cbits); count_launch(); }
     const size_t prof_smem = sizeof(uint32_t) * (kProfBuf + kProfHist) +
                              sizeof(int) * (2 * kBucketsMax + 2 * kProfThreads + 1 + 64);
     HYP_CUDA(cudaFuncSetAttribute(k_profile, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -925,7 +987,7 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
             { k_big_list<<<grid_for(n, 256, sm), 256, 0, s>>>(n, d_bflag, d_bpos, d_mlist); count_launch(); }
             { k_profile_warp<kProfMidT, kPMWarps><<<grid_for(nmid * 32, kPMWarps * 32, sm), kPMWarps * 32, 0, s>>>(
                 (int32_t)nmid, d_mlist, g->v_off, g->v_span, g->he_mem, g->tsum, g->id_bits, d_pairs, d_nl, d_deg,
-                d_max); count_launch(); }
+                d_max, d_cbits); count_launch(); }
         }
     }
     if (n > 0) { k_big_flags<<<grid_for(n, 256, sm), 256, 0, s>>>(n, g->v_off, g->tsum, kProfMidT, 0x7FFFFFFF, d_bflag); count_launch(); }
@@ -941,7 +1003,7 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
         if ((st = size_order(g, d_blist, nbig, false, d_border))) return st;
         { k_profile<<<(int)std::min<int64_t>(pblocks, nbig), kProfThreads, prof_smem, s>>>(
             I, g->v_span, d_border, (int32_t)nbig, g->id_bits, g->tsum, d_pairs, d_nl, d_deg, d_next, PS,
-            g->d_status, d_max); count_launch(); }
+            g->d_status, d_max, d_cbits); count_launch(); }
     }
     if ((st = check_device_status(g, "layer profile"))) return st;
     HYP_CUDA(cudaMemcpyAsync(hmax, d_max, sizeof(hmax), cudaMemcpyDeviceToHost, s));
@@ -1038,7 +1100,7 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
             HYP_CUDA(cudaMemsetAsync(g->v_dir, 0, sizeof(uint2) * nnz_a, s));
         }
     }
-    if ((st = build_chunk_index(g))) return st;
+    if ((st = build_chunk_index(g, d_cbits))) return st;
 
     // --- strata lists V_s (ascending ids)
     if ((st = dev_alloc(g, (void**)&g->vs_off, sizeof(int32_t) * (HYPERIM_NSTRATA + 1)))) return st;
