@@ -327,7 +327,8 @@ __device__ __forceinline__ void block_sets(LongSets& S, int64_t items, Find&& fi
     }
 }
 
-// inverted index (vertex -> RR ids), the members' numbers and the initial scores
+// inverted index (vertex -> RR ids), the members' numbers and the initial scores (cidx null: a vertex's
+// number is its id)
 __global__ void __launch_bounds__(kGThreads)
 k_scatter_active(const int64_t* __restrict__ rr_off, const int32_t* __restrict__ mem,
                  const uint8_t* __restrict__ rr_stratum, const uint32_t* __restrict__ rr_j,
@@ -347,9 +348,9 @@ k_scatter_active(const int64_t* __restrict__ rr_off, const int32_t* __restrict__
         },
         [&](int64_t x, unsigned long long tag) {
             const int32_t v = mem[x];
-            const uint32_t c = cidx[v];
+            const uint32_t c = cidx ? cidx[v] : (uint32_t)v;
             inv[inv_off[v] + atomicAdd(&cur[v], 1u)] = (uint32_t)(tag >> 4);
-            memc[x] = c;
+            if (cidx) memc[x] = c;
             atomicAdd(&score[c], W.w[tag & 15]);
         });
 }
@@ -360,7 +361,7 @@ struct GreedyOut {
 };
 
 struct GreedyParams {
-    const int32_t* act;
+    const int32_t* act;          // by number (null: every vertex takes part, its number is its id)
     unsigned long long* score;   // by number
     const unsigned int* nact;
     const int64_t* inv_off;      // by vertex
@@ -565,7 +566,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_greedy(GreedyParams P) {
     __shared__ LongSets sets;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t t0 = blockIdx.x * (int64_t)kGThreads + threadIdx.x, T = (int64_t)gridDim.x * kGThreads;
-    const unsigned int na = *P.nact;
+    const unsigned int na = P.act ? *P.nact : (unsigned int)P.n;
     unsigned int target = 0;
     int turn = 0;
     unsigned long long cover = 0, best_lo = ~0ull, best_hi = ~0ull;
@@ -583,7 +584,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_greedy(GreedyParams P) {
         uint32_t bi = 0xFFFFFFFFu;
         auto take = [&](unsigned long long x, int64_t c) {
             if (x > bs || (x == bs && x)) {
-                const uint32_t v = (uint32_t)P.act[c];
+                const uint32_t v = P.act ? (uint32_t)P.act[c] : (uint32_t)c;
                 if (better(x, v, bs, bi)) { bs = x; bi = v; }
             }
         };
@@ -696,7 +697,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_greedy(GreedyParams P) {
                     if (nc > kCandCap) nc = 0;  // too many at the threshold: no candidates
                     if (t0 < nc) {
                         own_c = __ldcg(P.cand + t0);
-                        own_v = (uint32_t)P.act[own_c];
+                        own_v = P.act ? (uint32_t)P.act[own_c] : own_c;
                         own_b = P.inv_off[own_v];
                         own_e = P.inv_off[own_v + 1];
                     }
@@ -1042,10 +1043,14 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
     if ((st = tmp.alloc(&cnt, bytes_cnt))) return st;
     if ((st = tmp.alloc(&inv_off, sizeof(int64_t) * ((size_t)n + 1)))) return st;
     if ((st = tmp.alloc(&inv, sizeof(uint32_t) * members))) return st;
-    if ((st = tmp.alloc(&memc, sizeof(uint32_t) * members))) return st;
     if ((st = tmp.alloc(&score, sizeof(unsigned long long) * (size_t)n))) return st;
-    if ((st = tmp.alloc(&act, sizeof(int32_t) * (size_t)n))) return st;
-    if ((st = tmp.alloc(&cidx, sizeof(uint32_t) * (size_t)n))) return st;
+    // under a budget the vertices keep their ids: no memory for numbers and renumbered members
+    const bool numbered = !graph_root(g)->budget;
+    if (numbered) {
+        if ((st = tmp.alloc(&memc, sizeof(uint32_t) * members))) return st;
+        if ((st = tmp.alloc(&act, sizeof(int32_t) * (size_t)n))) return st;
+        if ((st = tmp.alloc(&cidx, sizeof(uint32_t) * (size_t)n))) return st;
+    }
     if ((st = tmp.alloc(&zero, bytes_zero))) return st;
     if ((st = tmp.alloc(&pscore, sizeof(unsigned long long) * 3 * (size_t)blocks))) return st;
     if ((st = tmp.alloc(&pid, sizeof(uint32_t) * (size_t)blocks))) return st;
@@ -1060,14 +1065,21 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
         { k_count_occ_view<<<grid_cap(N * 32, 256, sm, 32), 256, 0, s>>>(p->rr_off, p->rr_mem, p->rr_stratum,
                                                                         p->rr_j, N, L, cnt); count_launch(); }
     if ((st = exclusive_scan_u32_to_i64(g, cnt, inv_off, n))) return st;
-    { k_active<<<(unsigned)((n + kActThreads * kActItems - 1) / (kActThreads * kActItems)), kActThreads, 0, s>>>(
-          cnt, n, act, cidx, score, &z->nact); count_launch(); }
+    if (numbered) {
+        k_active<<<(unsigned)(((int64_t)n + kActThreads * kActItems - 1) / (kActThreads * kActItems)), kActThreads, 0, s>>>(
+            cnt, n, act, cidx, score, &z->nact);
+        count_launch();
+    } else {
+        HYP_CUDA(cudaMemsetAsync(cnt, 0, bytes_cnt, s));
+        HYP_CUDA(cudaMemsetAsync(score, 0, sizeof(unsigned long long) * (size_t)n, s));
+    }
     if (N > 0)
         { k_scatter_active<<<grid_cap(N * 32 / kSetsPerWarp, kGThreads, sm, 32), kGThreads, 0, s>>>(p->rr_off, p->rr_mem, p->rr_stratum, p->rr_j,
                                                                        N, L, inv_off, cnt, inv, cidx, memc, score,
                                                                        W); count_launch(); }
     HYP_CUDA(cudaGetLastError());
-    GreedyParams G{act, score, &z->nact, inv_off, inv, p->rr_off, memc, p->rr_stratum,
+    GreedyParams G{act, score, &z->nact, inv_off, inv, p->rr_off,
+                   numbered ? memc : reinterpret_cast<const uint32_t*>(p->rr_mem), p->rr_stratum,
                    zero + sizeof(Zero) + (size_t)n, zero + sizeof(Zero), seeds_d, &z->out, W, n, k,
                    prefix_upper ? 1 : 0, cand, &z->ncand, pscore, pid, psum, z->hist, &z->bar, g->d_status};
     if (cluster) {

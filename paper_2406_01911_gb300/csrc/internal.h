@@ -81,6 +81,7 @@ __host__ __device__ inline int idx_sub_bits(int chunk_id_bits) {
 // [D[k 2^(b-c)], D[(k+1) 2^(b-c)]) when c <= b, or a sub-range of [D[r], D[r + 1]), r = k >>
 // (c - b), when c > b (about one member on average). Entries are uint16 (L < 2^16).
 constexpr int kDirMinLen = 4;
+constexpr int kDirMinLenBudget = 16;  // under a budget: directories of the longer ones alone
 constexpr int kDirMaxLen = 65535;
 constexpr int kDirMaxBits = 12;
 

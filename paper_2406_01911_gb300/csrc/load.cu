@@ -774,17 +774,18 @@ __global__ void k_mat_sect(int32_t n, const int32_t* __restrict__ v_off, const i
 }
 
 // directory bits of a hyperedge of L members (0: no directory)
-__device__ __forceinline__ uint32_t dir_bits(int32_t L, int id_bits) {
-    if (L <= kDirMinLen || L > kDirMaxLen) return 0;
+__device__ __forceinline__ uint32_t dir_bits(int32_t L, int id_bits, int min_len) {
+    if (L <= min_len || L > kDirMaxLen) return 0;
     uint32_t b = 1;
     while ((1 << b) < L) ++b;
     const uint32_t cap = (uint32_t)min(id_bits, kDirMaxBits);
     return b < cap ? b : cap;
 }
 
-__global__ void k_dir_size(const int32_t* __restrict__ he_off, int32_t m, int id_bits, uint32_t* __restrict__ size) {
+__global__ void k_dir_size(const int32_t* __restrict__ he_off, int32_t m, int id_bits, int min_len,
+                           uint32_t* __restrict__ size) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t b = dir_bits(he_off[e + 1] - he_off[e], id_bits);
+        const uint32_t b = dir_bits(he_off[e + 1] - he_off[e], id_bits, min_len);
         size[e] = b ? (1u << b) + 1u : 0u;
     }
 }
@@ -792,12 +793,12 @@ __global__ void k_dir_size(const int32_t* __restrict__ he_off, int32_t m, int id
 // one warp per hyperedge: member x (top b bits t_x) sets D[r] = x for t_{x-1} < r <= t_x; the
 // entries above the last member's bits hold L
 __global__ void k_dir_fill(const int32_t* __restrict__ he_off, const int32_t* __restrict__ he_mem, int32_t m,
-                           int id_bits, const int64_t* __restrict__ dir_off, uint16_t* __restrict__ dir) {
+                           int id_bits, int min_len, const int64_t* __restrict__ dir_off, uint16_t* __restrict__ dir) {
     const int lane = threadIdx.x & 31;
     for (int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; e < m;
          e += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int32_t b0 = he_off[e], L = he_off[e + 1] - b0;
-        const uint32_t b = dir_bits(L, id_bits);
+        const uint32_t b = dir_bits(L, id_bits, min_len);
         if (!b) continue;
         const int sh = id_bits - (int)b;
         uint16_t* D = dir + dir_off[e];
@@ -811,10 +812,11 @@ __global__ void k_dir_fill(const int32_t* __restrict__ he_off, const int32_t* __
 
 // per incidence (v_he order): {offset of its hyperedge's directory, bits} or {0, 0}
 __global__ void k_dir_incidence(const int32_t* __restrict__ v_he, int64_t nnz, const int32_t* __restrict__ he_off,
-                                int id_bits, const int64_t* __restrict__ dir_off, uint2* __restrict__ v_dir) {
+                                int id_bits, int min_len, const int64_t* __restrict__ dir_off,
+                                uint2* __restrict__ v_dir) {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < nnz; x += (int64_t)gridDim.x * blockDim.x) {
         const int32_t e = v_he[x];
-        const uint32_t b = dir_bits(he_off[e + 1] - he_off[e], id_bits);
+        const uint32_t b = dir_bits(he_off[e + 1] - he_off[e], id_bits, min_len);
         v_dir[x] = b ? make_uint2((uint32_t)dir_off[e], b) : make_uint2(0u, 0u);
     }
 }
@@ -941,8 +943,8 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
     if ((st = tmp.alloc(&d_next, sizeof(int)))) return st;
     HYP_CUDA(cudaMemsetAsync(d_next, 0, sizeof(int), s));
     // chunk bits of the larger neighbourhoods (both targets), from the profile's sorts
-    uint8_t* d_cbits = nullptr;
-    if ((st = tmp.alloc(&d_cbits, (size_t)n))) return st;
+    uint8_t* d_cbits = reinterpret_cast<uint8_t*>(d_tmp);  // free since the vertex lists were sorted
+    if (sizeof(int32_t) * nnz_alloc < (size_t)n && (st = tmp.alloc(&d_cbits, (size_t)n))) return st;
     // per-incidence spans first: both profile kernels gather through them
     if ((st = dev_alloc(g, (void**)&g->v_span, sizeof(int2) * nnz_a))) return st;
     if (nnz > 0)
@@ -1077,11 +1079,12 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
 
     // --- id directories of the larger hyperedges (read by the chunk path of the RR kernel)
     {
+        const int min_len = g->budget ? kDirMinLenBudget : kDirMinLen;
         uint32_t* d_dsize = nullptr;
         int64_t* d_doff = nullptr;
         if ((st = tmp.alloc(&d_dsize, sizeof(uint32_t) * ((size_t)m + 1)))) return st;
         if ((st = tmp.alloc(&d_doff, sizeof(int64_t) * ((size_t)m + 1)))) return st;
-        if (m > 0) { k_dir_size<<<grid_for(m, 256, sm), 256, 0, s>>>(g->he_off, m, g->id_bits, d_dsize); count_launch(); }
+        if (m > 0) { k_dir_size<<<grid_for(m, 256, sm), 256, 0, s>>>(g->he_off, m, g->id_bits, min_len, d_dsize); count_launch(); }
         if ((st = exclusive_scan_u32_to_i64(g, d_dsize, d_doff, m))) return st;
         int64_t dtotal = 0;
         HYP_CUDA(cudaMemcpyAsync(&dtotal, d_doff + m, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
@@ -1091,10 +1094,10 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
         if ((st = dev_alloc(g, (void**)&g->v_dir, sizeof(uint2) * nnz_a))) return st;
         if (dtotal > 0) {
             if ((st = dev_alloc(g, (void**)&g->he_dir, sizeof(uint16_t) * (size_t)dtotal))) return st;
-            { k_dir_fill<<<grid_for((int64_t)m * 32, 256, sm), 256, 0, s>>>(g->he_off, g->he_mem, m, g->id_bits, d_doff,
+            { k_dir_fill<<<grid_for((int64_t)m * 32, 256, sm), 256, 0, s>>>(g->he_off, g->he_mem, m, g->id_bits, min_len, d_doff,
                                                                          g->he_dir); count_launch(); }
             if (nnz > 0)
-                { k_dir_incidence<<<grid_for(nnz, 256, sm), 256, 0, s>>>(g->v_he, nnz, g->he_off, g->id_bits, d_doff,
+                { k_dir_incidence<<<grid_for(nnz, 256, sm), 256, 0, s>>>(g->v_he, nnz, g->he_off, g->id_bits, min_len, d_doff,
                                                                        g->v_dir); count_launch(); }
         } else {
             HYP_CUDA(cudaMemsetAsync(g->v_dir, 0, sizeof(uint2) * nnz_a, s));
@@ -1111,10 +1114,12 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
     HYP_CUDA(cudaMemcpyAsync(g->vs_off, hvs, sizeof(hvs), cudaMemcpyHostToDevice, s));
     {
         const int64_t runs = ((int64_t)n + kStratumRun - 1) / kStratumRun;
-        uint32_t* d_scnt = nullptr;
-        int64_t* d_spos = nullptr;
-        if ((st = tmp.alloc(&d_scnt, sizeof(uint32_t) * HYPERIM_NSTRATA * (size_t)runs))) return st;
-        if ((st = tmp.alloc(&d_spos, sizeof(int64_t) * (HYPERIM_NSTRATA * (size_t)runs + 1)))) return st;
+        uint32_t* d_scnt = d_cnt;  // n + 1 words and offsets, both free again
+        int64_t* d_spos = d_voff64;
+        if (HYPERIM_NSTRATA * runs > n) {
+            if ((st = tmp.alloc(&d_scnt, sizeof(uint32_t) * HYPERIM_NSTRATA * (size_t)runs))) return st;
+            if ((st = tmp.alloc(&d_spos, sizeof(int64_t) * (HYPERIM_NSTRATA * (size_t)runs + 1)))) return st;
+        }
         const int sgrid = grid_for(runs * 32, 128, sm);
         { k_stratum_count<<<sgrid, 128, 0, s>>>(g->stratum, n, runs, d_scnt); count_launch(); }
         if ((st = exclusive_scan_u32_to_i64(g, d_scnt, d_spos, HYPERIM_NSTRATA * runs))) return st;

@@ -2604,8 +2604,10 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     int32_t warp_limit = g->warp_set_limit;
     if (warp_limit == 0 && mean > 0.0 && mean <= kSmallMean && pools[0]->strategy != HYPERIM_STRAT_LT) warp_limit = kWQ;
     bool warp_phase = g->schedule != HYPERIM_SCHED_PLAIN && warp_limit > 0;
-    // LT sets are single paths: without a tuned warp phase they take the path phase
-    bool path_phase = g->schedule != HYPERIM_SCHED_PLAIN && !warp_phase && pools[0]->strategy == HYPERIM_STRAT_LT;
+    // LT sets are single paths: without a tuned warp phase they take the path phase (not under a budget,
+    // which stays for what a growth step cannot do without)
+    bool path_phase = g->schedule != HYPERIM_SCHED_PLAIN && !warp_phase && pools[0]->strategy == HYPERIM_STRAT_LT &&
+                      !graph_root(g)->budget;
     int wblocks = 0;
     if (warp_phase || path_phase) {
         int wper_sm = 0;
