@@ -1820,7 +1820,8 @@ struct WarpShared {
 // member set and the queue sit in global memory (they stay in L2: 48 KB a warp) because paths run
 // to hundreds of members (2M vertices, weighted cascade: mean 377, largest 1,708). A path of more
 // than 4,096 goes to the block phase. Measured on that graph, 10,010 sets: 843 ms with a block per set,
-// 80 ms with a warp per set.
+// 80 ms with a warp per set; 69 since a pick in an indexed neighbourhood reads an eighth of a chunk, 62 with
+// the members of such a part found in three dependent steps (58 in the latest run).
 __global__ void __launch_bounds__(kPThreads, 2) k_rr_warp(RRParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     WarpShared& S = *reinterpret_cast<WarpShared*>(smem_raw);
