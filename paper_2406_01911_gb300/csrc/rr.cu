@@ -57,6 +57,11 @@ constexpr int kWQ = 128;               // per-warp queue (members of the warp's 
 // set. Mean 1.7 members: the tiny query 0.85 -> 0.46 ms; mean 37: 27.9 -> 25.8 ms; mean 90 (2M vertices,
 // largest 12,000): 251 -> 243 ms. At a mean of 13,000 half of the sets would be begun twice.
 constexpr double kSmallMean = 200.0;
+// ... and only where every warp gets this many sets: with fewer the launch lasts as long as one warp's chain of
+// pops (and sets past kWQ are begun twice). 536 sets of 1,188 vertices, weighted cascade, the whole call: 886 us
+// before the warp phase was taken by size, 1,313 with it for any number of sets, 714 now; 2,000 sets 958 with the
+// warp phase and 793 without, 4,000 sets 957 and 1,024 (20,000 vertices: 1,811 and 1,741), 10,000 no different.
+constexpr int64_t kSmallSetsPerWarp = 4;
 constexpr int kWHashBits = 8;
 constexpr int kWHash = 1 << kWHashBits;  // per-warp open-addressing member set
 // path phase (LT sets): the warp's member set and queue in global memory
@@ -2603,7 +2608,9 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
         mean = hint > 0 && mean >= 0 ? std::max(mean, hint) : -1.0;
     }
     int32_t warp_limit = g->warp_set_limit;
-    if (warp_limit == 0 && mean > 0.0 && mean <= kSmallMean && pools[0]->strategy != HYPERIM_STRAT_LT) warp_limit = kWQ;
+    if (warp_limit == 0 && mean > 0.0 && mean <= kSmallMean && njobs >= kSmallSetsPerWarp * 2 * kPWarps * g->sm_count &&
+        pools[0]->strategy != HYPERIM_STRAT_LT)
+        warp_limit = kWQ;
     bool warp_phase = g->schedule != HYPERIM_SCHED_PLAIN && warp_limit > 0;
     // LT sets are single paths: without a tuned warp phase they take the path phase (not under a budget,
     // which stays for what a growth step cannot do without)
