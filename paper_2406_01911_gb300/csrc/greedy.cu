@@ -571,7 +571,9 @@ __global__ void __launch_bounds__(kGThreads, 1) k_greedy(GreedyParams P) {
     int turn = 0;
     unsigned long long cover = 0, best_lo = ~0ull, best_hi = ~0ull;
     if (threadIdx.x < HYPERIM_NSTRATA) s_lam[threadIdx.x] = 0;
-    __syncthreads();
+    // in a cluster every block has to run before one writes into another's shared memory (send_winner)
+    if (kCluster) grid_meet<kCluster>(P, target);
+    else __syncthreads();
     int32_t round = 0;
     unsigned int nc = 0;            // candidates (0: none, every active vertex is looked at)
     unsigned long long floor = 0;   // every other vertex scores less than this
