@@ -391,8 +391,9 @@ template <bool kCluster>
 __device__ bool grid_meet(const GreedyParams& P, unsigned int& target) {
     __shared__ int ok_s;
     if (kCluster) {  // the cluster's barrier: what a block wrote before is seen by the others after
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        // not .aligned: the lanes of a warp arrive here from loops of different lengths
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
         return true;
     }
     __syncthreads();

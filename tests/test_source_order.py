@@ -26,3 +26,9 @@ def test_cluster_meets_before_the_first_remote_store():
     """A block may write into another block's shared memory only once that block runs."""
     k = body(source("greedy.cu"), "k_greedy(GreedyParams P)")
     assert k.index("grid_meet<kCluster>") < k.index("send_winner")
+
+
+def test_cluster_barrier_takes_a_diverged_warp():
+    """.aligned asks that a warp's threads reach the barrier together; the callers come out of loops whose
+    length differs by lane."""
+    assert re.findall(r"barrier\.cluster\.\w+\.\w+(\.aligned)?;", source("greedy.cu")) == ["", ""]
