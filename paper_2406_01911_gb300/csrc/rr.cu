@@ -773,7 +773,14 @@ constexpr uint64_t kMemoMax = 1ull << 26;      // entries at most (256 MiB)
 constexpr uint64_t kMemoPerSet = 1ull << 14;   // and per new RR set (a short step re-pops little)
 constexpr double kMemoPops = 16.0;
 
-// slots and entries are written by other SMs during the launch: read at the L2, never from an L1 line
+// Slots and entries are written by other SMs during the launch. A slot is read with acquire, so that the
+// entries its warp wrote before it published the slot are seen by the reads that follow; entries are read at
+// the L2, never from an L1 line.
+__device__ __forceinline__ uint32_t ld_slot(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ uint32_t ld_strong(const uint32_t* p) {
     uint32_t v;
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -831,9 +838,11 @@ __device__ __forceinline__ void memo_emit(const uint32_t* buf, int got, int l, u
 }
 
 __device__ __forceinline__ void memo_publish(const RRParams& P, int32_t mu, unsigned long long at) {
-    __threadfence();  // every lane's members before the slot
     __syncwarp();
-    if ((threadIdx.x & 31) == 0) atomicExch(P.memo_slot + mu, kMemoFirst + (uint32_t)at);
+    if ((threadIdx.x & 31) == 0) {
+        __threadfence();  // every lane's members before the slot
+        atomicExch(P.memo_slot + mu, kMemoFirst + (uint32_t)at);
+    }
 }
 
 // The picks (or all members) of the needed layers, read from the entry at `at`.
@@ -886,7 +895,7 @@ __device__ uint32_t pop_lanes(const RRParams& P, SM& S, const Sink& sink, uint32
     if (act) {
         vi = P.vinfo[mu];
         tsum = P.tsum[mu];
-        if (P.memo_slot) kept = ld_strong(P.memo_slot + mu);
+        if (P.memo_slot) kept = ld_slot(P.memo_slot + mu);
     }
     const int l = vi.y, dh = vi.w;
     bool slow = act && (l > kLaneLayers || dh >= kLaneMaxDh || tsum >= kLaneMaxT);
@@ -1020,8 +1029,9 @@ __device__ bool pop_warp(const RRParams& P, SM& S, const Sink& sink, uint32_t j,
     hsum = __reduce_add_sync(0xFFFFFFFFu, hsum);
     const int32_t tsum = P.tsum[mu];
     uint32_t kept = kMemoNone;  // read by one lane: the slot may change while the warp reads it
-    if (P.memo_slot && dh != 1 && lane == 0) kept = ld_strong(P.memo_slot + mu);
+    if (P.memo_slot && dh != 1 && lane == 0) kept = ld_slot(P.memo_slot + mu);
     kept = __shfl_sync(0xFFFFFFFFu, kept, 0);
+    __syncwarp();  // what lane 0 acquired, for the other lanes too
     const bool hit = kept >= kMemoFirst && kept < kMemoBusy;
     if (lane == 0) {
         wst[S_SEL] += hsum;

@@ -32,3 +32,17 @@ def test_cluster_barrier_takes_a_diverged_warp():
     """.aligned asks that a warp's threads reach the barrier together; the callers come out of loops whose
     length differs by lane."""
     assert re.findall(r"barrier\.cluster\.\w+\.\w+(\.aligned)?;", source("greedy.cu")) == ["", ""]
+
+
+def test_kept_neighbourhoods_are_published_and_acquired():
+    """The entries are written, then the slot, after a fence of the thread that writes it; every read of a slot
+    acquires, in the warp's pop for all lanes (a shuffle orders no memory)."""
+    rr = source("rr.cu")
+    readers = set(re.findall(r"(\w+)\(P\.memo_slot \+ mu\)", rr))
+    assert len(readers) == 1
+    assert re.search(r"%s\(const uint32_t\* p\) \{[^}]*ld\.acquire\.gpu" % readers.pop(), rr)
+    publish = re.sub(r"\s+", " ", body(rr, "void memo_publish"))
+    assert "__syncwarp();" in publish and publish.index("__syncwarp();") < publish.index("__threadfence();")
+    assert re.search(r"__threadfence\(\);\s*atomicExch\(P\.memo_slot", publish)
+    warp = re.sub(r"\s+", " ", body(rr, "bool pop_warp("))
+    assert "kept = __shfl_sync(0xFFFFFFFFu, kept, 0); __syncwarp();" in warp
