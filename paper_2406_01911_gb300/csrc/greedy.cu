@@ -1047,13 +1047,6 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
     if ((st = tmp.alloc(&inv_off, sizeof(int64_t) * ((size_t)n + 1)))) return st;
     if ((st = tmp.alloc(&inv, sizeof(uint32_t) * members))) return st;
     if ((st = tmp.alloc(&score, sizeof(unsigned long long) * (size_t)n))) return st;
-    // under a budget the vertices keep their ids: no memory for numbers and renumbered members
-    const bool numbered = !graph_root(g)->budget;
-    if (numbered) {
-        if ((st = tmp.alloc(&memc, sizeof(uint32_t) * members))) return st;
-        if ((st = tmp.alloc(&act, sizeof(int32_t) * (size_t)n))) return st;
-        if ((st = tmp.alloc(&cidx, sizeof(uint32_t) * (size_t)n))) return st;
-    }
     if ((st = tmp.alloc(&zero, bytes_zero))) return st;
     if ((st = tmp.alloc(&pscore, sizeof(unsigned long long) * 3 * (size_t)blocks))) return st;
     if ((st = tmp.alloc(&pid, sizeof(uint32_t) * (size_t)blocks))) return st;
@@ -1068,6 +1061,20 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
         { k_count_occ_view<<<grid_cap(N * 32, 256, sm, 32), 256, 0, s>>>(p->rr_off, p->rr_mem, p->rr_stratum,
                                                                         p->rr_j, N, L, cnt); count_launch(); }
     if ((st = exclusive_scan_u32_to_i64(g, cnt, inv_off, n))) return st;
+    // under a budget, and where the memory for numbers and renumbered members is not to be had (all that the
+    // call cannot do without is there by now), the vertices keep their ids
+    bool numbered = false;
+    if (!graph_root(g)->budget) {
+        const size_t needed = tmp.count();
+        numbered = tmp.alloc(&memc, sizeof(uint32_t) * members) == HYPERIM_OK &&
+                   tmp.alloc(&act, sizeof(int32_t) * (size_t)n) == HYPERIM_OK &&
+                   tmp.alloc(&cidx, sizeof(uint32_t) * (size_t)n) == HYPERIM_OK;
+        if (!numbered) {
+            tmp.release_after(needed);
+            memc = cidx = nullptr;
+            act = nullptr;
+        }
+    }
     if (numbered) {
         k_active<<<(unsigned)(((int64_t)n + kActThreads * kActItems - 1) / (kActThreads * kActItems)), kActThreads, 0, s>>>(
             cnt, n, act, cidx, score, &z->nact);

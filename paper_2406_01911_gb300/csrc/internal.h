@@ -241,8 +241,11 @@ class CallBuffers {
     explicit CallBuffers(hyperim_graph* g) : g_(g) {}
     CallBuffers(const CallBuffers&) = delete;
     CallBuffers& operator=(const CallBuffers&) = delete;
-    ~CallBuffers() {
-        for (auto it = bufs_.rbegin(); it != bufs_.rend(); ++it) dev_free(g_, it->first, it->second);
+    ~CallBuffers() { release_after(0); }
+    // how many buffers there are, and: all but the first `keep` released (what a call did without in the end)
+    size_t count() const { return bufs_.size(); }
+    void release_after(size_t keep) {
+        for (; bufs_.size() > keep; bufs_.pop_back()) dev_free(g_, bufs_.back().first, bufs_.back().second);
     }
     template <typename T>
     hyperim_status alloc(T** p, size_t bytes) {

@@ -1,0 +1,72 @@
+"""What a call can do without it does without: a graph loaded with a budget uses no optional memory, and a
+graph without one, on a device allocator that refuses beyond what that graph's call took, gives the same
+results. Memory is counted in the bytes asked of the caller's allocator."""
+import numpy as np
+import pytest
+
+from tests import gpu_cases as G
+
+pytestmark = pytest.mark.gpu
+
+ROOM = 1 << 40
+
+
+@pytest.fixture(scope="module")
+def H():
+    import paper_2406_01911_gb300 as H
+    H.lib()
+    return H
+
+
+class Meter:
+    """Counts the live bytes of a device allocator and refuses what would take them past `cap`."""
+
+    def __init__(self, H):
+        import torch
+        self.live, self.peak, self.cap, self.size = 0, 0, None, {}
+
+        def alloc(nbytes, stream):
+            if self.cap is not None and self.live + nbytes > self.cap:
+                return 0
+            p = torch.cuda.caching_allocator_alloc(nbytes, 0, stream)
+            self.size[p] = nbytes
+            self.live += nbytes
+            self.peak = max(self.peak, self.live)
+            return p
+
+        def free(p, stream):
+            self.live -= self.size.pop(p)
+            torch.cuda.caching_allocator_delete(p)
+
+        self.allocator = H.DeviceAllocator(alloc, free)
+
+    def need(self, call):
+        """(what call() returns, the bytes it took beyond those live before)."""
+        self.peak = before = self.live
+        out = call()
+        return out, self.peak - before
+
+
+def twins(H, n, hes, model="uniform_pair", p=0.05):
+    """The same graph twice: without a budget, and with one that never binds."""
+    out = []
+    for budget in (0, ROOM):
+        m = Meter(H)
+        out.append((H.Graph(n, *G.csr(hes), model, int(p * G.P32), seed=3, hbm_budget_bytes=budget, allocator=m.allocator), m))
+    return out
+
+
+@pytest.mark.parametrize("theta", [40, 4000, 60_000])
+@pytest.mark.parametrize("upper", ["closed", "prefix"])
+def test_greedy_without_numbers(H, theta, upper):
+    """One block, one cluster, a grid: picks and bounds by number and by id, chosen and for want of memory."""
+    n, hes = G.random_graph(6, 3000, 2600, 9)
+    (a, ma), (b, mb) = twins(H, n, hes, p=0.2)
+    pa, pb = (g.pool(tag=0, roots="stratified").sample(theta) for g in (a, b))
+    want, res = a.select_seeds(pa, None, 25, mode="fixed", upper=upper)
+    (lean, rlean), need = mb.need(lambda: b.select_seeds(pb, None, 25, mode="fixed", upper=upper))
+    ma.cap = ma.live + need
+    tight, rtight = a.select_seeds(pa, None, 25, mode="fixed", upper=upper)
+    for s, r in ((lean, rlean), (tight, rtight)):
+        assert s.tolist() == want.tolist() and r["lambda_r1"].tolist() == res["lambda_r1"].tolist()
+        assert r["upper"] == res["upper"]
