@@ -32,7 +32,7 @@ hyperim_status cuda_fail(cudaError_t e, const char* what) {
                      std::string(what) + ": " + cudaGetErrorString(e));
 }
 
-hyperim_status dev_alloc(hyperim_graph* g, void** p, size_t bytes) {
+hyperim_status dev_try_alloc(hyperim_graph* g, void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     hyperim_graph* r = graph_root(g);  // one budget for all handles of a graph
@@ -81,6 +81,22 @@ void free_memo(hyperim_graph* g) {
     S.memo_slot = nullptr;
     S.memo = nullptr;
     S.memo_cap = 0;
+}
+
+void free_bin_p0(hyperim_graph* g) {
+    dev_free(g, g->scratch.bin_p0, sizeof(double) * (size_t)g->profile_entries);
+    g->scratch.bin_p0 = nullptr;
+}
+
+hyperim_status dev_alloc(hyperim_graph* g, void** p, size_t bytes) {
+    hyperim_status st = dev_try_alloc(g, p, bytes);
+    while (st == HYPERIM_ENOMEM && (g->scratch.memo || g->scratch.bin_p0)) {
+        if (g->scratch.memo) free_memo(g);
+        else free_bin_p0(g);
+        cudaStreamSynchronize(g->stream);  // the memory is free once the stream is there
+        st = dev_try_alloc(g, p, bytes);
+    }
+    return st;
 }
 
 std::mutex& graph_mutex() {
@@ -293,7 +309,7 @@ void free_handle(hyperim_graph* g, bool data) {
     dev_free(g, S.big, sizeof(uint32_t) * S.big_cap * S.blocks);
     dev_free(g, S.arena, sizeof(int32_t) * S.arena_cap);
     free_memo(g);
-    dev_free(g, S.bin_p0, sizeof(double) * (size_t)g->profile_entries);
+    free_bin_p0(g);
     if (data) {
         void* ptrs[] = {g->he_off, g->he_mem, g->v_off, g->v_he, g->tsum, g->v_span, g->vinfo, g->prof_off,
                         g->prof, g->cdf_tab, g->deg, g->stratum, g->vs_off, g->vs_list, g->idx, g->idx_tab, g->idx_sub,

@@ -1066,9 +1066,9 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
     bool numbered = false;
     if (!graph_root(g)->budget) {
         const size_t needed = tmp.count();
-        numbered = tmp.alloc(&memc, sizeof(uint32_t) * members) == HYPERIM_OK &&
-                   tmp.alloc(&act, sizeof(int32_t) * (size_t)n) == HYPERIM_OK &&
-                   tmp.alloc(&cidx, sizeof(uint32_t) * (size_t)n) == HYPERIM_OK;
+        numbered = tmp.try_alloc(&memc, sizeof(uint32_t) * members) &&
+                   tmp.try_alloc(&act, sizeof(int32_t) * (size_t)n) &&
+                   tmp.try_alloc(&cidx, sizeof(uint32_t) * (size_t)n);
         if (!numbered) {
             tmp.release_after(needed);
             memc = cidx = nullptr;

@@ -110,9 +110,9 @@ struct Scratch {
     // output arena
     int32_t* arena = nullptr;
     size_t arena_cap = 0;        // entries
-    // neighbourhoods kept within one growth step (see Memo in rr.cu); optional
+    // optional: the next growth step does without what is not there
     double* bin_p0 = nullptr;    // per profile entry: P(h = 0) of the Binomial strategy (see binomial_h)
-    uint32_t* memo_slot = nullptr;  // n words
+    uint32_t* memo_slot = nullptr;  // n words: neighbourhoods kept within one growth step (see Memo in rr.cu)
     uint32_t* memo = nullptr;
     size_t memo_cap = 0;         // entries
 };
@@ -228,11 +228,15 @@ hyperim_status cuda_fail(cudaError_t e, const char* what);
     } while (0)
 
 // device memory (capi.cu): stream-ordered allocation accounted against the graph's budget,
-// through the caller's allocator when the graph was loaded with one
+// through the caller's allocator when the graph was loaded with one. Before it fails for want of memory,
+// dev_alloc gives up what the handle keeps and can do without (Scratch::memo, Scratch::bin_p0: read them
+// from the handle after a call's allocations); dev_try_alloc, for such buffers themselves, does not.
 hyperim_status dev_alloc(hyperim_graph* g, void** p, size_t bytes);
+hyperim_status dev_try_alloc(hyperim_graph* g, void** p, size_t bytes);
 void dev_free(hyperim_graph* g, void* p, size_t bytes);
-// releases the handle's optional scratch (Scratch::memo), stream-ordered
+// releases the handle's optional scratch (Scratch::memo; Scratch::bin_p0), stream-ordered
 void free_memo(hyperim_graph* g);
+void free_bin_p0(hyperim_graph* g);
 
 // Device buffers of one call: every allocation made through it is released (stream-ordered)
 // when it goes out of scope, on every return path of the call.
@@ -242,6 +246,13 @@ class CallBuffers {
     CallBuffers(const CallBuffers&) = delete;
     CallBuffers& operator=(const CallBuffers&) = delete;
     ~CallBuffers() { release_after(0); }
+    // for a buffer that the call can do without
+    template <typename T>
+    bool try_alloc(T** p, size_t bytes) {
+        if (dev_try_alloc(g_, reinterpret_cast<void**>(p), bytes) != HYPERIM_OK) return false;
+        bufs_.emplace_back(static_cast<void*>(*p), bytes);
+        return true;
+    }
     // how many buffers there are, and: all but the first `keep` released (what a call did without in the end)
     size_t count() const { return bufs_.size(); }
     void release_after(size_t keep) {

@@ -2403,7 +2403,7 @@ hyperim_status ensure_bin_p0(hyperim_graph* g, int32_t strategy) {
     if (strategy != HYPERIM_STRAT_BINOMIAL_ONLY || S.bin_p0 || graph_root(g)->budget || g->profile_entries == 0)
         return HYPERIM_OK;
     const size_t bytes = sizeof(double) * (size_t)g->profile_entries;
-    if (dev_alloc(g, (void**)&S.bin_p0, bytes) != HYPERIM_OK) return HYPERIM_OK;
+    if (dev_try_alloc(g, (void**)&S.bin_p0, bytes) != HYPERIM_OK) return HYPERIM_OK;
     HYP_CUDA(cudaMemsetAsync(S.bin_p0, 0xFF, bytes, g->stream));
     return HYPERIM_OK;
 }
@@ -2432,8 +2432,8 @@ void ensure_memo(hyperim_graph* g, int64_t njobs) {
     if (S.memo && S.memo_cap >= want) return;
     free_memo(g);
     if (graph_root(g)->budget) return;
-    if (dev_alloc(g, (void**)&S.memo_slot, sizeof(uint32_t) * (size_t)g->n) != HYPERIM_OK) return;
-    if (dev_alloc(g, (void**)&S.memo, sizeof(uint32_t) * want) != HYPERIM_OK) {
+    if (dev_try_alloc(g, (void**)&S.memo_slot, sizeof(uint32_t) * (size_t)g->n) != HYPERIM_OK) return;
+    if (dev_try_alloc(g, (void**)&S.memo, sizeof(uint32_t) * want) != HYPERIM_OK) {
         dev_free(g, S.memo_slot, sizeof(uint32_t) * (size_t)g->n);
         S.memo_slot = nullptr;
         return;
@@ -2465,8 +2465,10 @@ uint64_t arena_want(const hyperim_graph* g, hyperim_pool* const* pools, int npoo
 }
 
 // after a growth: the handle's set-size hint, and an idle arena far larger than what the growth
-// used is released (the next growth allocates what its hint asks for)
+// used is released (the next growth allocates what its hint asks for), the memo too where the memory is the
+// caller's to hand out
 void after_growth(hyperim_graph* g, uint64_t used, int64_t njobs, int32_t** arena, uint64_t* cap) {
+    if (g->alloc_fn) free_memo(g);
     if (njobs > 0) g->set_size_hint = std::max(1.0, (double)used / (double)njobs);
     if (*arena && *cap > (1ull << 24) && *cap > 4 * used + 4096) {
         dev_free(g, *arena, sizeof(int32_t) * *cap);
@@ -2604,10 +2606,6 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     int blocks = g->sm_count * per_sm;
     if ((int64_t)blocks > njobs) blocks = (int)njobs;
     if ((st = ensure_scratch(g, blocks, vis_smem))) return st;
-    const bool use_memo = memo_pays(g, pools, npools, pool_start);
-    if (use_memo) ensure_memo(g, njobs);
-    if ((st = ensure_bin_p0(g, pools[0]->strategy))) return st;
-
     const uint64_t want = arena_want(g, pools, npools, pool_start, g->n);
     // the warp phase (one RR set per warp) runs first in the persistent schedule, unless the
     // graph's tuning turned it off; its grid
@@ -2651,6 +2649,15 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     if ((st = tmp.alloc(&d_size, sizeof(int32_t) * (size_t)njobs))) return st;
     if ((st = tmp.alloc(&d_esc, sizeof(int32_t) * (size_t)njobs))) return st;
     if ((st = tmp.alloc(&d_ctrl, sizeof(Ctrl)))) return st;
+    if (g->scratch.arena_cap < want) {
+        if (g->scratch.arena) dev_free(g, g->scratch.arena, sizeof(int32_t) * g->scratch.arena_cap);
+        g->scratch.arena = nullptr;
+        g->scratch.arena_cap = 0;
+        if ((st = dev_alloc(g, (void**)&g->scratch.arena, sizeof(int32_t) * want))) return st;
+        g->scratch.arena_cap = want;
+    }
+    // what the launch can do without comes after what it needs
+    const size_t needed = tmp.count();
     int32_t* d_path = nullptr;
     int path_bits = 0;
     if (path_phase) {
@@ -2658,13 +2665,16 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
         // of n members can need); without the memory for it the sets go to the block kernel
         path_bits = std::min(std::max(g->id_bits + 1, 6), kPathMaxBits);
         const size_t ids = (size_t)wblocks * kPWarps * (3ull << (path_bits - 1));
-        if (tmp.alloc(&d_path, sizeof(int32_t) * ids) == HYPERIM_OK) {
+        if (tmp.try_alloc(&d_path, sizeof(int32_t) * ids)) {
             HYP_CUDA(cudaMemsetAsync(d_path, 0xFF, sizeof(int32_t) * ids, s));
             warp_phase = true;
         } else {
             path_phase = false;
         }
     }
+    const bool use_memo = memo_pays(g, pools, npools, pool_start);
+    if (use_memo) ensure_memo(g, njobs);
+    if ((st = ensure_bin_p0(g, pools[0]->strategy))) return st;
     unsigned long long* d_used = &d_ctrl->arena_used;
     RRParams P;
     std::memset(&P, 0, sizeof(P));
@@ -2717,22 +2727,18 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     HYP_CUDA(cudaEventCreate(&ev1));
     double seconds = 0.0;
     int launches = 0;
-    if (g->scratch.arena_cap < want) {
-        if (g->scratch.arena) dev_free(g, g->scratch.arena, sizeof(int32_t) * g->scratch.arena_cap);
-        g->scratch.arena = nullptr;
-        g->scratch.arena_cap = 0;
-        if ((st = dev_alloc(g, (void**)&g->scratch.arena, sizeof(int32_t) * want))) return st;
-        g->scratch.arena_cap = want;
-    }
     P.arena = g->scratch.arena;
     P.arena_cap = g->scratch.arena_cap;
     P.rewrite = 0;
     HYP_CUDA(cudaMemsetAsync(d_ctrl, 0, sizeof(Ctrl), s));
     HYP_CUDA(cudaMemsetAsync(g->d_counters, 0, sizeof(RRCounters) * kMaxPools, s));
-    P.bin_p0 = P.strategy == HYPERIM_STRAT_BINOMIAL_ONLY ? g->scratch.bin_p0 : nullptr;
-    P.memo_slot = use_memo ? g->scratch.memo_slot : nullptr;
-    P.memo = g->scratch.memo;
-    P.memo_cap = g->scratch.memo_cap;
+    auto take_optional = [&] {  // before each launch: an allocation since the last may have given some up
+        P.bin_p0 = P.strategy == HYPERIM_STRAT_BINOMIAL_ONLY ? g->scratch.bin_p0 : nullptr;
+        P.memo_slot = use_memo ? g->scratch.memo_slot : nullptr;
+        P.memo = g->scratch.memo;
+        P.memo_cap = g->scratch.memo_cap;
+    };
+    take_optional();
     P.memo_used = &d_ctrl->memo_used;
     if (P.memo_slot) HYP_CUDA(cudaMemsetAsync(P.memo_slot, 0, sizeof(uint32_t) * (size_t)g->n, s));
     HYP_CUDA(cudaEventRecord(ev0, s));
@@ -2768,6 +2774,8 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
         return code;
     };
     if ((st = check_device_status(g, "RR generation"))) return failed(st);
+    tmp.release_after(needed);
+    P.path = nullptr;
     float ms = 0.f;
     HYP_CUDA(cudaEventElapsedTime(&ms, ev0, ev1));
     seconds += 1e-3 * (double)ms;
@@ -2794,6 +2802,7 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
         const int plain = P.plain;
         P.arena = na;
         P.arena_cap = new_cap;
+        take_optional();
         P.plain = 0;
         P.block_phase = 1;
         P.rewrite = 1;
@@ -2851,7 +2860,6 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
         deg_max = std::max<int64_t>(deg_max, G.g->max_deg);
         tsum_max = std::max<int64_t>(tsum_max, G.g->max_tsum);
         if (std::find(streams.begin(), streams.end(), G.g->stream) == streams.end()) streams.push_back(G.g->stream);
-        if ((st = ensure_bin_p0(G.g, G.pools[0]->strategy))) return st;
     }
     const int64_t njobs = gstart[ngroups];
     if (njobs == 0) return HYPERIM_OK;
@@ -2871,14 +2879,6 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
             for (cudaEvent_t e : *w) cudaEventDestroy(e);
         }
     } events{&ev0, &ev1, &waits};
-    for (size_t i = 1; i < streams.size(); ++i) {
-        cudaEvent_t e = nullptr;
-        HYP_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        waits.push_back(e);
-        HYP_CUDA(cudaEventRecord(e, streams[i]));
-        HYP_CUDA(cudaStreamWaitEvent(s, e, 0));
-    }
-
     if ((st = allow_rr_smem())) return st;
     cudaFuncAttributes fa;
     HYP_CUDA(cudaFuncGetAttributes(&fa, k_rr_batch));
@@ -2951,7 +2951,6 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
         P.root_mode = G.pools[0]->root_mode;
         P.strategy = G.pools[0]->strategy;
         P.npools = G.npools;
-        P.bin_p0 = P.strategy == HYPERIM_STRAT_BINOMIAL_ONLY ? G.g->scratch.bin_p0 : nullptr;
         for (int i = 0; i <= G.npools; ++i) P.pool_start[i] = pstart[(size_t)q * (kMaxPools + 1) + i];
         for (int i = 0; i < G.npools; ++i) {
             P.tags[i] = G.pools[i]->tag;
@@ -2994,8 +2993,15 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
     double seconds = 0.0;
     if ((st = dev_alloc(g0, (void**)&arena.p, sizeof(int32_t) * want))) return st;
     arena.cap = want;
-    // the memo of this call, after every allocation the launch needs (and only without a budget): slots
-    // of every group's vertices, entries shared by all groups
+    // what the launch can do without comes after what it needs: the handles' kept P(0), and the memo of this
+    // call (only without a budget): slots of every group's vertices, entries shared by all groups
+    const size_t needed = tmp.count();
+    for (int q = 0; q < ngroups; ++q)
+        if ((st = ensure_bin_p0(groups[q].g, groups[q].pools[0]->strategy))) return st;
+    auto take_bin_p0 = [&] {  // before each launch: an allocation since the last may have given some up
+        for (int q = 0; q < ngroups; ++q)
+            hp[q].bin_p0 = hp[q].strategy == HYPERIM_STRAT_BINOMIAL_ONLY ? groups[q].g->scratch.bin_p0 : nullptr;
+    };
     uint32_t *memo_slot = nullptr, *memo = nullptr;
     uint64_t memo_cap = 0;
     auto pays = [&](int q) {
@@ -3010,8 +3016,8 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
             tsum_all += groups[q].g->sum_tsum;
         }
         const uint64_t entries = memo_want(tsum_all, njobs);
-        if (slots && !graph_root(g0)->budget && tmp.alloc(&memo_slot, sizeof(uint32_t) * slots) == HYPERIM_OK &&
-            tmp.alloc(&memo, sizeof(uint32_t) * entries) == HYPERIM_OK) {
+        if (slots && !graph_root(g0)->budget && tmp.try_alloc(&memo_slot, sizeof(uint32_t) * slots) &&
+            tmp.try_alloc(&memo, sizeof(uint32_t) * entries)) {
             memo_cap = entries;
             HYP_CUDA(cudaMemsetAsync(memo_slot, 0, sizeof(uint32_t) * slots, s));
         }
@@ -3029,6 +3035,15 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
             slot0 += (size_t)groups[q].g->n;
         }
     }
+    take_bin_p0();
+    for (size_t i = 1; i < streams.size(); ++i) {
+        cudaEvent_t e = nullptr;
+        HYP_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        waits.push_back(e);
+        HYP_CUDA(cudaEventRecord(e, streams[i]));
+        HYP_CUDA(cudaStreamWaitEvent(s, e, 0));
+    }
+
     B.rerun = nullptr;
     B.rerun_count = nullptr;
     HYP_CUDA(cudaMemcpyAsync(d_groups, hp.data(), sizeof(RRParams) * hp.size(), cudaMemcpyHostToDevice, s));
@@ -3048,14 +3063,20 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
         // sets that did not fit, written to the slots the first launch reserved
         const uint64_t old_cap = arena.cap;
         const uint64_t new_cap = used + used / 8 + 4096;
-        int32_t* na = nullptr;
-        if ((st = dev_alloc(g0, (void**)&na, sizeof(int32_t) * new_cap))) return st;
+        int32_t *na = nullptr, *d_list = nullptr;
+        if (dev_try_alloc(g0, (void**)&na, sizeof(int32_t) * new_cap) != HYPERIM_OK ||
+            !tmp.try_alloc(&d_list, sizeof(int32_t) * (size_t)njobs)) {
+            // the sets left do without the memo
+            if (na) dev_free(g0, na, sizeof(int32_t) * new_cap);
+            tmp.release_after(needed);
+            for (RRParams& P : hp) P.memo_slot = nullptr;
+            if ((st = tmp.alloc(&d_list, sizeof(int32_t) * (size_t)njobs))) return st;
+            if ((st = dev_alloc(g0, (void**)&na, sizeof(int32_t) * new_cap))) return st;
+        }
         HYP_CUDA(cudaMemcpyAsync(na, arena.p, sizeof(int32_t) * old_cap, cudaMemcpyDeviceToDevice, s));
         dev_free(g0, arena.p, sizeof(int32_t) * old_cap);
         arena.p = na;
         arena.cap = new_cap;
-        int32_t* d_list = nullptr;
-        if ((st = tmp.alloc(&d_list, sizeof(int32_t) * (size_t)njobs))) return st;
         HYP_CUDA(cudaMemsetAsync(d_ctrl, 0, sizeof(int) * 2, s));  // job counter, list size
         { k_overflow_jobs<<<(int)std::min<int64_t>((njobs + 255) / 256, (int64_t)g0->sm_count * 8), 256, 0, s>>>(
               d_pos, d_size, njobs, old_cap, d_list, &d_ctrl->rerun_count); count_launch(); }
@@ -3064,6 +3085,7 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
             P.arena_cap = arena.cap;
             P.rewrite = 1;
         }
+        take_bin_p0();
         HYP_CUDA(cudaMemcpyAsync(d_groups, hp.data(), sizeof(RRParams) * hp.size(), cudaMemcpyHostToDevice, s));
         B.rerun = d_list;
         B.rerun_count = &d_ctrl->rerun_count;
@@ -3076,6 +3098,7 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
         seconds += 1e-3 * (double)ms;
     }
     if (seconds_out) *seconds_out = seconds;
+    tmp.release_after(needed);
     std::vector<RRCounters> c((size_t)ngroups * kMaxPools);
     HYP_CUDA(cudaMemcpyAsync(c.data(), d_counters, sizeof(RRCounters) * c.size(), cudaMemcpyDeviceToHost, s));
     // Compaction of every pool in one kernel on s: one scan of all the sizes, each pool's new total

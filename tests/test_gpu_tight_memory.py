@@ -70,3 +70,51 @@ def test_greedy_without_numbers(H, theta, upper):
     for s, r in ((lean, rlean), (tight, rtight)):
         assert s.tolist() == want.tolist() and r["lambda_r1"].tolist() == res["lambda_r1"].tolist()
         assert r["upper"] == res["upper"]
+
+
+def same_sets(pa, pb):
+    sa, sb = G.gpu_sets(pa), G.gpu_sets(pb)
+    return sa[0] == sb[0] and np.array_equal(sa[1], sb[1]) and np.array_equal(sa[2], sb[2])
+
+
+@pytest.mark.parametrize("strategy", ["paper", "binomial_only", "lt"])
+@pytest.mark.parametrize("arena", [0, 1])
+def test_growth_without_optional_memory(H, strategy, arena):
+    """Two growth steps (arena = 1: most sets built again by a repair launch), then a query, each on as much
+    memory as a graph takes that keeps nothing."""
+    n, hes = G.hub_graph(n=6000, hub_edges=40, hub_size=120, mid_edges=8, mid_size=200, m_rest=2500)
+    (a, ma), (b, mb) = twins(H, n, hes, p=0.03)
+    for g in (a, b):
+        g.set_tuning(arena_entries_per_set=arena)
+    pa, pb = (g.pool(tag=0, roots="stratified", strategy=strategy) for g in (a, b))
+    for theta in (300, 900):
+        _, need = mb.need(lambda: pb.sample(theta))
+        ma.cap = ma.live + need
+        pa.sample(theta)
+        ma.cap = None
+        assert same_sets(pa, pb)
+
+    def query(g):
+        return g.select_seeds(g.pool(1, "stratified", strategy), g.pool(2, "stratified", strategy), 5, mode="brr", eps=0.4)
+
+    (sb, rb), need = mb.need(lambda: query(b))
+    ma.cap = ma.live + need
+    sa, ra = query(a)
+    assert sa.tolist() == sb.tolist() and ra["lambda_r1"].tolist() == rb["lambda_r1"].tolist()
+
+
+@pytest.mark.parametrize("strategy", ["paper", "binomial_only"])
+@pytest.mark.parametrize("arena", [0, 1])
+def test_batch_without_optional_memory(H, strategy, arena):
+    n, hes = G.random_graph(3, 2000, 1500, 9)
+    (a, ma), (b, mb) = twins(H, n, hes, p=0.08)
+
+    def batch(g):
+        g.set_tuning(arena_entries_per_set=arena)
+        out = H.hyperim_select_seeds_batch([(g, g.pool(t, "stratified", strategy), g.pool(t + 1, "stratified", strategy), k, 0.3, 1.0)
+                                            for t, k in ((0, 3), (2, 9))])
+        return [(s.tolist(), r["theta"], r["lambda_r1"].tolist(), r["lambda_r2"].tolist()) for s, r in out]
+
+    want, need = mb.need(lambda: batch(b))
+    ma.cap = ma.live + need
+    assert batch(a) == want
