@@ -88,14 +88,25 @@ void free_bin_p0(hyperim_graph* g) {
     g->scratch.bin_p0 = nullptr;
 }
 
+// gives up one buffer that the handle can do without; false: it keeps none
+static bool give_up_one(hyperim_graph* g) {
+    if (g->scratch.memo) {
+        free_memo(g);
+    } else if (g->scratch.bin_p0) {
+        free_bin_p0(g);
+    } else {
+        std::lock_guard<std::mutex> lk(graph_mutex());
+        if (g->owner || g->share_handles > 0 || !g->idx_sub) return false;  // shares read them on their own streams
+        dev_free(g, g->idx_sub, sizeof(uint4) * (size_t)g->idx_entries);
+        g->idx_sub = nullptr;
+    }
+    cudaStreamSynchronize(g->stream);  // the memory is free once the stream is there
+    return true;
+}
+
 hyperim_status dev_alloc(hyperim_graph* g, void** p, size_t bytes) {
     hyperim_status st = dev_try_alloc(g, p, bytes);
-    while (st == HYPERIM_ENOMEM && (g->scratch.memo || g->scratch.bin_p0)) {
-        if (g->scratch.memo) free_memo(g);
-        else free_bin_p0(g);
-        cudaStreamSynchronize(g->stream);  // the memory is free once the stream is there
-        st = dev_try_alloc(g, p, bytes);
-    }
+    while (st == HYPERIM_ENOMEM && give_up_one(g)) st = dev_try_alloc(g, p, bytes);
     return st;
 }
 
@@ -229,16 +240,8 @@ const char* hyperim_last_error(void) { return g_last_error.c_str(); }
 
 uint64_t hyperim_kernel_launches(void) { return g_launches.load(std::memory_order_relaxed); }
 
-hyperim_status hyperim_load(const hyperim_load_args* a, hyperim_graph_t* out) {
-    if (!a || !out) return set_error(HYPERIM_EINVAL, "null argument");
-    *out = nullptr;
-    if (a->n < 1 || a->n >= 0x7FFFFFFF) return set_error(HYPERIM_EINVAL, "n must lie in [1, 2^31 - 1)");
-    if (a->m < 0) return set_error(HYPERIM_EINVAL, "m must be >= 0");
-    if (!a->he_off) return set_error(HYPERIM_EINVAL, "he_off is null");
-    if (a->model < 0 || a->model > 2) return set_error(HYPERIM_EINVAL, "unknown probability model");
-    if (a->uniform_threshold > HYPERIM_P_ONE) return set_error(HYPERIM_EINVAL, "uniform_threshold > 2^32");
-    if ((a->dev_alloc == nullptr) != (a->dev_free == nullptr))
-        return set_error(HYPERIM_EINVAL, "dev_alloc and dev_free must be given together");
+// one try at a load (lean: without optional memory); the arguments have been looked at
+static hyperim_status load_once(const hyperim_load_args* a, bool lean, hyperim_graph_t* out) {
     hyperim_graph* g = new (std::nothrow) hyperim_graph();
     if (!g) return set_error(HYPERIM_ENOMEM, "host allocation failed");
     g->n = a->n;
@@ -248,6 +251,7 @@ hyperim_status hyperim_load(const hyperim_load_args* a, hyperim_graph_t* out) {
     g->seed = a->seed;
     g->stream = (cudaStream_t)a->cuda_stream;
     g->budget = a->hbm_budget_bytes;
+    g->lean = lean;
     g->alloc_fn = a->dev_alloc;
     g->free_fn = a->dev_free;
     g->alloc_ctx = a->alloc_ctx;
@@ -293,6 +297,21 @@ hyperim_status hyperim_load(const hyperim_load_args* a, hyperim_graph_t* out) {
     }
     *out = g;
     return HYPERIM_OK;
+}
+
+hyperim_status hyperim_load(const hyperim_load_args* a, hyperim_graph_t* out) {
+    if (!a || !out) return set_error(HYPERIM_EINVAL, "null argument");
+    *out = nullptr;
+    if (a->n < 1 || a->n >= 0x7FFFFFFF) return set_error(HYPERIM_EINVAL, "n must lie in [1, 2^31 - 1)");
+    if (a->m < 0) return set_error(HYPERIM_EINVAL, "m must be >= 0");
+    if (!a->he_off) return set_error(HYPERIM_EINVAL, "he_off is null");
+    if (a->model < 0 || a->model > 2) return set_error(HYPERIM_EINVAL, "unknown probability model");
+    if (a->uniform_threshold > HYPERIM_P_ONE) return set_error(HYPERIM_EINVAL, "uniform_threshold > 2^32");
+    if ((a->dev_alloc == nullptr) != (a->dev_free == nullptr))
+        return set_error(HYPERIM_EINVAL, "dev_alloc and dev_free must be given together");
+    const hyperim_status st = load_once(a, false, out);
+    // no room: once more without what the graph can do without (a budgeted load takes none of it anyway)
+    return st == HYPERIM_ENOMEM && a->hbm_budget_bytes == 0 ? load_once(a, true, out) : st;
 }
 
 namespace {
@@ -341,6 +360,10 @@ void hyperim_graph_free(hyperim_graph_t g) {
         hyperim_graph* r = g->owner;
         free_handle(g, false);
         delete g;
+        {
+            std::lock_guard<std::mutex> lk(graph_mutex());
+            --r->share_handles;
+        }
         release_root(r);
         return;
     }
@@ -364,8 +387,11 @@ hyperim_status hyperim_graph_share(hyperim_graph_t g, void* cuda_stream, hyperim
     {
         std::lock_guard<std::mutex> lk(graph_mutex());
         ++r->shares;
+        ++r->share_handles;
+        h->idx_sub = r->idx_sub;
     }
     h->owner = r;
+    h->lean = r->lean;
     h->stream = (cudaStream_t)cuda_stream;
     h->n = r->n;
     h->m = r->m;
@@ -391,7 +417,6 @@ hyperim_status hyperim_graph_share(hyperim_graph_t g, void* cuda_stream, hyperim
     h->vs_list = r->vs_list;
     h->idx = r->idx;
     h->idx_tab = r->idx_tab;
-    h->idx_sub = r->idx_sub;
     h->idx_entries = r->idx_entries;
     h->idx_vertices = r->idx_vertices;
     h->profile_entries = r->profile_entries;

@@ -1064,7 +1064,7 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
     // under a budget, and where the memory for numbers and renumbered members is not to be had (all that the
     // call cannot do without is there by now), the vertices keep their ids
     bool numbered = false;
-    if (!graph_root(g)->budget) {
+    if (takes_optional(g)) {
         const size_t needed = tmp.count();
         numbered = tmp.try_alloc(&memc, sizeof(uint32_t) * members) &&
                    tmp.try_alloc(&act, sizeof(int32_t) * (size_t)n) &&

@@ -347,12 +347,10 @@ hyperim_status build_chunk_index(hyperim_graph* g, const uint8_t* chunk_bits) {
         int fblocks = (int)std::min<int64_t>(ncand, (int64_t)sm * per_sm);
         // keep the scratch area within 2 GiB
         while (fblocks > sm && (int64_t)fblocks * cap * 4 > ((int64_t)2 << 30)) fblocks -= sm;
-        // the eighths: not under a budget, nor without the memory
-        if (!graph_root(g)->budget &&
-            dev_alloc(g, (void**)&g->idx_sub, sizeof(uint4) * (size_t)total) != HYPERIM_OK)
-            g->idx_sub = nullptr;
         uint32_t* d_scratch = nullptr;
         if ((st = tmp.alloc(&d_scratch, sizeof(uint32_t) * (size_t)cap * fblocks))) return st;
+        // the eighths, if there is room
+        if (takes_optional(g)) dev_try_alloc(g, (void**)&g->idx_sub, sizeof(uint4) * (size_t)total);
         HYP_CUDA(cudaMemsetAsync(d_next, 0, sizeof(int), s));
         { k_idx_fill<<<fblocks, kFillThreads, kFillSmem, s>>>(d_list, nl, d_bits, d_entries, d_off, g->vinfo, g->v_span,
                                                   g->he_mem, g->tsum, g->prof, g->id_bits, g->idx_tab, g->idx_sub, d_scratch,

@@ -67,7 +67,7 @@ constexpr int kIdxBitsShift = 56;
 // Each entry (layer, chunk) of the index also has, in a second table at the same offset, the members
 // of the layer in the chunk's first 0..7 eighths (eight uint16 in one 16-byte word; a chunk of fewer
 // than 8 ids has fewer parts): a pick then names an eighth of a chunk, 2^idx_sub_bits(id_bits - c) of
-// them per chunk. Left out under a budget.
+// them per chunk. Optional (takes_optional), and given up by a handle that is short of memory.
 constexpr int kIdxSubBits = 3;
 __host__ __device__ inline int idx_sub_bits(int chunk_id_bits) {
     return chunk_id_bits < kIdxSubBits ? chunk_id_bits : kIdxSubBits;
@@ -81,7 +81,7 @@ __host__ __device__ inline int idx_sub_bits(int chunk_id_bits) {
 // [D[k 2^(b-c)], D[(k+1) 2^(b-c)]) when c <= b, or a sub-range of [D[r], D[r + 1]), r = k >>
 // (c - b), when c > b (about one member on average). Entries are uint16 (L < 2^16).
 constexpr int kDirMinLen = 4;
-constexpr int kDirMinLenBudget = 16;  // under a budget: directories of the longer ones alone
+constexpr int kDirMinLenLean = 16;  // without optional memory: directories of the longer ones alone
 constexpr int kDirMaxLen = 65535;
 constexpr int kDirMaxBits = 12;
 
@@ -127,6 +127,7 @@ struct hyperim_graph {
     uint64_t seed = 0;
     cudaStream_t stream = nullptr;
     size_t budget = 0;
+    bool lean = false;           // takes no optional memory: loaded without the room for it
     std::atomic<size_t> device_bytes{0};  // on the loaded graph: all handles of it together
     int id_bits = 1;             // ceil(log2 n)
     // incidence store
@@ -184,6 +185,7 @@ struct hyperim_graph {
     // it is released once it has been freed and no share is left
     hyperim_graph* owner = nullptr;
     int shares = 0;              // live shares and pools of the loaded graph, under hyperim::graph_mutex()
+    int share_handles = 0;       // of these the shares, likewise
     bool freed = false;
 };
 
@@ -213,6 +215,9 @@ namespace hyperim {
 // the loaded graph behind a handle (itself, or the graph a share was made from)
 inline hyperim_graph* graph_root(hyperim_graph* g) { return g->owner ? g->owner : g; }
 inline const hyperim_graph* graph_root(const hyperim_graph* g) { return g->owner ? g->owner : g; }
+// whether a handle may take memory that its calls can do without: not under a budget, which stays for what
+// they need
+inline bool takes_optional(const hyperim_graph* g) { return !graph_root(g)->budget && !g->lean; }
 std::mutex& graph_mutex();
 
 // launch accounting (capi.cu): every kernel launch of the library goes through count_launch()
@@ -229,8 +234,9 @@ hyperim_status cuda_fail(cudaError_t e, const char* what);
 
 // device memory (capi.cu): stream-ordered allocation accounted against the graph's budget,
 // through the caller's allocator when the graph was loaded with one. Before it fails for want of memory,
-// dev_alloc gives up what the handle keeps and can do without (Scratch::memo, Scratch::bin_p0: read them
-// from the handle after a call's allocations); dev_try_alloc, for such buffers themselves, does not.
+// dev_alloc gives up what the handle keeps and can do without (Scratch::memo, Scratch::bin_p0, and idx_sub of
+// a graph without shares: read them from the handle after a call's allocations); dev_try_alloc, for such
+// buffers themselves, does not.
 hyperim_status dev_alloc(hyperim_graph* g, void** p, size_t bytes);
 hyperim_status dev_try_alloc(hyperim_graph* g, void** p, size_t bytes);
 void dev_free(hyperim_graph* g, void* p, size_t bytes);

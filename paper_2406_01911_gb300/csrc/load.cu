@@ -1079,7 +1079,7 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
 
     // --- id directories of the larger hyperedges (read by the chunk path of the RR kernel)
     {
-        const int min_len = g->budget ? kDirMinLenBudget : kDirMinLen;
+        const int min_len = takes_optional(g) ? kDirMinLen : kDirMinLenLean;
         uint32_t* d_dsize = nullptr;
         int64_t* d_doff = nullptr;
         if ((st = tmp.alloc(&d_dsize, sizeof(uint32_t) * ((size_t)m + 1)))) return st;

@@ -2400,7 +2400,7 @@ hyperim_status ensure_scratch(hyperim_graph* g, int blocks, bool vis_smem) {
 // without the memory: the draws then find P(0) each time.
 hyperim_status ensure_bin_p0(hyperim_graph* g, int32_t strategy) {
     Scratch& S = g->scratch;
-    if (strategy != HYPERIM_STRAT_BINOMIAL_ONLY || S.bin_p0 || graph_root(g)->budget || g->profile_entries == 0)
+    if (strategy != HYPERIM_STRAT_BINOMIAL_ONLY || S.bin_p0 || !takes_optional(g) || g->profile_entries == 0)
         return HYPERIM_OK;
     const size_t bytes = sizeof(double) * (size_t)g->profile_entries;
     if (dev_try_alloc(g, (void**)&S.bin_p0, bytes) != HYPERIM_OK) return HYPERIM_OK;
@@ -2431,7 +2431,7 @@ void ensure_memo(hyperim_graph* g, int64_t njobs) {
     const uint64_t want = memo_want(g->sum_tsum, njobs);
     if (S.memo && S.memo_cap >= want) return;
     free_memo(g);
-    if (graph_root(g)->budget) return;
+    if (!takes_optional(g)) return;
     if (dev_try_alloc(g, (void**)&S.memo_slot, sizeof(uint32_t) * (size_t)g->n) != HYPERIM_OK) return;
     if (dev_try_alloc(g, (void**)&S.memo, sizeof(uint32_t) * want) != HYPERIM_OK) {
         dev_free(g, S.memo_slot, sizeof(uint32_t) * (size_t)g->n);
@@ -2623,7 +2623,7 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     // LT sets are single paths: without a tuned warp phase they take the path phase (not under a budget,
     // which stays for what a growth step cannot do without)
     bool path_phase = g->schedule != HYPERIM_SCHED_PLAIN && !warp_phase && pools[0]->strategy == HYPERIM_STRAT_LT &&
-                      !graph_root(g)->budget;
+                      takes_optional(g);
     int wblocks = 0;
     if (warp_phase || path_phase) {
         int wper_sm = 0;
@@ -2737,6 +2737,7 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
         P.memo_slot = use_memo ? g->scratch.memo_slot : nullptr;
         P.memo = g->scratch.memo;
         P.memo_cap = g->scratch.memo_cap;
+        P.idx_sub = g->idx_sub;
     };
     take_optional();
     P.memo_used = &d_ctrl->memo_used;
@@ -2998,9 +2999,11 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
     const size_t needed = tmp.count();
     for (int q = 0; q < ngroups; ++q)
         if ((st = ensure_bin_p0(groups[q].g, groups[q].pools[0]->strategy))) return st;
-    auto take_bin_p0 = [&] {  // before each launch: an allocation since the last may have given some up
-        for (int q = 0; q < ngroups; ++q)
+    auto take_optional = [&] {  // before each launch: an allocation since the last may have given some up
+        for (int q = 0; q < ngroups; ++q) {
             hp[q].bin_p0 = hp[q].strategy == HYPERIM_STRAT_BINOMIAL_ONLY ? groups[q].g->scratch.bin_p0 : nullptr;
+            hp[q].idx_sub = groups[q].g->idx_sub;
+        }
     };
     uint32_t *memo_slot = nullptr, *memo = nullptr;
     uint64_t memo_cap = 0;
@@ -3016,7 +3019,7 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
             tsum_all += groups[q].g->sum_tsum;
         }
         const uint64_t entries = memo_want(tsum_all, njobs);
-        if (slots && !graph_root(g0)->budget && tmp.try_alloc(&memo_slot, sizeof(uint32_t) * slots) &&
+        if (slots && takes_optional(g0) && tmp.try_alloc(&memo_slot, sizeof(uint32_t) * slots) &&
             tmp.try_alloc(&memo, sizeof(uint32_t) * entries)) {
             memo_cap = entries;
             HYP_CUDA(cudaMemsetAsync(memo_slot, 0, sizeof(uint32_t) * slots, s));
@@ -3035,7 +3038,7 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
             slot0 += (size_t)groups[q].g->n;
         }
     }
-    take_bin_p0();
+    take_optional();
     for (size_t i = 1; i < streams.size(); ++i) {
         cudaEvent_t e = nullptr;
         HYP_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -3085,7 +3088,7 @@ hyperim_status sample_rr_batch(hyperim_graph* g0, const RRGroup* groups, int ngr
             P.arena_cap = arena.cap;
             P.rewrite = 1;
         }
-        take_bin_p0();
+        take_optional();
         HYP_CUDA(cudaMemcpyAsync(d_groups, hp.data(), sizeof(RRParams) * hp.size(), cudaMemcpyHostToDevice, s));
         B.rerun = d_list;
         B.rerun_count = &d_ctrl->rerun_count;
@@ -3205,7 +3208,7 @@ hyperim_status forward_spread(hyperim_graph* g, const int32_t* seeds_host, int32
     // more than one block per SM takes more queues than RR generation keeps: at most 1 GiB of them, and
     // none under a budget
     if (blocks > g->sm_count &&
-        (graph_root(g)->budget || (size_t)(blocks - g->sm_count) * (size_t)g->n * sizeof(int32_t) > ((size_t)1 << 30)))
+        (!takes_optional(g) || (size_t)(blocks - g->sm_count) * (size_t)g->n * sizeof(int32_t) > ((size_t)1 << 30)))
         blocks = g->sm_count;
     if ((st = ensure_scratch(g, blocks, vis_smem))) return st;
     int32_t* d_seeds = nullptr;

@@ -118,3 +118,26 @@ def test_batch_without_optional_memory(H, strategy, arena):
     want, need = mb.need(lambda: batch(b))
     ma.cap = ma.live + need
     assert batch(a) == want
+
+
+@pytest.mark.parametrize("name", ["chunks", "short"])
+def test_load_without_optional_memory(H, name):
+    """Neighbourhoods with a chunk index and its eighths, then sets in as much memory as a graph without them
+    takes; hyperedges of 5 to 16 members, whose directories are left out too when they have no room."""
+    n, hes = {"chunks": lambda: G.layered_hub_graph(n=12000, groups=8, size=90, m_rest=3000),
+              "short": lambda: (4000, [list(range(i, i + 9)) for i in range(3900)])}[name]()
+    lists = G.csr(hes)
+    mb = Meter(H)
+    b, need = mb.need(lambda: H.Graph(n, *lists, "wc", 0, seed=3, hbm_budget_bytes=ROOM, allocator=mb.allocator))
+    ma = Meter(H)
+    ma.cap = need
+    a = H.Graph(n, *lists, "wc", 0, seed=3, allocator=ma.allocator)
+    for key, value in b.profile().items():
+        assert np.array_equal(a.profile()[key], value), key
+    (a, ma), (b, mb) = twins(H, n, hes, "wc")
+    extra = ma.live - mb.live - 16 * a.stats()["index_entries"]  # directories, once loaded, stay
+    pa, pb = a.pool(tag=0, roots="plain"), b.pool(tag=0, roots="plain")
+    _, need = mb.need(lambda: pb.sample(20_000))
+    ma.cap = mb.live + need + extra
+    pa.sample(20_000)
+    assert same_sets(pa, pb)
