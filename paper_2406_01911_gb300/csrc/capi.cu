@@ -322,8 +322,8 @@ void free_handle(hyperim_graph* g, bool data) {
     const Scratch& S = g->scratch;
     dev_free(g, g->d_status, sizeof(DevStatus));
     dev_free(g, g->d_counters, 2 * sizeof(RRCounters));
-    dev_free(g, S.list, sizeof(int32_t) * S.list_cap * S.blocks);
-    dev_free(g, S.bitmap, sizeof(uint32_t) * S.bitmap_words * S.blocks);
+    dev_free(g, S.list, sizeof(int32_t) * S.list_cap * S.queue_blocks);
+    dev_free(g, S.bitmap, sizeof(uint32_t) * S.bitmap_words * S.queue_blocks);
     dev_free(g, S.picks, sizeof(uint32_t) * S.pick_cap * S.blocks);
     dev_free(g, S.big, sizeof(uint32_t) * S.big_cap * S.blocks);
     dev_free(g, S.arena, sizeof(int32_t) * S.arena_cap);

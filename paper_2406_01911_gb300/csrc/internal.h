@@ -97,14 +97,16 @@ constexpr int kDirMaxBits = 12;
 constexpr uint32_t kPOneFlag = 0x80000000u;
 
 struct Scratch {
-    // per resident block of the RR kernel
-    int blocks = 0;
+    // per resident block of the RR or forward kernel (queue_blocks of them)
+    int queue_blocks = 0;
     size_t list_cap = 0;         // entries per block (>= n)
     size_t bitmap_words = 0;     // words per block of the global visited bitmap (0 if on-chip)
-    size_t big_cap = 0;          // entries per block for bucketed neighbourhoods
-    size_t pick_cap = 0;         // entries per block for picks
     int32_t* list = nullptr;
     uint32_t* bitmap = nullptr;
+    // per resident block of the RR kernel
+    int blocks = 0;
+    size_t big_cap = 0;          // entries per block for bucketed neighbourhoods
+    size_t pick_cap = 0;         // entries per block for picks
     uint32_t* big = nullptr;
     uint32_t* picks = nullptr;
     // output arena

@@ -2364,33 +2364,56 @@ int wait_rounds(const hyperim_graph* g) {
     return (int)std::min<uint32_t>(w, 0x7FFFFFFFu);
 }
 
-hyperim_status ensure_scratch(hyperim_graph* g, int blocks, bool vis_smem) {
+// The queues of `blocks` blocks and, where it is not on chip, their visited bitmaps. optional: nothing is
+// given up for them.
+hyperim_status ensure_queues(hyperim_graph* g, int blocks, bool vis_smem, bool optional = false) {
     Scratch& S = g->scratch;
     const size_t list_cap = (size_t)g->n;
     const size_t vis_words = vis_smem ? 0 : ((size_t)g->n + 31) / 32;
-    const size_t pick_cap = (size_t)std::max<int64_t>(g->max_deg, 1);  // picks of one pop
-    const size_t big_cap = (size_t)std::max<int64_t>(g->max_tsum, 1);
-    if (S.blocks >= blocks && S.list_cap >= list_cap && S.bitmap_words >= vis_words &&
-        S.pick_cap >= pick_cap && S.big_cap >= big_cap)
-        return HYPERIM_OK;
-    if (S.list) dev_free(g, S.list, sizeof(int32_t) * S.list_cap * S.blocks);
-    if (S.bitmap) dev_free(g, S.bitmap, sizeof(uint32_t) * S.bitmap_words * S.blocks);
-    if (S.picks) dev_free(g, S.picks, sizeof(uint32_t) * S.pick_cap * S.blocks);
-    if (S.big) dev_free(g, S.big, sizeof(uint32_t) * S.big_cap * S.blocks);
-    S = Scratch{0, 0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, S.arena, S.arena_cap, S.bin_p0,
-                S.memo_slot, S.memo, S.memo_cap};
-    hyperim_status st;
-    if ((st = dev_alloc(g, (void**)&S.list, sizeof(int32_t) * list_cap * blocks))) return st;
-    HYP_CUDA(cudaMemsetAsync(S.list, 0xFF, sizeof(int32_t) * list_cap * blocks, g->stream));  // empty slots
-    if (vis_words) {
-        if ((st = dev_alloc(g, (void**)&S.bitmap, sizeof(uint32_t) * vis_words * blocks))) return st;
-        HYP_CUDA(cudaMemsetAsync(S.bitmap, 0, sizeof(uint32_t) * vis_words * blocks, g->stream));
-    }
-    if ((st = dev_alloc(g, (void**)&S.picks, sizeof(uint32_t) * pick_cap * blocks))) return st;
-    if ((st = dev_alloc(g, (void**)&S.big, sizeof(uint32_t) * big_cap * blocks))) return st;
-    S.blocks = blocks;
+    if (S.queue_blocks >= blocks && S.list_cap >= list_cap && S.bitmap_words >= vis_words) return HYPERIM_OK;
+    dev_free(g, S.list, sizeof(int32_t) * S.list_cap * S.queue_blocks);
+    dev_free(g, S.bitmap, sizeof(uint32_t) * S.bitmap_words * S.queue_blocks);
+    S.list = nullptr;
+    S.bitmap = nullptr;
+    S.queue_blocks = 0;
+    auto get = optional ? dev_try_alloc : dev_alloc;
+    int32_t* list = nullptr;
+    uint32_t* bitmap = nullptr;
+    hyperim_status st = get(g, (void**)&list, sizeof(int32_t) * list_cap * blocks);
+    if (st == HYPERIM_OK && vis_words && (st = get(g, (void**)&bitmap, sizeof(uint32_t) * vis_words * blocks)))
+        dev_free(g, list, sizeof(int32_t) * list_cap * blocks);
+    if (st) return st;
+    S.list = list;
+    S.bitmap = bitmap;
+    S.queue_blocks = blocks;
     S.list_cap = list_cap;
     S.bitmap_words = vis_words;
+    HYP_CUDA(cudaMemsetAsync(S.list, 0xFF, sizeof(int32_t) * list_cap * blocks, g->stream));  // empty slots
+    if (vis_words) HYP_CUDA(cudaMemsetAsync(S.bitmap, 0, sizeof(uint32_t) * vis_words * blocks, g->stream));
+    return HYPERIM_OK;
+}
+
+// ... and what RR generation needs besides: a pop's picks and its bucketed neighbourhood.
+hyperim_status ensure_scratch(hyperim_graph* g, int blocks, bool vis_smem) {
+    Scratch& S = g->scratch;
+    hyperim_status st;
+    if ((st = ensure_queues(g, blocks, vis_smem))) return st;
+    const size_t pick_cap = (size_t)std::max<int64_t>(g->max_deg, 1);  // picks of one pop
+    const size_t big_cap = (size_t)std::max<int64_t>(g->max_tsum, 1);
+    if (S.blocks >= blocks && S.pick_cap >= pick_cap && S.big_cap >= big_cap) return HYPERIM_OK;
+    dev_free(g, S.picks, sizeof(uint32_t) * S.pick_cap * S.blocks);
+    dev_free(g, S.big, sizeof(uint32_t) * S.big_cap * S.blocks);
+    S.picks = S.big = nullptr;
+    S.blocks = 0;
+    uint32_t *picks = nullptr, *big = nullptr;
+    if ((st = dev_alloc(g, (void**)&picks, sizeof(uint32_t) * pick_cap * blocks))) return st;
+    if ((st = dev_alloc(g, (void**)&big, sizeof(uint32_t) * big_cap * blocks))) {
+        dev_free(g, picks, sizeof(uint32_t) * pick_cap * blocks);
+        return st;
+    }
+    S.picks = picks;
+    S.big = big;
+    S.blocks = blocks;
     S.pick_cap = pick_cap;
     S.big_cap = big_cap;
     return HYPERIM_OK;
@@ -2771,7 +2794,7 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     HYP_CUDA(cudaMemcpyAsync(cycles, d_ctrl->set_cycles, sizeof(cycles), cudaMemcpyDeviceToHost, s));
     auto failed = [&](hyperim_status code) {
         // a failed launch may leave queue slots filled: empty them for the next one
-        cudaMemsetAsync(g->scratch.list, 0xFF, sizeof(int32_t) * g->scratch.list_cap * g->scratch.blocks, s);
+        cudaMemsetAsync(g->scratch.list, 0xFF, sizeof(int32_t) * g->scratch.list_cap * g->scratch.queue_blocks, s);
         return code;
     };
     if ((st = check_device_status(g, "RR generation"))) return failed(st);
@@ -3205,12 +3228,9 @@ hyperim_status forward_spread(hyperim_graph* g, const int32_t* seeds_host, int32
     if (per_sm < 1) return set_error(HYPERIM_ECUDA, "forward kernel does not fit on an SM");
     int blocks = g->sm_count * per_sm;
     if ((uint64_t)blocks > nsims) blocks = (int)nsims;
-    // more than one block per SM takes more queues than RR generation keeps: at most 1 GiB of them, and
-    // none under a budget
-    if (blocks > g->sm_count &&
-        (!takes_optional(g) || (size_t)(blocks - g->sm_count) * (size_t)g->n * sizeof(int32_t) > ((size_t)1 << 30)))
-        blocks = g->sm_count;
-    if ((st = ensure_scratch(g, blocks, vis_smem))) return st;
+    // More than one block per SM takes queues (and bitmaps) that the call can do without: at most 1 GiB of
+    // them, after what it needs, and one block per SM where they are not to be had. (Of the RR kernel's other
+    // scratch, far larger where a hub's hyperedges are, the cascade uses none.)
     int32_t* d_seeds = nullptr;
     uint32_t* d_counts = nullptr;
     unsigned long long* d_next = nullptr;
@@ -3221,6 +3241,12 @@ hyperim_status forward_spread(hyperim_graph* g, const int32_t* seeds_host, int32
     if ((st = tmp.alloc(&d_next, sizeof(unsigned long long)))) return st;
     if (k > 0) HYP_CUDA(cudaMemcpyAsync(d_seeds, seeds_host, sizeof(int32_t) * (size_t)k, cudaMemcpyHostToDevice, s));
     HYP_CUDA(cudaMemsetAsync(d_next, 0, sizeof(unsigned long long), s));
+    const size_t queue = sizeof(int32_t) * (size_t)g->n + (vis_smem ? 0 : sizeof(uint32_t) * (((size_t)g->n + 31) / 32));
+    if (blocks > g->sm_count &&
+        (!takes_optional(g) || (size_t)(blocks - g->sm_count) * queue > ((size_t)1 << 30) ||
+         ensure_queues(g, blocks, vis_smem, true) != HYPERIM_OK))
+        blocks = g->sm_count;
+    if ((st = ensure_queues(g, blocks, vis_smem))) return st;
     FwdParams F;
     std::memset(&F, 0, sizeof(F));
     RRParams& P = F.P;
@@ -3255,7 +3281,7 @@ hyperim_status forward_spread(hyperim_graph* g, const int32_t* seeds_host, int32
     count_launch();
     HYP_CUDA(cudaGetLastError());
     if ((st = check_device_status(g, "forward spread"))) {
-        cudaMemsetAsync(g->scratch.list, 0xFF, sizeof(int32_t) * g->scratch.list_cap * g->scratch.blocks, s);
+        cudaMemsetAsync(g->scratch.list, 0xFF, sizeof(int32_t) * g->scratch.list_cap * g->scratch.queue_blocks, s);
         return st;
     }
     HYP_CUDA(cudaMemcpyAsync(counts_host, d_counts, sizeof(uint32_t) * (size_t)nsims, cudaMemcpyDeviceToHost, s));

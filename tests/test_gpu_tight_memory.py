@@ -141,3 +141,21 @@ def test_load_without_optional_memory(H, name):
     ma.cap = mb.live + need + extra
     pa.sample(20_000)
     assert same_sets(pa, pb)
+
+
+def test_forward_without_a_second_block(H):
+    """A hub whose hyperedges hold 200 times n members: the blocks beyond one per SM take no more than their
+    queues, and the counts are the same without them, under a budget or for want of memory."""
+    import torch
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    n, rng = 5000, np.random.default_rng(8)
+    hes = [[0] + rng.choice(n - 1, size=2500, replace=False).tolist() for _ in range(400)]
+    (a, ma), (b, mb) = twins(H, n, hes, p=0.0005)
+    live = ma.live
+    (want, _, _), more = ma.need(lambda: a.forward_spread([1, 2, 3], 2 * sm + 90, seed=4))
+    (lean, _, _), need = mb.need(lambda: b.forward_spread([1, 2, 3], 2 * sm + 90, seed=4))
+    assert more - need <= sm * 4 * n and ma.live - live <= 2 * sm * 4 * n
+    (a, ma), _ = twins(H, n, hes, p=0.0005)
+    ma.cap = ma.live + need
+    tight, _, _ = a.forward_spread([1, 2, 3], 2 * sm + 90, seed=4)
+    assert lean.tolist() == want.tolist() == tight.tolist()
