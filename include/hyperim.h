@@ -100,6 +100,12 @@ typedef struct hyperim_pool* hyperim_pool_t;
  *   passes its own). The hooks may be called from any thread that calls into the library
  *   (query server workers included) and must outlive the graph, its shares and its pools. The
  *   HBM budget still counts every byte requested through them.
+ *   Optional memory: without a budget a load also takes 16 bytes per entry of the chunk index and
+ *   id directories of hyperedges of 5 to 16 members (at most 2 entries of 2 bytes a member), and
+ *   calls keep or take up to 256 MiB of neighbourhoods, 8 bytes a layer (Binomial strategy),
+ *   48 KiB per resident warp (LT sets), renumbered members (greedy), up to 1 GiB of queues
+ *   (forward). None of it is taken under a budget or where it is not to be had, and a handle
+ *   that runs short gives up what it keeps of it; results never depend on it.
  * ------------------------------------------------------------------------------------------ */
 typedef struct {
     int32_t n;                   /* |V| */
@@ -581,11 +587,12 @@ hyperim_status hyperim_coverage_noalloc(int32_t n, const int64_t* rr_off, const 
  *   run alone (hyperim_select_seeds on fresh pools).
  *   A worker keeps one share at a time (the RR kernel's scratch of a share holds a queue of n
  *   entries per resident block), replacing it when its next query is on another graph.
- *   Admission by HBM budget: before a query starts, if the device bytes held by the server's
- *   graphs exceed hbm_budget_bytes (0 = no limit), the pools of graphs with no running query are
- *   released (least recently used first; they are regrown on demand, with the same sets); if the
- *   total is still above the budget the query waits until a running one finishes (it starts
- *   anyway when nothing runs). Latency = submit to completion (host steady clock).
+ *   Admission by HBM budget: before a query starts, if the device bytes that the server's graphs
+ *   need (without the optional memory of their loads, see hyperim_load) exceed hbm_budget_bytes
+ *   (0 = no limit; with a limit the workers take no optional memory), the pools of graphs with
+ *   no running query are released (least recently used first; they are regrown on demand, with
+ *   the same sets); if the total is still above the budget the query waits until a running one
+ *   finishes (it starts anyway when nothing runs). Latency = submit to completion (host steady clock).
  * ------------------------------------------------------------------------------------------ */
 typedef struct hyperim_server* hyperim_server_t;
 

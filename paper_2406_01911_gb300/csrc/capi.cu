@@ -99,6 +99,7 @@ static bool give_up_one(hyperim_graph* g) {
         if (g->owner || g->share_handles > 0 || !g->idx_sub) return false;  // shares read them on their own streams
         dev_free(g, g->idx_sub, sizeof(uint4) * (size_t)g->idx_entries);
         g->idx_sub = nullptr;
+        g->optional_bytes -= sizeof(uint4) * (size_t)g->idx_entries;
     }
     cudaStreamSynchronize(g->stream);  // the memory is free once the stream is there
     return true;

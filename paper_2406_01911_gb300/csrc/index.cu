@@ -350,7 +350,8 @@ hyperim_status build_chunk_index(hyperim_graph* g, const uint8_t* chunk_bits) {
         uint32_t* d_scratch = nullptr;
         if ((st = tmp.alloc(&d_scratch, sizeof(uint32_t) * (size_t)cap * fblocks))) return st;
         // the eighths, if there is room
-        if (takes_optional(g)) dev_try_alloc(g, (void**)&g->idx_sub, sizeof(uint4) * (size_t)total);
+        if (takes_optional(g) && dev_try_alloc(g, (void**)&g->idx_sub, sizeof(uint4) * (size_t)total) == HYPERIM_OK)
+            g->optional_bytes += sizeof(uint4) * (size_t)total;
         HYP_CUDA(cudaMemsetAsync(d_next, 0, sizeof(int), s));
         { k_idx_fill<<<fblocks, kFillThreads, kFillSmem, s>>>(d_list, nl, d_bits, d_entries, d_off, g->vinfo, g->v_span,
                                                   g->he_mem, g->tsum, g->prof, g->id_bits, g->idx_tab, g->idx_sub, d_scratch,

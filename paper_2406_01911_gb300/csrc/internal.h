@@ -129,8 +129,9 @@ struct hyperim_graph {
     uint64_t seed = 0;
     cudaStream_t stream = nullptr;
     size_t budget = 0;
-    bool lean = false;           // takes no optional memory: loaded without the room for it
+    bool lean = false;           // takes no optional memory: loaded without room for it, or a budgeted server's share
     std::atomic<size_t> device_bytes{0};  // on the loaded graph: all handles of it together
+    std::atomic<size_t> optional_bytes{0};  // of these, what the load took without needing it (see takes_optional)
     int id_bits = 1;             // ceil(log2 n)
     // incidence store
     int32_t* he_off = nullptr;   // m + 1

@@ -782,12 +782,18 @@ __device__ __forceinline__ uint32_t dir_bits(int32_t L, int id_bits, int min_len
     return b < cap ? b : cap;
 }
 
+// size: entries of every hyperedge's directory; optional: those of directories that a lean graph leaves out
 __global__ void k_dir_size(const int32_t* __restrict__ he_off, int32_t m, int id_bits, int min_len,
-                           uint32_t* __restrict__ size) {
+                           uint32_t* __restrict__ size, unsigned long long* __restrict__ optional) {
+    unsigned long long extra = 0;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t b = dir_bits(he_off[e + 1] - he_off[e], id_bits, min_len);
+        const int32_t L = he_off[e + 1] - he_off[e];
+        const uint32_t b = dir_bits(L, id_bits, min_len);
         size[e] = b ? (1u << b) + 1u : 0u;
+        if (L <= kDirMinLenLean) extra += size[e];
     }
+    for (int o = 16; o > 0; o >>= 1) extra += __shfl_xor_sync(0xFFFFFFFFu, extra, o);
+    if ((threadIdx.x & 31) == 0 && extra) atomicAdd(optional, extra);
 }
 
 // one warp per hyperedge: member x (top b bits t_x) sets D[r] = x for t_{x-1} < r <= t_x; the
@@ -1084,11 +1090,14 @@ hyperim_status build_graph(hyperim_graph* g, const int32_t* he_off_in, const int
         int64_t* d_doff = nullptr;
         if ((st = tmp.alloc(&d_dsize, sizeof(uint32_t) * ((size_t)m + 1)))) return st;
         if ((st = tmp.alloc(&d_doff, sizeof(int64_t) * ((size_t)m + 1)))) return st;
-        if (m > 0) { k_dir_size<<<grid_for(m, 256, sm), 256, 0, s>>>(g->he_off, m, g->id_bits, min_len, d_dsize); count_launch(); }
+        if (m > 0) { k_dir_size<<<grid_for(m, 256, sm), 256, 0, s>>>(g->he_off, m, g->id_bits, min_len, d_dsize, d_max + 7); count_launch(); }
         if ((st = exclusive_scan_u32_to_i64(g, d_dsize, d_doff, m))) return st;
         int64_t dtotal = 0;
+        unsigned long long dextra = 0;
         HYP_CUDA(cudaMemcpyAsync(&dtotal, d_doff + m, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        HYP_CUDA(cudaMemcpyAsync(&dextra, d_max + 7, sizeof(dextra), cudaMemcpyDeviceToHost, s));
         HYP_CUDA(cudaStreamSynchronize(s));
+        g->optional_bytes += sizeof(uint16_t) * (size_t)dextra;
         if (dtotal >= (int64_t)0xFFFFFFFFll) dtotal = 0;  // offsets must fit 32 bits: no directories
         g->dir_entries = dtotal;
         if ((st = dev_alloc(g, (void**)&g->v_dir, sizeof(uint2) * nnz_a))) return st;

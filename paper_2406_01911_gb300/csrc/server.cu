@@ -72,9 +72,11 @@ struct hyperim_server {
     clk::time_point first_submit, last_done;
     std::vector<std::thread> threads;
 
-    size_t held_bytes() const {
+    // the device bytes of all graphs; needed: without what their loads could have done without, which the
+    // budget does not count (it may not cost a query its pools or its turn)
+    size_t held_bytes(bool needed = true) const {
         size_t b = 0;
-        for (const ServerGraph& sg : graphs) b += sg.g->device_bytes.load();
+        for (const ServerGraph& sg : graphs) b += sg.g->device_bytes.load() - (needed ? sg.g->optional_bytes.load() : 0);
         return b;
     }
 
@@ -155,6 +157,7 @@ void hyperim_server::worker_main(int w) {
                 for (auto& kv : mine) hyperim_graph_free(kv.second);
                 mine.clear();
                 if ((st = hyperim_graph_share(sg->g, streams[(size_t)w], &h)) == HYPERIM_OK) mine[job.q.graph_id] = h;
+                if (h && budget) h->lean = true;
             }
         }
         if (st == HYPERIM_OK) {
@@ -288,7 +291,7 @@ hyperim_status hyperim_server_stats(hyperim_server_t s, hyperim_server_stats_t* 
     out->failed = s->failed;
     out->evictions = s->evictions;
     out->max_running = s->max_running;
-    out->device_bytes = s->held_bytes();
+    out->device_bytes = s->held_bytes(false);
     for (const ServerGraph& sg : s->graphs) {
         out->rr_sets_generated += sg.evicted_sets;
         if (sg.r1) out->rr_sets_generated += (uint64_t)sg.r1->count;
