@@ -213,9 +213,11 @@ hyperim_status hyperim_graph_set_schedule(hyperim_graph_t g, int32_t schedule);
  *   estimate: the draws are keyed by (RR, vertex, layer), so only the time differs.
  *   warp_set_limit: in the persistent schedule every RR set is first built by one warp alone
  *     (its members in on-chip memory) while it has at most this many members (1..128) and no
- *     pop needs the block path; larger sets are built again by a whole block. 0, the
- *     default: every set by a block, or, where the sets so far are small on average (and for LT
- *     sets, which are paths), by warps first (hyperim_graph_autotune measures the alternatives).
+ *     pop needs the block path; larger sets are built again by a whole block. 0: every set by a
+ *     block. A handle whose tuning was never set also reports 0, but decides by itself: sets by
+ *     warps first where the sets so far are small on average and many are asked for (and LT
+ *     sets, which are paths), else every set by a block. A call of hyperim_graph_set_tuning ends
+ *     that, whichever field it is made for; hyperim_graph_autotune measures the alternatives.
  *   early_sets_per_block: BRR (hyperim_select_seeds) grows R1 and R2 in its first launch to at
  *     least this many sets per resident block of the RR kernel per pool (the rounds up to that
  *     theta read their prefixes of it). >= 1; default 4.
@@ -240,9 +242,9 @@ hyperim_status hyperim_graph_get_tuning(hyperim_graph_t g, hyperim_tuning* out);
  *   threshold, n and nnz, the shares of the 16 strata, the largest neighbourhood and degree, in
  *   logarithmic buckets) and (root_mode, strategy) form a key; if the process has tuned a graph
  *   of that key before, its choice is applied at once (from_cache = 1). Otherwise every
- *   candidate -- warp_set_limit in {0 (no fixed limit), 16, 32, 64, 128} -- grows a scratch
- *   pool (tag 255) to `sets` RR sets (0: 8 per SM), the same sets each time since they are keyed
- *   by (stratum, index), and the candidate with the least RR-kernel time (CUDA events, best of
+ *   candidate -- warp_set_limit in {0 (none fixed: the handle decides), 16, 32, 64, 128} --
+ *   grows a scratch pool (tag 255) to `sets` RR sets (0: 8 per SM, where a handle that decides
+ *   takes blocks), the same sets each time since they are keyed by (stratum, index), and the candidate with the least RR-kernel time (CUDA events, best of
  *   two) is applied to g and cached under the key, with the per-set SM cycles (mean, maximum)
  *   the candidate without a fixed limit measured; a graph that takes a cached choice and has no
  *   launch of its own yet starts with those cycles (used by BRR's growing ahead, see

@@ -439,7 +439,9 @@ class Graph:
                 "arena_entries_per_set": t.arena_entries_per_set}
 
     def set_tuning(self, warp_set_limit=None, early_sets_per_block=None, arena_entries_per_set=None):
-        """RR-generation scheduling (hyperim_graph_set_tuning); the results never change."""
+        """RR-generation scheduling (hyperim_graph_set_tuning); the results never change. None leaves a
+        field as tuning() reports it; a graph whose tuning was never set chooses warps or blocks by the
+        sets' size, any call of this ends that (warp_set_limit 0: every set by a block)."""
         cur = self.tuning()
         pick = lambda v, k: int(cur[k] if v is None else v)
         t = Tuning(pick(warp_set_limit, "warp_set_limit"), pick(early_sets_per_block, "early_sets_per_block"),

@@ -433,6 +433,7 @@ hyperim_status hyperim_graph_share(hyperim_graph_t g, void* cuda_stream, hyperim
     h->schedule = r->schedule;
     h->wait_limit = r->wait_limit;
     h->warp_set_limit = r->warp_set_limit;
+    h->warp_by_size = r->warp_by_size;
     h->early_sets_per_block = r->early_sets_per_block;
     h->arena_entries_per_set = r->arena_entries_per_set;
     h->set_size_hint = r->set_size_hint;
@@ -544,6 +545,7 @@ hyperim_status hyperim_graph_set_tuning(hyperim_graph_t g, const hyperim_tuning*
     if (t->arena_entries_per_set < 0 || t->arena_entries_per_set > (1 << 20))
         return set_error(HYPERIM_EINVAL, "arena_entries_per_set outside [0, 2^20]");
     g->warp_set_limit = t->warp_set_limit;
+    g->warp_by_size = false;
     g->early_sets_per_block = t->early_sets_per_block;
     g->arena_entries_per_set = t->arena_entries_per_set;
     return HYPERIM_OK;
@@ -618,6 +620,7 @@ hyperim_status hyperim_graph_autotune(hyperim_graph_t g, int32_t root_mode, int3
             t.early_sets_per_block = g->early_sets_per_block;
             t.arena_entries_per_set = g->arena_entries_per_set;
             g->warp_set_limit = t.warp_set_limit;
+            g->warp_by_size = true;
             if (g->set_cycles_mean <= 0.0) {
                 g->set_cycles_mean = it->second.cycles_mean;
                 g->set_cycles_max = it->second.cycles_max;
@@ -629,8 +632,10 @@ hyperim_status hyperim_graph_autotune(hyperim_graph_t g, int32_t root_mode, int3
     }
     if (sets == 0) sets = 8 * (uint64_t)std::max(g->sm_count, 1);
     const int32_t keep_w = g->warp_set_limit, keep_sched = g->schedule;
+    const bool keep_by_size = g->warp_by_size;
+    g->warp_by_size = true;
     g->schedule = HYPERIM_SCHED_PERSISTENT;
-    const int32_t cand[5] = {0, 16, 32, 64, 128};  // warp-phase set limits (0: none)
+    const int32_t cand[5] = {0, 16, 32, 64, 128};  // warp-phase set limits (0: none fixed, by the sets' size)
     double best = -1.0, best_mean = 0.0, best_max = 0.0;
     hyperim_tuning choice{keep_w, g->early_sets_per_block, g->arena_entries_per_set};
     hyperim_status st = HYPERIM_OK;
@@ -650,7 +655,7 @@ hyperim_status hyperim_graph_autotune(hyperim_graph_t g, int32_t root_mode, int3
                 hyperim_pool_free(p);
                 if (st == HYPERIM_OK && (secs < 0.0 || t < secs)) {
                     secs = t;
-                    c_mean = g->set_cycles_mean;  // the growth's per-set cycles (block kernel's sets)
+                    c_mean = g->set_cycles_mean;  // the growth's per-set cycles
                     c_max = g->set_cycles_max;
                 }
             }
@@ -662,7 +667,7 @@ hyperim_status hyperim_graph_autotune(hyperim_graph_t g, int32_t root_mode, int3
                 best = secs;
                 choice.warp_set_limit = cand[ci];
             }
-            if (cand[ci] == 0) {  // every set on the block kernel: its cycles describe all of them
+            if (cand[ci] == 0) {  // the phases that a handle without a fixed limit uses for so many sets
                 best_mean = c_mean;
                 best_max = c_max;
             }
@@ -672,6 +677,7 @@ hyperim_status hyperim_graph_autotune(hyperim_graph_t g, int32_t root_mode, int3
     g->schedule = keep_sched;
     if (st != HYPERIM_OK) {
         g->warp_set_limit = keep_w;
+        g->warp_by_size = keep_by_size;
         return st;
     }
     g->warp_set_limit = choice.warp_set_limit;

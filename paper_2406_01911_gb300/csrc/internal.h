@@ -170,7 +170,8 @@ struct hyperim_graph {
     int sm_count = 0;
     int32_t schedule = 0;        // hyperim_schedule of RR generation
     uint32_t wait_limit = 0;     // iterations of a bounded device wait (0: the default)
-    int32_t warp_set_limit = 0;  // RR sets up to this size are built by one warp (0: by the size of the sets so far)
+    int32_t warp_set_limit = 0;  // RR sets up to this size are built by one warp (0: none, see warp_by_size)
+    bool warp_by_size = true;    // no limit was set: the warp phase where the sets so far are small, or paths
     int32_t early_sets_per_block = 4;  // BRR's first launch: sets per resident block and pool
     double set_size_hint = 0.0;  // mean RR-set size of this handle's last growth (0: none yet)
     int32_t arena_entries_per_set = 0;  // tuning: initial output arena per new set (0: automatic)

@@ -2639,14 +2639,14 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
         mean = hint > 0 && mean >= 0 ? std::max(mean, hint) : -1.0;
     }
     int32_t warp_limit = g->warp_set_limit;
-    if (warp_limit == 0 && mean > 0.0 && mean <= kSmallMean && njobs >= kSmallSetsPerWarp * 2 * kPWarps * g->sm_count &&
+    if (warp_limit == 0 && g->warp_by_size && mean > 0.0 && mean <= kSmallMean && njobs >= kSmallSetsPerWarp * 2 * kPWarps * g->sm_count &&
         pools[0]->strategy != HYPERIM_STRAT_LT)
         warp_limit = kWQ;
     bool warp_phase = g->schedule != HYPERIM_SCHED_PLAIN && warp_limit > 0;
     // LT sets are single paths: without a tuned warp phase they take the path phase (not under a budget,
     // which stays for what a growth step cannot do without)
-    bool path_phase = g->schedule != HYPERIM_SCHED_PLAIN && !warp_phase && pools[0]->strategy == HYPERIM_STRAT_LT &&
-                      takes_optional(g);
+    bool path_phase = g->schedule != HYPERIM_SCHED_PLAIN && !warp_phase && g->warp_by_size &&
+                      pools[0]->strategy == HYPERIM_STRAT_LT && takes_optional(g);
     int wblocks = 0;
     if (warp_phase || path_phase) {
         int wper_sm = 0;

@@ -84,7 +84,7 @@ def test_growth_without_optional_memory(H, strategy, arena):
     memory as a graph takes that keeps nothing."""
     n, hes = G.hub_graph(n=6000, hub_edges=40, hub_size=120, mid_edges=8, mid_size=200, m_rest=2500)
     (a, ma), (b, mb) = twins(H, n, hes, p=0.03)
-    for g in (a, b):
+    for g in (a, b) if arena else ():
         g.set_tuning(arena_entries_per_set=arena)
     pa, pb = (g.pool(tag=0, roots="stratified", strategy=strategy) for g in (a, b))
     for theta in (300, 900):
@@ -95,6 +95,7 @@ def test_growth_without_optional_memory(H, strategy, arena):
         assert same_sets(pa, pb)
 
     def query(g):
+        g.set_schedule("plain")  # growing ahead follows measured times, and the bytes taken with it
         return g.select_seeds(g.pool(1, "stratified", strategy), g.pool(2, "stratified", strategy), 5, mode="brr", eps=0.4)
 
     (sb, rb), need = mb.need(lambda: query(b))
@@ -110,9 +111,15 @@ def test_batch_without_optional_memory(H, strategy, arena):
     (a, ma), (b, mb) = twins(H, n, hes, p=0.08)
 
     def batch(g):
+        # the batch takes pools by their handles' addresses, and the bytes it needs follow that order
+        made = []
+        for tag in range(4):
+            made.append(g.pool(tag, "stratified", strategy))
+            while tag and made[-1].handle.value < pools[-1].handle.value:
+                made.append(g.pool(tag, "stratified", strategy))
+            pools = made[:1] if tag == 0 else [*pools, made[-1]]
         g.set_tuning(arena_entries_per_set=arena)
-        out = H.hyperim_select_seeds_batch([(g, g.pool(t, "stratified", strategy), g.pool(t + 1, "stratified", strategy), k, 0.3, 1.0)
-                                            for t, k in ((0, 3), (2, 9))])
+        out = H.hyperim_select_seeds_batch([(g, pools[0], pools[1], 3, 0.3, 1.0), (g, pools[2], pools[3], 9, 0.3, 1.0)])
         return [(s.tolist(), r["theta"], r["lambda_r1"].tolist(), r["lambda_r2"].tolist()) for s, r in out]
 
     want, need = mb.need(lambda: batch(b))
