@@ -266,11 +266,12 @@ hyperim_status hyperim_graph_autotune(hyperim_graph_t g, int32_t root_mode, int3
 /* ------------------------------------------------------------------------------------------
  * hyperim_graph_set_wait_limit -- bound of the device-side waits of this handle's kernels (a
  *   warp of the RR or forward kernel waiting for its block's work queue: a claimable vertex, or
- *   the id of a claimed slot still being stored). A wait that runs `iterations` rounds without
- *   progress gives up: the kernel records it, every block leaves its current set and the
- *   launch ends; the call returns HYPERIM_ETIMEDOUT and its results are discarded (the handle
- *   stays usable, pools keep the sets of earlier growth steps). 0 restores the default of 2^24
- *   rounds (about a second of sleeping per wait). Not part of the paper: a failure detector of
+ *   the id of a claimed slot still being stored; a block of the greedy waiting for its grid). A
+ *   wait that runs `iterations` rounds without progress gives up: the kernel records it, every
+ *   block leaves its current set or round and the launch ends; the call returns
+ *   HYPERIM_ETIMEDOUT and its results are discarded (the handle stays usable, pools keep the sets
+ *   of earlier growth steps). 0 restores the default of 2^24 rounds (about a second of sleeping
+ *   per wait for a queue). Not part of the paper: a failure detector of
  *   this library. Shares made afterwards inherit the value. EINVAL: g NULL. No device work.
  * ------------------------------------------------------------------------------------------ */
 hyperim_status hyperim_graph_set_wait_limit(hyperim_graph_t g, uint32_t iterations);

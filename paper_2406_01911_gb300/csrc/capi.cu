@@ -140,8 +140,9 @@ hyperim_status check_device_status(hyperim_graph* g, const char* where) {
         return set_error(HYPERIM_EOVERFLOW, msg + "scratch capacity exceeded at vertex " +
                                                 std::to_string(h.detail));
     case kErrSpin:
-        return set_error(HYPERIM_ETIMEDOUT, msg + "a bounded work-queue wait gave up in job " +
-                                                std::to_string(h.detail));
+        return set_error(HYPERIM_ETIMEDOUT, msg + (h.detail < 0 ? std::string("a bounded barrier wait gave up")
+                                                                : "a bounded work-queue wait gave up in job " +
+                                                                      std::to_string(h.detail)));
     default:
         return set_error(HYPERIM_ECUDA, msg + "device error " + std::to_string(h.code));
     }

@@ -224,7 +224,6 @@ __global__ void k_retire(const int32_t* __restrict__ best, const int64_t* __rest
 constexpr int kGThreads = 512;
 constexpr int kGWarps = kGThreads / 32;
 constexpr int64_t kGMembersPerBlock = 1 << 14;
-constexpr int kGSpin = 1 << 24;  // rounds of a barrier wait (seconds) before it gives up
 constexpr int kGCluster = 16;
 constexpr int64_t kGClusterMembers = 1 << 22;
 constexpr unsigned int kCand = 4096, kCandCap = kGCluster * kGThreads;  // at most one per thread
@@ -384,6 +383,7 @@ struct GreedyParams {
     unsigned int* hist;          // 3 x kTopBins, zeroed
     unsigned int* bar;           // zeroed
     DevStatus* st;
+    int spin_limit;              // rounds of a barrier wait before it gives up
 };
 
 // All blocks of the launch meet; false when the bounded wait gave up here.
@@ -406,7 +406,7 @@ __device__ bool grid_meet(const GreedyParams& P, unsigned int& target) {
         unsigned int seen;
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(P.bar) : "memory");
-        } while ((int)(seen - target) < 0 && ++it < kGSpin);
+        } while ((int)(seen - target) < 0 && ++it < P.spin_limit);
         ok_s = (int)(seen - target) >= 0;
         if (!ok_s && atomicCAS(&P.st->code, 0, (int32_t)kErrSpin) == 0) P.st->detail = -1;
         __threadfence();
@@ -1091,7 +1091,7 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
     GreedyParams G{act, score, &z->nact, inv_off, inv, p->rr_off,
                    numbered ? memc : reinterpret_cast<const uint32_t*>(p->rr_mem), p->rr_stratum,
                    zero + sizeof(Zero) + (size_t)n, zero + sizeof(Zero), seeds_d, &z->out, W, n, k,
-                   prefix_upper ? 1 : 0, cand, &z->ncand, pscore, pid, psum, z->hist, &z->bar, g->d_status};
+                   prefix_upper ? 1 : 0, cand, &z->ncand, pscore, pid, psum, z->hist, &z->bar, g->d_status, wait_rounds(g)};
     if (cluster) {
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute at{};

@@ -23,7 +23,7 @@ enum DevErr : int32_t {
     kErrWords = 4,         // a layer draw needed more than 2^18 Philox words
     kErrCapacity = 5,      // a scratch capacity was exceeded
     kErrBucket = 6,        // id bucket larger than the on-chip buffer
-    kErrSpin = 7,          // a bounded wait of the RR kernel's work queue ran out
+    kErrSpin = 7,          // a bounded wait ran out: a work queue's (detail: the job), or the greedy's barrier (-1)
 };
 
 struct DevStatus {
@@ -222,6 +222,11 @@ inline const hyperim_graph* graph_root(const hyperim_graph* g) { return g->owner
 // whether a handle may take memory that its calls can do without: not under a budget, which stays for what
 // they need
 inline bool takes_optional(const hyperim_graph* g) { return !graph_root(g)->budget && !g->lean; }
+// rounds of a bounded device wait (hyperim_graph_set_wait_limit; default 2^24)
+inline int wait_rounds(const hyperim_graph* g) {
+    const uint32_t w = g->wait_limit ? g->wait_limit : 1u << 24;
+    return (int)(w < 0x7FFFFFFFu ? w : 0x7FFFFFFFu);
+}
 std::mutex& graph_mutex();
 
 // launch accounting (capi.cu): every kernel launch of the library goes through count_launch()

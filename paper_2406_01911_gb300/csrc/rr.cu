@@ -2358,12 +2358,6 @@ hyperim_status allow_rr_smem() {
     return HYPERIM_OK;
 }
 
-// rounds of a bounded device wait (hyperim_graph_set_wait_limit; default 2^24)
-int wait_rounds(const hyperim_graph* g) {
-    const uint32_t w = g->wait_limit ? g->wait_limit : (1u << 24);
-    return (int)std::min<uint32_t>(w, 0x7FFFFFFFu);
-}
-
 // The queues of `blocks` blocks and, where it is not on chip, their visited bitmaps. optional: nothing is
 // given up for them.
 hyperim_status ensure_queues(hyperim_graph* g, int blocks, bool vis_smem, bool optional = false) {
