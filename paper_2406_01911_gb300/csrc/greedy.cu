@@ -213,8 +213,13 @@ __global__ void k_retire(const int32_t* __restrict__ best, const int64_t* __rest
 //     its index range in registers: what is left of an argmax is one read of a score. Scores only
 //     decrease, so while the best candidate still reaches that threshold it is the best of all (every
 //     vertex at the threshold is a candidate, so ties are settled among them); when it does not, one
-//     round looks at every active vertex and the candidates are chosen anew. (A grid of 152 blocks loses
-//     more in the select's histograms than it gains: 106 -> 112 ms on the 100k query.)
+//     round looks at every active vertex and the candidates are chosen anew. Where more share the threshold
+//     than fit, or fewer have a score, there are none, and the select (five passes) is tried again a round later,
+//     then 2, 4, 8 .. rounds later. (A grid of 152 blocks loses more in the select's histograms than it gains:
+//     106 -> 112 ms on the 100k query.)
+// 100 seeds from sets of 1.2 members on 2M vertices, nearly all scores alike: 40,000 and 400,000 sets took 3.9 and
+// 11.5 ms with a select every round and the id read after the score, 0.9 and 2.0 ms so (1.8 and 1.9 with two
+// launches a round).
 // 200 seeds chosen on the pools of 40,000 sets of that graph, with the estimate: 4.9 ms with two launches a
 // round, 4.0 ms with a cooperative launch over 152 blocks and no candidates, 3.3 ms so (k_greedy itself 2.7
 // and 2.2 ms: a round is still a chain of six or seven dependent L2 reads); the index build 0.42 -> 0.14 ms
@@ -578,6 +583,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_greedy(GreedyParams P) {
     int32_t round = 0;
     unsigned int nc = 0;            // candidates (0: none, every active vertex is looked at)
     unsigned long long floor = 0;   // every other vertex scores less than this
+    int32_t next_try = 0, wait = 1;  // candidates are not looked for before this round
     uint32_t own_c = 0, own_v = 0xFFFFFFFFu;  // this thread's candidate: number, vertex, index range
     int64_t own_b = 0, own_e = 0;
     for (;; ++round) {
@@ -585,11 +591,8 @@ __global__ void __launch_bounds__(kGThreads, 1) k_greedy(GreedyParams P) {
         // the best (score, lowest id): per block, then over the blocks' winners by every block
         unsigned long long bs = 0;
         uint32_t bi = 0xFFFFFFFFu;
-        auto take = [&](unsigned long long x, int64_t c) {
-            if (x > bs || (x == bs && x)) {
-                const uint32_t v = P.act ? (uint32_t)P.act[c] : (uint32_t)c;
-                if (better(x, v, bs, bi)) { bs = x; bi = v; }
-            }
+        auto take = [&](unsigned long long x, uint32_t v) {
+            if (x && better(x, v, bs, bi)) { bs = x; bi = v; }
         };
         auto reduce = [&]() {  // over the block; the result is warp 0's
             for (int o = 16; o > 0; o >>= 1) {
@@ -677,15 +680,18 @@ __global__ void __launch_bounds__(kGThreads, 1) k_greedy(GreedyParams P) {
             for (int64_t q = t0; q < na4; q += T) {
                 const ulonglong2 a = __ldcg(reinterpret_cast<const ulonglong2*>(P.score) + 2 * q);
                 const ulonglong2 b = __ldcg(reinterpret_cast<const ulonglong2*>(P.score) + 2 * q + 1);
-                take(a.x, 4 * q);
-                take(a.y, 4 * q + 1);
-                take(b.x, 4 * q + 2);
-                take(b.y, 4 * q + 3);
+                // the ids with the scores, not after them: where nearly all scores are alike every one of them decides
+                uint4 v = make_uint4((uint32_t)(4 * q), (uint32_t)(4 * q + 1), (uint32_t)(4 * q + 2), (uint32_t)(4 * q + 3));
+                if (P.act) v = reinterpret_cast<const uint4*>(P.act)[q];
+                take(a.x, v.x);
+                take(a.y, v.y);
+                take(b.x, v.z);
+                take(b.y, v.w);
             }
-            for (int64_t c = 4 * na4 + t0; c < na; c += T) take(__ldcg(P.score + c), c);
+            for (int64_t c = 4 * na4 + t0; c < na; c += T) take(__ldcg(P.score + c), P.act ? (uint32_t)P.act[c] : (uint32_t)c);
             if (!share()) return;
             nc = 0;
-            if (kCluster && !P.prefix && na > 4 * kCand && P.k - round > 8 && win_s) {
+            if (kCluster && !P.prefix && na > 4 * kCand && P.k - round > 8 && win_s && round >= next_try) {
                 unsigned int kleft;
                 if (blockIdx.x == 0 && threadIdx.x == 0) *P.ncand = 0;
                 if (!kth_score<kCluster>(P, na, win_s, kCand, h, turn, target, floor, kleft)) return;
@@ -704,6 +710,12 @@ __global__ void __launch_bounds__(kGThreads, 1) k_greedy(GreedyParams P) {
                         own_b = P.inv_off[own_v];
                         own_e = P.inv_off[own_v + 1];
                     }
+                }
+                if (nc) {
+                    wait = 1;
+                } else {
+                    next_try = round + wait;
+                    wait *= 2;
                 }
             }
         }
