@@ -231,6 +231,7 @@ constexpr int kGWarps = kGThreads / 32;
 constexpr int64_t kGMembersPerBlock = 1 << 14;
 constexpr int kGCluster = 16;
 constexpr int64_t kGClusterMembers = 1 << 22;
+constexpr int64_t kGClusterScan = 1 << 19;
 constexpr unsigned int kCand = 4096, kCandCap = kGCluster * kGThreads;  // at most one per thread
 constexpr int kTopBits = 11;
 constexpr int kTopBins = 1 << kTopBits;
@@ -1030,16 +1031,6 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
     for (int i = 0; i < HYPERIM_NSTRATA; ++i)
         W.w[i] = stratum_weight(g, p->root_mode, view_ns[i], i);
     hyperim_status st;
-    // blocks: by the pool's members, all resident together when more than one
-    int blocks = (int)std::min<int64_t>(std::max<int64_t>(T / kGMembersPerBlock, 1), sm);
-    const bool cluster = blocks > 1 && T <= kGClusterMembers && cluster_fits();
-    if (cluster) {
-        blocks = kGCluster;
-    } else if (blocks > 1) {
-        int per_sm = 0;
-        HYP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_greedy<false>, kGThreads, 0));
-        blocks = std::max(1, std::min(blocks, per_sm * sm));
-    }
     CallBuffers tmp(g);
     uint32_t *cnt = nullptr, *inv = nullptr, *cidx = nullptr, *memc = nullptr, *pid = nullptr, *cand = nullptr;
     int64_t* inv_off = nullptr;
@@ -1060,11 +1051,12 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
     if ((st = tmp.alloc(&inv, sizeof(uint32_t) * members))) return st;
     if ((st = tmp.alloc(&score, sizeof(unsigned long long) * (size_t)n))) return st;
     if ((st = tmp.alloc(&zero, bytes_zero))) return st;
-    if ((st = tmp.alloc(&pscore, sizeof(unsigned long long) * 3 * (size_t)blocks))) return st;
-    if ((st = tmp.alloc(&pid, sizeof(uint32_t) * (size_t)blocks))) return st;
+    const int most_blocks = std::max(sm, kGCluster);
+    if ((st = tmp.alloc(&pscore, sizeof(unsigned long long) * 3 * (size_t)most_blocks))) return st;
+    if ((st = tmp.alloc(&pid, sizeof(uint32_t) * (size_t)most_blocks))) return st;
     if ((st = tmp.alloc(&cand, sizeof(uint32_t) * kCandCap))) return st;
     if ((st = tmp.alloc(&seeds_d, sizeof(int32_t) * (size_t)k))) return st;
-    psum = pscore + blocks;
+    psum = pscore + most_blocks;
     Zero* z = reinterpret_cast<Zero*>(zero);
     HYP_CUDA(cudaMemsetAsync(cnt, 0, bytes_cnt, s));
     HYP_CUDA(cudaMemsetAsync(zero, 0, bytes_zero, s));
@@ -1100,6 +1092,22 @@ hyperim_status greedy(hyperim_graph* g, hyperim_pool* p, int32_t k, int32_t* see
                                                                        N, L, inv_off, cnt, inv, cidx, memc, score,
                                                                        W); count_launch(); }
     HYP_CUDA(cudaGetLastError());
+    // Blocks: by the pool's members, all resident together when more than one; by the vertices too where they
+    // are not numbered, since a look at every vertex then reads all n scores. Without numbers a cluster's 16 SMs
+    // do that quickly enough up to kGClusterScan vertices, beyond it only with members for a sixteenth of them
+    // (else there are no candidates to keep). 100 seeds under a budget, by members alone / now (with two launches a
+    // round): 5,389 members of 2M vertices 26.9 / 0.9 ms (1.8), 34,034 29.6 / 1.0 (1.9), 341,753 1.2 / 1.1 (1.9)
+    // and 1.4 in the grid, 3,548 of 200k 3.4 / 0.9 (1.6), 26,041 of 600k 1.0 in the grid, 2.0 in a cluster.
+    const int64_t work = numbered ? T : std::max<int64_t>(T, n);
+    int blocks = (int)std::min<int64_t>(std::max<int64_t>(work / kGMembersPerBlock, 1), sm);
+    const bool cluster = blocks > 1 && T <= kGClusterMembers && (numbered || n <= kGClusterScan || T >= n / 16) && cluster_fits();
+    if (cluster) {
+        blocks = kGCluster;
+    } else if (blocks > 1) {
+        int per_sm = 0;
+        HYP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_greedy<false>, kGThreads, 0));
+        blocks = std::max(1, std::min(blocks, per_sm * sm));
+    }
     GreedyParams G{act, score, &z->nact, inv_off, inv, p->rr_off,
                    numbered ? memc : reinterpret_cast<const uint32_t*>(p->rr_mem), p->rr_stratum,
                    zero + sizeof(Zero) + (size_t)n, zero + sizeof(Zero), seeds_d, &z->out, W, n, k,

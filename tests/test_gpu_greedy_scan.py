@@ -57,3 +57,12 @@ def test_scores_alike(H, theta):
     assert same_as_stepwise(H, g, pool)
     a, b = seconds(g, pool), stepwise_seconds(H, g, pool)
     assert a < b  # the stepwise form takes two launches and a wait of the host for every round
+
+
+@pytest.mark.parametrize("n,theta", [(40_000, 500), (300_000, 3000), (600_000, 3000), (600_000, 60_000), (2_000_000, 3000)])
+def test_few_members_without_numbers(H, n, theta):
+    """Under a budget the vertices keep their ids, and a round may read every vertex's score."""
+    g = graph(H, 1 << 40, n)
+    pool = g.pool(tag=0, roots="stratified").sample(theta)
+    assert same_as_stepwise(H, g, pool)
+    assert seconds(g, pool) < stepwise_seconds(H, g, pool)
