@@ -1162,7 +1162,7 @@ hyperim_status coverage(hyperim_graph* g, hyperim_pool* p, const int32_t* seeds_
     }
     if (N > 0 && on_chip) {
         const int per = cover_per(N, g->sm_count);
-        { k_cover_sets<<<grid_cap((N + per - 1) / per * 32, kCoverThreads, g->sm_count, 8), kCoverThreads,
+        { k_cover_sets<<<cover_blocks(N, per, k, g->sm_count), kCoverThreads,
                        cover_smem(k), s>>>(p->rr_off, p->rr_mem, p->rr_stratum, p->rr_j, N, L, g->n, sd, k, per,
                                            lam); count_launch(); }
     } else if (N > 0)

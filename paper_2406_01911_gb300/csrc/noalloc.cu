@@ -117,9 +117,7 @@ extern "C" hyperim_status hyperim_coverage_noalloc(int32_t n, const int64_t* rr_
         cudaError_t e = cudaMemsetAsync(lambda_s, 0, sizeof(unsigned long long) * HYPERIM_NSTRATA, s);
         if (e == cudaSuccess && count > 0) {
             const int per = cover_per(count, sm);
-            const int64_t warps = (count + per - 1) / per;
-            const int64_t want = (warps * 32 + kCoverThreads - 1) / kCoverThreads;
-            k_na_cover_sets<<<(int)(want < (int64_t)sm * 8 ? want : (int64_t)sm * 8), kCoverThreads, cover_smem(k), s>>>(
+            k_na_cover_sets<<<cover_blocks(count, per, k, sm), kCoverThreads, cover_smem(k), s>>>(
                 rr_off, rr_mem, rr_stratum, count, n, seeds, k, per, lambda_s);
             count_launch();
             e = cudaGetLastError();
