@@ -41,7 +41,7 @@ __global__ void k_check_offsets(const int32_t* off, int32_t m, DevStatus* st) {
 // ---- short lists sorted on chip -------------------------------------------------------------------
 // Lists (hyperedges, or the hyperedges of a vertex) sorted ascending, one warp per list: up to 32
 // entries across the lanes, up to kListWarp in the warp's part of shared memory, up to kListBlock by
-// the whole block after its warps are done; longer ones by counting smaller entries, n^2 reads. (Every
+// the whole block after its warps are done; longer ones by counting smaller entries, n^2 compares. (Every
 // list above 32 took the n^2 way before: 155 us on a graph of 14,142 vertices, 3.3 + 2.7 ms on 2M.)
 constexpr int kListThreads = 256;
 constexpr int kListWarps = kListThreads / 32;
@@ -68,26 +68,78 @@ __device__ int sort_unique(const int32_t* __restrict__ in, int len, uint32_t* bu
     return kept;
 }
 
-// the same for a list that fits nowhere on chip (first: one flag byte per entry)
+// The same for a list that fits nowhere on chip (first: one flag byte per entry): every entry is compared with
+// all of them, which pass through the block's buffer kListBlock at a time, kCountEach entries per thread and read.
+// (Read from global memory one by one: a vertex in 30,000 pairs 214 ms of load, 178 with a warp per list, 17 so; a
+// hyperedge of 50,000 members 584 and 4,700, now 153.)
+// tile(j): what entry j is compared as; each(i, j0, m): entries i, i + kListThreads, .. with buf[0, m), entries j0 on.
+constexpr int kCountEach = 8;
+template <typename Tile, typename Each>
+__device__ __forceinline__ void against_all(int64_t len, uint32_t* buf, Tile&& tile, Each&& each) {
+    for (int64_t i0 = 0; i0 < len; i0 += kListThreads * kCountEach)
+        for (int64_t j0 = 0; j0 < len; j0 += kListBlock) {
+            const int m = (int)min(len - j0, (int64_t)kListBlock);
+            for (int j = threadIdx.x; j < m; j += kListThreads) buf[j] = tile(j0 + j);
+            __syncthreads();
+            each(i0 + threadIdx.x, j0, m);
+            __syncthreads();
+        }
+}
+
+// distinct: no value repeats
 __device__ int count_unique(const int32_t* __restrict__ in, int64_t len, int32_t* __restrict__ out,
-                            uint8_t* __restrict__ first, int* tmp) {
-    for (int64_t i = threadIdx.x; i < len; i += kListThreads) {
-        const int32_t x = in[i];
-        bool dup = false;
-        for (int64_t j = 0; j < i && !dup; ++j) dup = in[j] == x;
-        first[i] = dup ? 0 : 1;
-    }
+                            uint8_t* __restrict__ first, bool distinct, uint32_t* buf, int* tmp) {
     if (threadIdx.x == 0) tmp[0] = 0;
-    __syncthreads();
+    uint32_t x[kCountEach];
+    int below[kCountEach];
+    bool dup[kCountEach];
+    auto begin = [&](int64_t i) {
+#pragma unroll
+        for (int u = 0; u < kCountEach; ++u) {
+            const int64_t at = i + u * kListThreads;
+            x[u] = at < len ? (uint32_t)in[at] : 0u;
+            below[u] = 0;
+            dup[u] = false;
+        }
+    };
+    if (!distinct)
+        against_all(len, buf, [&](int64_t j) { return (uint32_t)in[j]; }, [&](int64_t i, int64_t j0, int m) {
+            if (j0 == 0) begin(i);
+            int before[kCountEach];  // entries of the buffer before the thread's own
+#pragma unroll
+            for (int u = 0; u < kCountEach; ++u)
+                before[u] = (int)max(min(i + u * kListThreads - j0, (int64_t)m), (int64_t)0);
+#pragma unroll 4
+            for (int j = 0; j < m; ++j) {
+                const uint32_t y = buf[j];
+#pragma unroll
+                for (int u = 0; u < kCountEach; ++u) dup[u] = dup[u] || (y == x[u] && j < before[u]);
+            }
+            if (j0 + m == len)
+#pragma unroll
+                for (int u = 0; u < kCountEach; ++u)
+                    if (i + u * kListThreads < len) first[i + u * kListThreads] = dup[u] ? 0 : 1;
+        });
     int mine = 0;
-    for (int64_t i = threadIdx.x; i < len; i += kListThreads) {
-        if (!first[i]) continue;
-        const int32_t x = in[i];
-        int64_t below = 0;
-        for (int64_t j = 0; j < len; ++j) below += (first[j] && in[j] < x) ? 1 : 0;
-        out[below] = x;
-        ++mine;
-    }
+    // repeats are the largest key: below nobody
+    against_all(len, buf, [&](int64_t j) { return distinct || first[j] ? (uint32_t)in[j] : kSentinel; },
+                [&](int64_t i, int64_t j0, int m) {
+                    if (j0 == 0) begin(i);
+#pragma unroll 4
+                    for (int j = 0; j < m; ++j) {
+                        const uint32_t y = buf[j];
+#pragma unroll
+                        for (int u = 0; u < kCountEach; ++u) below[u] += y < x[u] ? 1 : 0;
+                    }
+                    if (j0 + m == len)
+#pragma unroll
+                        for (int u = 0; u < kCountEach; ++u) {
+                            const int64_t at = i + u * kListThreads;
+                            if (at >= len || !(distinct || first[at])) continue;
+                            out[below[u]] = (int32_t)x[u];
+                            ++mine;
+                        }
+                });
     atomicAdd(&tmp[0], mine);
     __syncthreads();
     const int kept = tmp[0];
@@ -97,7 +149,7 @@ __device__ int count_unique(const int32_t* __restrict__ in, int64_t len, int32_t
 
 // list i of `lists` is in[off[i], off[i + 1]), its sorted set goes to out at the same place;
 // done(i, kept) is called by one thread, check(i, x) for every entry
-template <typename Off, typename Check, typename Done>
+template <bool kDistinct, typename Off, typename Check, typename Done>
 __device__ __forceinline__ void sort_lists(const Off* __restrict__ off, int32_t lists, const int32_t* __restrict__ in,
                                            int32_t* __restrict__ out, uint8_t* __restrict__ first, Check&& check,
                                            Done&& done) {
@@ -142,7 +194,7 @@ __device__ __forceinline__ void sort_lists(const Off* __restrict__ off, int32_t 
             const int64_t b = (int64_t)off[l], len = (int64_t)off[l + 1] - b;
             for (int64_t x = threadIdx.x; x < len; x += kListThreads) check(l, in[b + x]);
             const int kept = len <= kListBlock ? sort_unique<kListThreads>(in + b, (int)len, buf, out + b, tmp)
-                                               : count_unique(in + b, len, out + b, first + b, tmp);
+                                               : count_unique(in + b, len, out + b, first + b, kDistinct, buf, tmp);
             if (threadIdx.x == 0) done(l, kept);
         }
         __syncthreads();
@@ -153,7 +205,7 @@ __device__ __forceinline__ void sort_lists(const Off* __restrict__ off, int32_t 
 __global__ void __launch_bounds__(kListThreads)
 k_normalise(const int32_t* __restrict__ off, const int32_t* __restrict__ mem, int32_t m, int32_t n,
             int32_t* __restrict__ out, uint8_t* __restrict__ first, uint32_t* __restrict__ newsize, DevStatus* st) {
-    sort_lists(off, m, mem, out, first,
+    sort_lists<false>(off, m, mem, out, first,
                [&](int64_t e, int32_t x) {
                    if (x < 0 || x >= n) dev_fail(st, kErrBadMember, (int32_t)e);
                },
@@ -204,7 +256,7 @@ __global__ void k_scatter_vhe(const int32_t* __restrict__ he_off, const int32_t*
 __global__ void __launch_bounds__(kListThreads)
 k_sort_vhe(const int64_t* __restrict__ v_off64, int32_t n, const int32_t* __restrict__ in, int32_t* __restrict__ out,
            uint8_t* __restrict__ first, int32_t* __restrict__ v_off32) {
-    sort_lists(v_off64, n, in, out, first, [](int64_t, int32_t) {},
+    sort_lists<true>(v_off64, n, in, out, first, [](int64_t, int32_t) {},
                [&](int64_t v, int) {
                    v_off32[v] = (int32_t)v_off64[v];
                    if (v == n - 1) v_off32[n] = (int32_t)v_off64[n];
