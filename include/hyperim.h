@@ -560,7 +560,8 @@ hyperim_status hyperim_forward_spread(hyperim_graph_t g, const int32_t* seeds_ho
  *   valid until this call's work on cuda_stream has finished: no thread may grow or free that
  *   pool in the meantime (growth moves the pool's arrays and frees the old ones). Output (device, caller-owned): lambda_s[16] gets
  *   the number of RR sets of each stratum that contain a seed; the call zeroes it first.
- *   Scratch: one flag byte per vertex in a fixed array of HYPERIM_NOALLOC_MAX_N bytes built into
+ *   Scratch: none in device memory up to 2,048 seeds (repeats counted): they are held on chip.
+ *   Beyond that one flag byte per vertex in a fixed array of HYPERIM_NOALLOC_MAX_N bytes built into
  *   the library; every GPU that loads the library holds those bytes until the process exits.
  *   EINVAL: n < 1 or n > HYPERIM_NOALLOC_MAX_N (the scratch is too small), count < 0, k < 0,
  *   null pointers. Never calls cudaMalloc, cudaFree or any other allocating routine.
@@ -568,10 +569,10 @@ hyperim_status hyperim_forward_spread(hyperim_graph_t g, const int32_t* seeds_ho
  *   set-up step): make that first call before any stream capture. The cached address belongs
  *   to the device's current context: after cudaDeviceReset the library must be reloaded (the
  *   process restarted) before this entry point is used on that device again. The work is queued on
- *   cuda_stream (NULL = legacy default stream) and the call returns without waiting. Every call
- *   uses the same scratch array, which keeps the last call's flags until the next call clears
- *   it: calls whose work overlaps on the GPU (other streams, other threads) race and return wrong
- *   counts, so order them on one stream.
+ *   cuda_stream (NULL = legacy default stream) and the call returns without waiting. Calls with
+ *   more than 2,048 seeds use the same scratch array, which keeps the last such call's flags until
+ *   the next clears it: where their work overlaps on the GPU (other streams, other threads) they
+ *   race and return wrong counts, so order them on one stream. Calls with fewer may overlap.
  * ------------------------------------------------------------------------------------------ */
 #define HYPERIM_NOALLOC_MAX_N (1u << 24)
 hyperim_status hyperim_coverage_noalloc(int32_t n, const int64_t* rr_off, const int32_t* rr_mem,

@@ -57,10 +57,12 @@ constexpr int kWQ = 128;               // per-warp queue (members of the warp's 
 // set. Mean 1.7 members: the tiny query 0.85 -> 0.46 ms; mean 37: 27.9 -> 25.8 ms; mean 90 (2M vertices,
 // largest 12,000): 251 -> 243 ms. At a mean of 13,000 half of the sets would be begun twice.
 constexpr double kSmallMean = 200.0;
-// ... and only where every warp gets this many sets: with fewer the launch lasts as long as one warp's chain of
-// pops (and sets past kWQ are begun twice). 536 sets of 1,188 vertices, weighted cascade, the whole call: 886 us
-// before the warp phase was taken by size, 1,313 with it for any number of sets, 714 now; 2,000 sets 958 with the
-// warp phase and 793 without, 4,000 sets 957 and 1,024 (20,000 vertices: 1,811 and 1,741), 10,000 no different.
+// ... and only where every warp gets this many sets (9,728 on 152 SMs): with fewer the launch lasts as long as one
+// warp's chain of pops (and sets past kWQ are begun twice). 536 sets of 1,188 vertices, weighted cascade, the whole
+// call: 886 us before the warp phase was taken by size, 1,313 with it for any number of sets, 714 now; 2,000 sets 958
+// with the warp phase and 793 without, 4,000 sets 957 and 1,024 (20,000 vertices: 1,811 and 1,741), 10,000 no
+// different. The line lies on the careful side: it counts sets, while the chain's length follows their sizes, so
+// that a pool of tiny sets below it could gain from the warp phase and is built by blocks.
 constexpr int64_t kSmallSetsPerWarp = 4;
 constexpr int kWHashBits = 8;
 constexpr int kWHash = 1 << kWHashBits;  // per-warp open-addressing member set
@@ -2635,9 +2637,9 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
     if ((int64_t)blocks > njobs) blocks = (int)njobs;
     if ((st = ensure_scratch(g, blocks, vis_smem))) return st;
     const uint64_t want = arena_want(g, pools, npools, pool_start, g->n);
-    // the warp phase (one RR set per warp) runs first in the persistent schedule, unless the
-    // graph's tuning turned it off; its grid
-    // the sets' mean size so far, when every pool's is known
+    // The warp phase (one RR set per warp) runs first in the persistent schedule where the handle's tuning
+    // sets a limit, or, on a handle without one, where the sets are small: their mean size so far, when every
+    // pool's is known. (A new graph's first pool has none and is built by blocks.)
     double mean = 0.0;
     for (int q = 0; q < npools; ++q) {
         const double hint = pools[q]->mean_size_hint > 0 ? pools[q]->mean_size_hint : g->set_size_hint;
@@ -2665,7 +2667,7 @@ hyperim_status sample_rr_multi(hyperim_graph* g, hyperim_pool* const* pools, int
         int esc_count;
         int pad;
         unsigned long long arena_used;
-        unsigned long long set_cycles[3];  // sum, max, count over the sets the block kernel built
+        unsigned long long set_cycles[3];  // sum, max, count over the launch's sets, whichever phase built them
         unsigned long long memo_used;
     };
     int64_t* d_pos = nullptr;
