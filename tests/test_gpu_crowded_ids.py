@@ -48,5 +48,6 @@ def test_crowded_load_time():
             best = min(best, time.perf_counter() - t)
         return best
 
-    # 76M index entries against 1M: 1.3 times as long, 5 times when every group of chunks walked every key
-    assert seconds(False) < 3 * seconds(True)
+    # 76M index entries against 1M, graph freed again: 2.9 times as long, 8 times when every group of chunks
+    # walked every key
+    assert seconds(False) < 5 * seconds(True)
